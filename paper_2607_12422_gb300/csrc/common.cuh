@@ -166,6 +166,17 @@ __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap *map) {
 
 // ------------------------------------------------------------------ tcgen05 (5th-gen tensor core)
 
+// True in exactly one lane of a converged warp.  The thread that issues tcgen05.mma must be chosen
+// this way, in code inlined into the kernel: the compiler then knows that one lane is active and
+// keeps the instruction's descriptors in uniform registers.  Behind `lane == 0` it cannot, and a
+// 128 x 32 x 16 MMA with a commit every four takes 110 cycles to issue instead of 64 (41 without
+// commits; 128 x 256 x 16: 129 either way, the tensor core's own rate).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred P;\n\telect.sync _|P, 0xffffffff;\n\tselp.u32 %0, 1, 0, P;\n\t}" : "=r"(p));
+    return p != 0;
+}
+
 // Allocate `ncols` TMEM columns (power of two >= 32); whole warp; address written to smem.
 __device__ __forceinline__ void tmem_alloc(uint32_t *dst_smem, uint32_t ncols) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(dst_smem)),

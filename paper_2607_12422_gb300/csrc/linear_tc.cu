@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(LIN_THREADS, 1)
             for (int s = issued > NSTAGE ? issued - NSTAGE : 0; s < issued; ++s)
                 mbar_wait(&full[s % NSTAGE], (s / NSTAGE) & 1, nullptr, 0, nullptr);
         }
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1 && elect_one()) {
         // ---- MMA issuer: 4 x (128 x BN x 16) per 64-wide stage into the TMEM accumulator
         const uint32_t idesc = idesc_bf16_f32(128, BN);
         bool ok = true;
@@ -280,7 +280,7 @@ __global__ void __launch_bounds__(LMH_THREADS, 1)
             for (int h = g > LMH_STAGES ? g - LMH_STAGES : 0; h < g; ++h)
                 mbar_wait(&full[h % LMH_STAGES], (h / LMH_STAGES) & 1, nullptr, 0, nullptr);
         }
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1 && elect_one()) {
         // ---- MMA issuer: per tile 4 x (128 x BN x 16) per K atom into accumulator j & 1
         const uint32_t idesc = idesc_bf16_f32(128, BN);
         bool ok = mbar_wait(x_full, 0, status, DEV_TIMEOUT_LOAD, abort_flag);

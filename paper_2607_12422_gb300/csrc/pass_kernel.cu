@@ -1040,9 +1040,9 @@ __device__ __noinline__ void run_producer(const MKParams &P, const MKItem *my, i
             drain_wait(&S.full[h % P.nslot], (h / P.nslot) & 1);
 }
 
-// ---- warp 1 lane 0: MMA issuer.  Per linear item, 4 (or 8) x 4 tcgen05.mma (128 x bn x 16,
+// ---- warp 1, one elected lane: MMA issuer.  Per linear item, 4 (or 8) x 4 tcgen05.mma (128 x bn x 16,
 // bf16 -> fp32) into the TMEM accumulator; frees ring slots with tcgen05.commit.
-__device__ __noinline__ void run_mma(const MKParams &P, const MKItem *my, int n_my, uint8_t *ring, uint8_t *uni,
+__device__ __forceinline__ void run_mma(const MKParams &P, const MKItem *my, int n_my, uint8_t *ring, uint8_t *uni,
                                      uint32_t tmem, CtaState &S) {
     const uint32_t idesc = idesc_bf16_f32(128, P.bn);
     uint32_t kt = 0, li = 0, l8 = 0;
@@ -1416,7 +1416,8 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_pass(const __grid_constant__ 
     if (warp == 0) {
         if (lane == 0) run_producer(P, my, n_my, ring, S);
     } else if (warp == 1) {
-        if (lane == 0) run_mma(P, my, n_my, ring, uni, tmem, S);
+        if (elect_one()) run_mma(P, my, n_my, ring, uni, tmem, S);
+        __syncwarp();
     } else {
         run_compute<DRAFT, DH>(P, my, n_my, uni, tmem, S, tid);
     }
