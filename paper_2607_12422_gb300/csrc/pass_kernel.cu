@@ -1005,12 +1005,14 @@ struct CtaState {
     uint4 gain[MAX_ATOMS * KT / 8];
 };
 
-// ---- warp 0 lane 0: weight producer.  Walks the CTA's linear items ahead of the others and
+// ---- warp 0, one elected lane: weight producer.  Walks the CTA's linear items ahead of the others and
 // streams their 128 x 64 weight tiles into the ring (1-D bulk TMA, L2 evict-first); weights depend
 // on nothing, so the ring fills across phase boundaries.
-__device__ __noinline__ void run_producer(const MKParams &P, const MKItem *my, int n_my, uint8_t *ring, CtaState &S) {
+__device__ __forceinline__ void run_producer(const MKParams &P, const MKItem *my, int n_my, uint8_t *ring, CtaState &S) {
     const uint64_t pol = l2_policy_evict_first();
-    uint32_t kt = 0;
+    const int nslot = P.nslot;
+    int slot = 0, kt = 0;
+    uint32_t ph = 1;  // (a fresh barrier counts as having completed the phase before its first)
 #pragma unroll 1
     for (int i = 0; i < n_my && !aborted(P); ++i) {
         const MKItem it = my[i];
@@ -1023,21 +1025,21 @@ __device__ __noinline__ void run_producer(const MKParams &P, const MKItem *my, i
             P.wt[lin] + P.wt_stride[lin] * it.layer + ((size_t)it.a * kts + (size_t)it.b * P.katoms[lin]) * TILE_BYTES;
         bool ok = true;
 #pragma unroll 1
-        for (int j = 0; j < P.katoms[lin]; ++j, ++kt) {
-            const int slot = kt % P.nslot;
-            if (kt >= (uint32_t)P.nslot && !mbar_wait_mk(&S.empty[slot], ((kt / P.nslot) - 1) & 1, P, DEV_TIMEOUT_SLOT)) {
+        for (int j = P.katoms[lin]; j > 0; --j, ++kt) {
+            if (!mbar_wait_mk(&S.empty[slot], ph, P, DEV_TIMEOUT_SLOT)) {
                 ok = false;
                 break;
             }
             mbar_arrive_expect_tx(&S.full[slot], bytes);
-            bulk_g2s(ring + (size_t)slot * TILE_BYTES, src + (size_t)j * TILE_BYTES, bytes, &S.full[slot], pol);
+            bulk_g2s(ring + slot * TILE_BYTES, src, bytes, &S.full[slot], pol);
+            src += TILE_BYTES;
+            if (++slot == nslot) slot = 0, ph ^= 1;
         }
         if (!ok) break;
     }
     if (aborted(P))  // the last nslot tiles issued may still be in flight: let them land
 #pragma unroll 1
-        for (uint32_t h = kt > (uint32_t)P.nslot ? kt - P.nslot : 0; h < kt; ++h)
-            drain_wait(&S.full[h % P.nslot], (h / P.nslot) & 1);
+        for (int h = kt > nslot ? kt - nslot : 0; h < kt; ++h) drain_wait(&S.full[h % nslot], (h / nslot) & 1);
 }
 
 // ---- warp 1, one elected lane: MMA issuer.  Per linear item, 4 (or 8) x 4 tcgen05.mma (128 x bn x 16,
@@ -1045,7 +1047,9 @@ __device__ __noinline__ void run_producer(const MKParams &P, const MKItem *my, i
 __device__ __forceinline__ void run_mma(const MKParams &P, const MKItem *my, int n_my, uint8_t *ring, uint8_t *uni,
                                      uint32_t tmem, CtaState &S) {
     const uint32_t idesc = idesc_bf16_f32(128, P.bn);
-    uint32_t kt = 0, li = 0, l8 = 0;
+    const int nslot = P.nslot;
+    int slot = 0;
+    uint32_t ph = 0, li = 0, l8 = 0;
 #pragma unroll 1
     for (int i = 0; i < n_my; ++i) {
         const MKItem it = my[i];
@@ -1055,7 +1059,7 @@ __device__ __forceinline__ void run_mma(const MKParams &P, const MKItem *my, int
         tc_fence_after();
         bool ok = true;
 #pragma unroll 1
-        for (int j = 0; j < na; ++j, ++kt) {
+        for (int j = 0; j < na; ++j) {
             if (j == HALF_ATOMS) {
                 // second half of a wide slice: its operand is staged after the first half's reads
                 // completed (same area) or was staged with it
@@ -1066,19 +1070,19 @@ __device__ __forceinline__ void run_mma(const MKParams &P, const MKItem *my, int
                 }
                 tc_fence_after();
             }
-            const int slot = kt % P.nslot;
-            if (!mbar_wait_mk(&S.full[slot], (kt / P.nslot) & 1, P, DEV_TIMEOUT_LOAD)) {
+            if (!mbar_wait_mk(&S.full[slot], ph, P, DEV_TIMEOUT_LOAD)) {
                 ok = false;
                 break;
             }
             tc_fence_after();
-            const uint64_t ad = sw128_kmajor_desc(ring + (size_t)slot * TILE_BYTES);
+            const uint64_t ad = sw128_kmajor_desc(ring + slot * TILE_BYTES);
             const int bj = (P.b_dbl || j < HALF_ATOMS) ? j : j - HALF_ATOMS;
             const uint64_t bd = sw128_kmajor_desc(uni + (size_t)bj * P.bn * 128);
 #pragma unroll
             for (int kk = 0; kk < KT / 16; ++kk)
                 mma_bf16_ss(tmem, ad + 2ull * kk, bd + 2ull * kk, idesc, (j | kk) != 0 ? 1u : 0u);
             mma_commit(&S.empty[slot]);
+            if (++slot == nslot) slot = 0, ph ^= 1;
         }
         if (!ok) break;
         mma_commit(&S.acc_full);
@@ -1374,7 +1378,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_pass(const __grid_constant__ 
     uint8_t *ring = base;
     uint8_t *uni = base + P.ring_bytes;  // activation tile / attention staging
     __shared__ CtaState S;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = tid >> 5;
     const MKItem *my = P.items + P.cta_off[blockIdx.x];
     const int n_my = P.cta_off[blockIdx.x + 1] - P.cta_off[blockIdx.x];
 
@@ -1414,7 +1418,8 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_pass(const __grid_constant__ 
     tc_fence_after();
     const uint32_t tmem = S.tmem_slot;
     if (warp == 0) {
-        if (lane == 0) run_producer(P, my, n_my, ring, S);
+        if (elect_one()) run_producer(P, my, n_my, ring, S);
+        __syncwarp();
     } else if (warp == 1) {
         if (elect_one()) run_mma(P, my, n_my, ring, uni, tmem, S);
         __syncwarp();
