@@ -22,9 +22,9 @@ size_t pbd_op_linear_workspace_bytes(int32_t M, int32_t K, int32_t N, int32_t r)
  *     u = bf16(x A^T)                    [M, r]
  *     y = bf16(x W^T + scale * u B^T)    [M, N]   (fp32 accumulation, one final rounding)
  * d_x [M, K], d_w [N, K], d_a [r, K], d_b [N, r], d_y [M, N]: bf16, row-major, 16-byte aligned.
- * d_a == NULL or d_b == NULL (or r == 0) switches the delta off.  Runs the same tensor-core
- * kernel as the decoder passes (K split in 256-wide slices, fp32 partial sums in the workspace,
- * fixed-order reduction).  Requirements: N % 128 == 0, K % 64 == 0, 1 <= M <= 4096, r <= 32.
+ * d_a == NULL or d_b == NULL (or r == 0) switches the delta off.  W and A are read in place; K is
+ * summed in 256-wide slices in one fixed order, as in the decoder passes, so without the adapter a
+ * row's result does not depend on M.  Requirements: N % 128 == 0, K % 64 == 0, 1 <= M <= 4096, r <= 32.
  * The workspace (d_ws, >= pbd_op_linear_workspace_bytes, 1024-byte aligned) is scratch; its first
  * word is the kernel's status word, cleared by each call and read by pbd_op_status.
  * The return value covers argument checks and launches only: a bounded device wait that ran out
@@ -53,16 +53,15 @@ pbd_status pbd_op_linear(int32_t M, int32_t K, int32_t N, int32_t r, float scale
  * any stream capture begins.
  *
  * Size limit: the call needs 2048 + (N/128 + (r > 0)) * (K/64) * 16384 + 4 * s * M * (N + r)
- * bytes, s = K/256 when K is a multiple of 256 and 1 otherwise (the re-tiled weight, the
+ * bytes, s = K/256 when K is a multiple of 256 and 1 otherwise (room for a tiled weight, the
  * adapter rows and the fp32 split-K partial sums).  Larger problems return PBD_ERR_CAPACITY
  * before anything is launched, and the message gives both sizes; use pbd_op_linear for them.
  * Within 16 MiB fit, for instance, an N = 6144, K = 1024 weight with r = 16 up to M = 39, and
  * an N = 1024, K = 3072 weight with r = 16 up to M = 194.
  *
  * Zeroing: every call clears, on d_stream, the one part of the scratch that must start at zero,
- * the kernel's status word.  Every other byte a call reads (the re-tiled weight and adapter rows,
- * the partial sums) is written by that same call first, so a call never sees an earlier call's
- * data.
+ * the kernel's status word.  Every other byte a call reads there is written by that same call
+ * first, so a call never sees an earlier call's data.
  *
  * Device errors: as for pbd_op_linear, the return value covers argument checks and launches;
  * pbd_op_linear_static_status reports a device wait that ran out.  Ask before the next call on

@@ -1,8 +1,7 @@
 // op_linear_static.cu -- pbd_op_linear_static (include/pbd_ops.h): the block linear of
 // pbd_op_linear, with its scratch taken from a fixed-size device array that belongs to this
 // library instead of from a caller workspace.  A call therefore neither receives nor allocates
-// device memory: it re-tiles the weight into the array, runs the same tensor-core kernel and
-// split-K reduction, and writes y.
+// device memory: it runs the same kernels and the same fixed-order sums, and writes y.
 //
 // The array exists once per device; it is created when the CUDA runtime loads this library's
 // device code on that device, and its address is looked up once per device (first call with
@@ -19,9 +18,9 @@
 #include "pbd_internal.h"
 
 // Layout inside the array (offsets from the first 1024-byte boundary in it):
-//   [0, 256)         status word of the tensor-core kernel (cleared by every call)
-//   [1024, ...)      the weight (and adapter A rows) re-tiled in 128 x 64 tiles of 16 KiB
-//   [..., ...)       fp32 split-K partial sums [k_splits][M][N + r]
+//   [0, 256)     status word of the tensor-core kernels (cleared by every call)
+//   [1024, ...)  room for the weight and the adapter's rows as 16 KiB tiles, then for split-K partial sums;
+//                the second part holds the adapter's u rows (and padded B rows) of calls with many rows
 static __device__ __align__(256) unsigned char g_linear_scratch[PBD_OP_LINEAR_STATIC_SCRATCH_BYTES];
 
 using namespace pbd;
@@ -108,37 +107,10 @@ extern "C" pbd_status pbd_op_linear_static(int32_t M, int32_t K, int32_t N, int3
     const pbd_status s = scratch_of_current_device(&ws);
     if (s != PBD_OK) return s;
 
-    const int bn = M <= 32 ? 32 : M <= 64 ? 64 : M <= 128 ? 128 : 256;
-    CUtensorMap map;
-    if (!encode_bf16_map(&map, d_x, M, K, bn))
-        return fail(PBD_ERR_INVALID_ARG, "pbd_op_linear_static: x not TMA-mappable (16-byte alignment)");
-
-    cudaStream_t st = static_cast<cudaStream_t>(d_stream);
-    int *status = reinterpret_cast<int *>(ws);
-    TiledWeight w;
-    w.tiles = ws + p.tiles_off;
-    w.n_main = N;
-    w.lora_rows = rr;
-    w.K = K;
-    Partials P;
-    P.p = reinterpret_cast<float *>(ws + p.part_off);
-    P.k_splits = p.k_splits;
-    P.rows_alloc = M;
-    P.n_total = N + rr;
-    uint8_t *tiles = ws + p.tiles_off;
-
-    cudaError_t e;
-    // What must start at zero on every call: the status word, which the kernel only ever raises.
-    // The weight tiles and the partial sums this call reads are written by this call first (the
-    // kernel copies only the adapter tile's first r rows, and stores only rows it computed).
-    if ((e = cudaMemsetAsync(status, 0, 256, st)) != cudaSuccess) return fail_cuda("clear status", e);
-    if ((e = launch_repack_tiled(d_w, N, K, tiles, 0, st)) != cudaSuccess) return fail_cuda("repack W", e);
-    if (lora && (e = launch_repack_tiled(d_a, rr, K, tiles, N, st)) != cudaSuccess) return fail_cuda("repack A", e);
-    if ((e = launch_linear_partials(&map, bn, w, lora ? 1 : 0, M, P, status, st)) != cudaSuccess)
-        return fail_cuda("linear", e);
-    if ((e = launch_linear_finalize(P, M, N, rr, scale, d_b, d_y, st)) != cudaSuccess)
-        return fail_cuda("finalize", e);
-    return PBD_OK;
+    // What must start at zero on every call, the status word and the tile counters, is cleared by
+    // it; every other byte this call reads is written by this call first.
+    return run_linear_op(M, K, N, rr, scale, d_x, d_w, d_a, d_b, d_y, LinearScratch{ws, ws + p.tiles_off, ws + p.part_off},
+                         static_cast<cudaStream_t>(d_stream), "pbd_op_linear_static");
 }
 
 extern "C" pbd_status pbd_op_linear_static_status(void *d_stream, int32_t *h_device_code) {

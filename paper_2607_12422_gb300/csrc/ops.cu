@@ -4,51 +4,20 @@
 //   k_prefill_finish  cached length and first token after a prompt
 //   k_repack_tiled    row-major bf16 weights -> 128 x 64 tiles in the 128-byte swizzle layout
 //   k_read_kv         paged cache -> contiguous rows (tests of the commit rule)
-//   k_linear_finalize split-K sum + adapter delta of the standalone linear entry point
+//   k_pack_b          adapter B rows padded to 32 columns (standalone linear)
 #include "common.cuh"
 #include "pbd_internal.h"
 
 namespace pbd {
 
-constexpr int ROW_THREADS = 256;
-constexpr int MAX_R = 64;
-
-// Sum of the k_splits partials of (row m, feature f) in split order.
-__device__ __forceinline__ float sum_splits(const Partials &P, int m, int f) {
-    float a = P.p[(size_t)m * P.n_total + f];
-    for (int s = 1; s < P.k_splits; ++s) a = __fadd_rn(a, P.p[((size_t)s * P.rows_alloc + m) * P.n_total + f]);
-    return a;
+__global__ void k_pack_b(const bf16 *__restrict__ b, int N, int r, bf16 *__restrict__ out) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= N * 32) return;
+    out[i] = (i & 31) < r ? b[(size_t)(i >> 5) * r + (i & 31)] : __float2bfloat16_rn(0.f);
 }
 
-// Adapter contribution of one output feature: sum_j u_j * B[f, j] (fp32, j in order).
-__device__ __forceinline__ float lora_dot(const float *u, const bf16 *Brow, int r) {
-    float a = 0.f;
-    for (int j = 0; j < r; ++j) a = __fadd_rn(a, __fmul_rn(u[j], bf2f(Brow[j])));
-    return a;
-}
-
-// Standalone linear epilogue: y = bf16(sum of splits + scale * u B^T), u = bf16(adapter rows).
-__global__ void __launch_bounds__(ROW_THREADS)
-    k_linear_finalize(Partials P, int N, int r, float scale, const bf16 *__restrict__ lora_b, bf16 *__restrict__ y) {
-    __shared__ float su[MAX_R];
-    const int m = blockIdx.x;
-    if (r > 0) {
-        if ((int)threadIdx.x < r) su[threadIdx.x] = rbf(sum_splits(P, m, N + threadIdx.x));
-        __syncthreads();
-    }
-    const int f = blockIdx.y * ROW_THREADS + threadIdx.x;
-    if (f >= N) return;
-    float acc = sum_splits(P, m, f);
-    if (r > 0) acc = __fadd_rn(acc, __fmul_rn(scale, lora_dot(su, lora_b + (size_t)f * r, r)));
-    y[(size_t)m * N + f] = f2bf(acc);
-}
-
-cudaError_t launch_linear_finalize(const Partials &P, int M, int N, int r, float scale, const void *lora_b, void *y,
-                                   cudaStream_t st) {
-    if (r > MAX_R) return cudaErrorInvalidValue;
-    dim3 grid(M, (N + ROW_THREADS - 1) / ROW_THREADS);
-    k_linear_finalize<<<grid, ROW_THREADS, 0, st>>>(P, N, r, scale, static_cast<const bf16 *>(lora_b),
-                                                    static_cast<bf16 *>(y));
+cudaError_t launch_pack_b(const void *b, int N, int r, void *out, cudaStream_t st) {
+    k_pack_b<<<(N * 32 + 255) / 256, 256, 0, st>>>(static_cast<const bf16 *>(b), N, r, static_cast<bf16 *>(out));
     return cudaGetLastError();
 }
 
@@ -142,10 +111,6 @@ cudaError_t launch_repack_tiled_map(const void *src, int rows, int K, void *dst_
                                                                 static_cast<bf16 *>(dst_tiles), dst_row0, group,
                                                                 stride);
     return cudaGetLastError();
-}
-
-cudaError_t launch_repack_tiled(const void *src, int rows, int K, void *dst_tiles, int dst_row0, cudaStream_t st) {
-    return launch_repack_tiled_map(src, rows, K, dst_tiles, dst_row0, rows, 0, st);
 }
 
 __global__ void k_read_kv(KVCache kv, int Hkv, int d, int layer, int seq, int n, bf16 *__restrict__ k_out,

@@ -1,7 +1,6 @@
 // ops_api.cu -- single-kernel C entry points (include/pbd_ops.h) and the TMA descriptor helper
-// shared with the context code.  The linear entry point re-tiles W (and A) into the workspace,
-// runs the same tensor-core kernel and split-K reduction as the decoder passes, and finishes
-// with bf16(x W^T + s * bf16(x A^T) B^T).
+// shared with the context code.  The linear and the lm_head read the caller's row-major weights
+// through tensor maps and sum over K in the same slices and order as the decoder passes.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -39,8 +38,6 @@ bool encode_bf16_map(CUtensorMap *map, const void *base, int rows, int cols, int
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
-
-int op_bn(int M) { return M <= 32 ? 32 : M <= 64 ? 64 : M <= 128 ? 128 : 256; }
 
 }  // namespace pbd
 
@@ -97,6 +94,85 @@ pbd_status read_device_code(const int *d_status, cudaStream_t st, int *code, con
     return PBD_OK;
 }
 
+// Few rows (one operand tile of at most 64 tokens) and a K whose slices fit one cluster: linear_op.cu, one
+// launch that spreads the K slices over CTAs.  More rows: gemm.cu, whose CTAs keep whole tiles' sums in registers; the
+// adapter's u = bf16(x A^T) comes first, as one more such linear, and enters the tile as one more
+// MMA group.
+pbd_status run_linear_op(int M, int K, int N, int r, float scale, const void *d_x, const void *d_w, const void *d_a,
+                         const void *d_b, void *d_y, const LinearScratch &ws, cudaStream_t st, const char *who) {
+    auto bad = [&](pbd_status s, const char *what, cudaError_t e = cudaSuccess) {
+        char b[160];
+        snprintf(b, sizeof b, "%s: %s", who, what);
+        return op_fail(s, b, e);
+    };
+    const int kt = K / KT, ks = kt % 4 == 0 ? kt / 4 : 1, f_tiles = N / TILE_ROWS;
+    const bool few = M <= LINEAR_OP_MAX_ROWS && ks <= LINEAR_OP_MAX_SLICES;
+    int *status = reinterpret_cast<int *>(ws.status);
+    cudaError_t e;
+    if ((e = configure_linear_kernels()) != cudaSuccess) return bad(PBD_ERR_CUDA, "configure", e);
+    if (few) {
+        LinOpArgs a;
+        a.bn = M <= 32 ? 32 : 64;
+        if (!encode_bf16_map(&a.xmap, d_x, M, K, a.bn)) return bad(PBD_ERR_INVALID_ARG, "x not TMA-mappable");
+        if (!encode_bf16_map(&a.wmap, d_w, N, K, TILE_ROWS)) return bad(PBD_ERR_INVALID_ARG, "W not TMA-mappable");
+        a.amap = a.wmap;
+        if (r > 0 && !encode_bf16_map(&a.amap, d_a, r, K, r)) return bad(PBD_ERR_INVALID_ARG, "A not TMA-mappable");
+        a.kt_per = kt / ks;
+        a.ks = ks;
+        a.M = M;
+        a.N = N;
+        a.r = r;
+        a.scale = scale;
+        a.b = static_cast<const bf16 *>(d_b);
+        a.y = static_cast<bf16 *>(d_y);
+        a.vec_store = (reinterpret_cast<uintptr_t>(d_y) & 7) == 0;
+        a.status = status;
+        if ((e = cudaMemsetAsync(status, 0, 256, st)) != cudaSuccess) return bad(PBD_ERR_CUDA, "memset", e);
+        if ((e = launch_linear_op(a, st)) != cudaSuccess) return bad(PBD_ERR_CUDA, "linear", e);
+        return PBD_OK;
+    }
+    GemmArgs a{};
+    a.bn = gemm_pick_bn(M, f_tiles, kt, 256, gemm_ctas());
+    if (!encode_bf16_map(&a.xmap, d_x, M, K, a.bn)) return bad(PBD_ERR_INVALID_ARG, "x not TMA-mappable");
+    if (!encode_bf16_map(&a.wmap, d_w, N, K, TILE_ROWS)) return bad(PBD_ERR_INVALID_ARG, "W not TMA-mappable");
+    a.k_tiles = kt;
+    a.slice_atoms = kt / ks;
+    a.n_slices = ks;
+    a.f_tiles = f_tiles;
+    a.M = M;
+    a.rows = N;
+    a.scale = scale;
+    a.y = static_cast<bf16 *>(d_y);
+    a.ld = N;
+    a.vec_store = (reinterpret_cast<uintptr_t>(d_y) & 15) == 0;
+    a.status = status;
+    if ((e = cudaMemsetAsync(status, 0, 256, st)) != cudaSuccess) return bad(PBD_ERR_CUDA, "memset", e);
+    if (r > 0) {
+        uint8_t *u = ws.part, *bp = ws.part + ((size_t)M * 64 + 1023) / 1024 * 1024;  // [M][32], [N][32]
+        GemmArgs g = a;
+        g.bn = 64;
+        if (!encode_bf16_map(&g.xmap, d_x, M, K, g.bn)) return bad(PBD_ERR_INVALID_ARG, "x not TMA-mappable");
+        if (!encode_bf16_map(&g.wmap, d_a, r, K, TILE_ROWS)) return bad(PBD_ERR_INVALID_ARG, "A not TMA-mappable");
+        g.f_tiles = 1;
+        g.rows = 32;  // (rows past r are zero)
+        g.y = reinterpret_cast<bf16 *>(u);
+        g.ld = 32;
+        g.vec_store = 1;
+        if ((e = launch_gemm(GEMM_Y, g, 0, st)) != cudaSuccess) return bad(PBD_ERR_CUDA, "adapter rows", e);
+        a.delta = 1;
+        bool ok = encode_bf16_map(&a.umap, u, M, 32, a.bn);
+        if (r % 8 == 0 && (reinterpret_cast<uintptr_t>(d_b) & 15) == 0) {
+            ok = ok && encode_bf16_map(&a.bmap, d_b, N, r, TILE_ROWS);
+        } else {  // no TMA layout: rows padded to 32
+            if ((e = launch_pack_b(d_b, N, r, bp, st)) != cudaSuccess) return bad(PBD_ERR_CUDA, "pack B", e);
+            ok = ok && encode_bf16_map(&a.bmap, bp, N, 32, TILE_ROWS);
+        }
+        if (!ok) return bad(PBD_ERR_CUDA, "tensor map encode failed");
+    }
+    if ((e = launch_gemm(GEMM_Y, a, 0, st)) != cudaSuccess) return bad(PBD_ERR_CUDA, "linear", e);
+    return PBD_OK;
+}
+
 const char *device_code_name(int code) {
     switch (code) {
         case DEV_TIMEOUT_LOAD: return "a weight or operand copy never completed";
@@ -135,37 +211,10 @@ pbd_status pbd_op_linear(int32_t M, int32_t K, int32_t N, int32_t r, float scale
     if (!d_x || !d_w || !d_y) return op_fail(PBD_ERR_INVALID_ARG, "pbd_op_linear: null pointer");
     if (!d_ws || (reinterpret_cast<uintptr_t>(d_ws) & 1023) || ws_bytes < p.total)
         return op_fail(PBD_ERR_WORKSPACE, "pbd_op_linear: workspace missing, misaligned or too small");
-    cudaStream_t st = static_cast<cudaStream_t>(d_stream);
     uint8_t *ws = static_cast<uint8_t *>(d_ws);
-    int *status = reinterpret_cast<int *>(ws + p.status_off);
-    TiledWeight w;
-    w.tiles = ws + p.tiles_off;
-    w.n_main = N;
-    w.lora_rows = rr;
-    w.K = K;
-    Partials P;
-    P.p = reinterpret_cast<float *>(ws + p.part_off);
-    P.k_splits = p.k_splits;
-    P.rows_alloc = M;
-    P.n_total = N + rr;
-    const int bn = op_bn(M);
-    CUtensorMap map;
-    if (!encode_bf16_map(&map, d_x, M, K, bn)) return op_fail(PBD_ERR_INVALID_ARG, "pbd_op_linear: x not TMA-mappable");
-    cudaError_t e;
-    if ((e = configure_linear_kernels()) != cudaSuccess) return op_fail(PBD_ERR_CUDA, "configure", e);
-    if ((e = cudaMemsetAsync(status, 0, 256, st)) != cudaSuccess) return op_fail(PBD_ERR_CUDA, "memset", e);
-    if ((e = cudaMemsetAsync(const_cast<void *>(w.tiles), 0, (size_t)p.row_tiles * (K / KT) * TILE_BYTES, st)) !=
-        cudaSuccess)
-        return op_fail(PBD_ERR_CUDA, "memset", e);
-    if ((e = launch_repack_tiled(d_w, N, K, const_cast<void *>(w.tiles), 0, st)) != cudaSuccess)
-        return op_fail(PBD_ERR_CUDA, "repack W", e);
-    if (lora && (e = launch_repack_tiled(d_a, rr, K, const_cast<void *>(w.tiles), N, st)) != cudaSuccess)
-        return op_fail(PBD_ERR_CUDA, "repack A", e);
-    if ((e = launch_linear_partials(&map, bn, w, lora ? 1 : 0, M, P, status, st)) != cudaSuccess)
-        return op_fail(PBD_ERR_CUDA, "linear", e);
-    if ((e = launch_linear_finalize(P, M, N, rr, scale, d_b, d_y, st)) != cudaSuccess)
-        return op_fail(PBD_ERR_CUDA, "finalize", e);
-    return PBD_OK;
+    return run_linear_op(M, K, N, rr, scale, d_x, d_w, d_a, d_b, d_y,
+                         LinearScratch{ws + p.status_off, ws + p.tiles_off, ws + p.part_off},
+                         static_cast<cudaStream_t>(d_stream), "pbd_op_linear");
 }
 
 size_t pbd_op_lm_head_workspace_bytes(int32_t M, int32_t H, int32_t V) {
@@ -187,24 +236,24 @@ pbd_status pbd_op_lm_head_argmax(int32_t M, int32_t H, int32_t V, const void *d_
     int *status = reinterpret_cast<int *>(ws);
     const size_t tiles_bytes = (size_t)(V / TILE_ROWS) * (H / KT) * TILE_BYTES;
     TiledWeight w;
-    w.tiles = ws + 1024;
+    w.tiles = nullptr;  // read through w_map where the caller has it
     w.n_main = V;
     w.lora_rows = 0;
     w.K = H;
     float *tmax = reinterpret_cast<float *>(ws + 1024 + (tiles_bytes + 1023) / 1024 * 1024);
     int *targ = reinterpret_cast<int *>(tmax + (size_t)(V / TILE_ROWS) * M);
-    const int bn = op_bn(M);
-    CUtensorMap map;
-    if (!encode_bf16_map(&map, d_x, M, H, bn))
+    CUtensorMap map, w_map;
+    if (!encode_bf16_map(&map, d_x, M, H, lm_head_box(M, H)))
         return op_fail(PBD_ERR_INVALID_ARG, "pbd_op_lm_head_argmax: x not TMA-mappable");
+    if (!encode_bf16_map(&w_map, d_embed, V, H, TILE_ROWS))
+        return op_fail(PBD_ERR_INVALID_ARG, "pbd_op_lm_head_argmax: embed not TMA-mappable");
     cudaError_t e;
+    int n_parts = 0;
     if ((e = configure_linear_kernels()) != cudaSuccess) return op_fail(PBD_ERR_CUDA, "configure", e);
     if ((e = cudaMemsetAsync(status, 0, 256, st)) != cudaSuccess) return op_fail(PBD_ERR_CUDA, "memset", e);
-    if ((e = launch_repack_tiled(d_embed, V, H, const_cast<void *>(w.tiles), 0, st)) != cudaSuccess)
-        return op_fail(PBD_ERR_CUDA, "repack", e);
-    if ((e = launch_lm_head(&map, bn, w, M, tmax, targ, d_logits_opt, status, st)) != cudaSuccess)
+    if ((e = launch_lm_head(map, w, &w_map, M, tmax, targ, &n_parts, d_logits_opt, status, st)) != cudaSuccess)
         return op_fail(PBD_ERR_CUDA, "lm_head", e);
-    if ((e = launch_argmax_reduce(tmax, targ, V / TILE_ROWS, M, d_ids, st)) != cudaSuccess)
+    if ((e = launch_argmax_reduce(tmax, targ, n_parts, M, d_ids, st)) != cudaSuccess)
         return op_fail(PBD_ERR_CUDA, "argmax", e);
     return PBD_OK;
 }

@@ -31,8 +31,6 @@ namespace {
 thread_local std::string g_last_error;
 
 constexpr size_t ALIGN = 1024;
-constexpr int N_BN = 4;
-const int BN_CHOICES[N_BN] = {32, 64, 128, 256};
 constexpr int POLL_ROUNDS = 4;
 
 enum Phase { PH_NONE = 0, PH_READY, PH_DRAFTED, PH_VERIFIED };
@@ -49,18 +47,6 @@ struct Bump {
         return p;
     }
 };
-
-int pick_bn(int M) {
-    for (int i = 0; i < N_BN; ++i)
-        if (M <= BN_CHOICES[i]) return BN_CHOICES[i];
-    return 256;
-}
-
-int bn_index(int bn) {
-    for (int i = 0; i < N_BN; ++i)
-        if (BN_CHOICES[i] == bn) return i;
-    return N_BN - 1;
-}
 
 struct Sched {
     MKItem *items = nullptr;  // device
@@ -99,7 +85,7 @@ struct pbd_ctx {
     CounterLayout cl;
     Sched sched[N_PK];
     SeqState s;
-    CUtensorMap maps[N_BN];  // x_ro, per box height
+    CUtensorMap maps[16];    // x_ro, box height 16 (i + 1)
     CUtensorMap kmap, vmap;  // paged K and V caches
     // host state
     int batch = 0, max_new = 0;
@@ -303,9 +289,9 @@ size_t layout(pbd_ctx *c, void *base) {
 }
 
 pbd_status make_maps(pbd_ctx *c) {
-    for (int i = 0; i < N_BN; ++i)
-        if (!encode_bf16_map(&c->maps[i], c->x_ro, c->ro_alloc, c->cfg.hidden, BN_CHOICES[i]))
-            return fail(c, PBD_ERR_CUDA, "tensor map encode failed (box rows %d)", BN_CHOICES[i]);
+    for (int i = 0; i < 16; ++i)
+        if (!encode_bf16_map(&c->maps[i], c->x_ro, c->ro_alloc, c->cfg.hidden, 16 * (i + 1)))
+            return fail(c, PBD_ERR_CUDA, "tensor map encode failed (box rows %d)", 16 * (i + 1));
     // K and V caches seen as rows of head_dim values: (layer, page, kv head, token) -> one row
     const int kv_rows = c->cfg.n_layers * c->n_pages * c->cfg.n_kv_heads * PAGE;
     if (!encode_bf16_map(&c->kmap, c->kv.k, kv_rows, c->cfg.head_dim, PAGE) ||
@@ -517,10 +503,10 @@ pbd_status enqueue_pass_kernel(pbd_ctx *c, const PassDesc &pd, int kind) {
 pbd_status enqueue_readout(pbd_ctx *c, const PassDesc &pd, int *ids_out, float *logits) {
     const int n_ro = pd.nb * pd.ro_count;
     if (n_ro <= 0) return PBD_OK;
-    const int bro = pick_bn(n_ro);
-    CK(launch_lm_head(&c->maps[bn_index(bro)], bro, c->w_lm, n_ro, c->tile_max, c->tile_arg, logits, c->status,
-                      c->st));
-    CK(launch_argmax_reduce(c->tile_max, c->tile_arg, c->cfg.vocab / TILE_ROWS, n_ro, ids_out, c->st));
+    int n_parts = 0;
+    CK(launch_lm_head(c->maps[lm_head_box(n_ro, c->cfg.hidden) / 16 - 1], c->w_lm, nullptr, n_ro, c->tile_max,
+                      c->tile_arg, &n_parts, logits, c->status, c->st));
+    CK(launch_argmax_reduce(c->tile_max, c->tile_arg, n_parts, n_ro, ids_out, c->st));
     return PBD_OK;
 }
 

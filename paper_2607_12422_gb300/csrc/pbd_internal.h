@@ -3,6 +3,7 @@
 #pragma once
 
 #include <cuda.h>
+#include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -11,6 +12,8 @@
 #include "../../include/pbd.h"
 
 namespace pbd {
+
+typedef __nv_bfloat16 bf16;
 
 constexpr int PAGE = 16;           // KV page length in tokens
 constexpr int ATT_SPLIT = 128;     // key positions per attention split (position-aligned)
@@ -56,14 +59,6 @@ struct TiledWeight {
     int n_main;      // main output features (multiple of 128)
     int lora_rows;   // rows of the adapter tile (r x number of adapters)
     int K;           // input features (multiple of 64)
-};
-
-// Split-K partial sums, fp32 [k_splits][rows_alloc][n_total], n_total = n_main + lora_rows.
-struct Partials {
-    float *p;
-    int k_splits;
-    int rows_alloc;
-    int n_total;
 };
 
 // ---- persistent pass kernel (pass_kernel.cu) ----
@@ -151,17 +146,57 @@ cudaError_t launch_pass_kernel(const MKLaunch &L, cudaStream_t st);
 
 // ---- launchers (each returns cudaGetLastError()) ----
 
-// Tensor-core linear: part[s][m][f] = sum over split s of x[m,k] * W[f,k], for f in the main
-// rows (and the adapter rows when with_lora).  x is read through a TMA map with box {64, BN}.
-cudaError_t launch_linear_partials(const CUtensorMap *x_map, int bn, const TiledWeight &w, int with_lora, int M,
-                                   const Partials &out, int *status, cudaStream_t st);
+// Standalone linear of few rows (linear_op.cu), one launch.
+struct LinOpArgs {
+    CUtensorMap xmap, wmap, amap;  // boxes {64, bn}, {64, 128}, {64, r}
+    int bn, kt_per, ks, M, N, r;   // kt_per: 64-wide K atoms per slice; ks <= LINEAR_OP_MAX_SLICES
+    float scale;
+    const bf16 *b;
+    bf16 *y;
+    int vec_store;  // y is 8-byte aligned
+    int *status;
+};
+constexpr int LINEAR_OP_MAX_ROWS = 64;
+constexpr int LINEAR_OP_MAX_SLICES = 16;  // one cluster
+cudaError_t launch_linear_op(const LinOpArgs &a, cudaStream_t st);
+cudaError_t configure_linear_op();
 
-// lm_head over the read-out rows: per 128-row vocabulary tile the (max, argmax) of each row,
-// and optionally the fp32 logits [rows][V].
-cudaError_t launch_lm_head(const CUtensorMap *x_map, int bn, const TiledWeight &w, int M, float *tile_max,
-                           int *tile_arg, float *logits, int *status, cudaStream_t st);
+// Linears of many rows (gemm.cu).  The caller fills everything but m_tiles and stages.
+enum GemmMode { GEMM_Y = 0, GEMM_GATE_UP = 1, GEMM_HEAD = 2 };
+struct GemmArgs {
+    CUtensorMap xmap;        // token rows, box {64, bn}
+    CUtensorMap wmap;        // row-major weight, box {64, 128} (when wt is null)
+    CUtensorMap bmap, umap;  // adapter (delta): B rows, box {64, 128}; u rows, box {64, bn}
+    const uint8_t *wt;       // pre-tiled weight (GEMM_GATE_UP: gate and up interleaved in 64-row blocks)
+    int k_tiles, slice_atoms, n_slices;  // 64-wide K atoms; atoms per slice; slices
+    int f_tiles;             // 128-feature tiles (GEMM_GATE_UP: of act features)
+    int bn, M;               // token tile (a multiple of 16, at most 256; 128 for GEMM_GATE_UP), token rows
+    int rows;                // features stored (the vocabulary for GEMM_HEAD)
+    int delta;               // adapter on: y += scale * u B^T
+    float scale;
+    bf16 *y;                 // [M][ld]
+    int ld, vec_store;       // vec_store: y is 16-byte aligned and ld a multiple of 8
+    float *logits;           // GEMM_HEAD: [M][rows] or null
+    float *tile_max;         // GEMM_HEAD: per CTA and token the (max, lowest argmax), [grid][M]
+    int *tile_arg;
+    int *status;
+    int m_tiles, stages;
+};
+// ctas: CTAs at most (0: one per SM)
+cudaError_t launch_gemm(GemmMode mode, GemmArgs &a, int ctas, cudaStream_t st);
+int gemm_pick_bn(int M, int f_tiles, int k_tiles, int max_bn, int ctas);
+int gemm_ctas();  // CTAs of a launch with ctas = 0
+cudaError_t configure_gemm_kernels();
 
-cudaError_t launch_argmax_reduce(const float *tile_max, const int *tile_arg, int n_tiles, int rows, int *ids_out,
+// lm_head over M <= 256 read-out rows: per CTA the (max, lowest argmax) of each row ([*n_parts][M]
+// entries of tile_max / tile_arg, at most V / 128 of them), and optionally the fp32 logits [M][V].
+// x_map: box {64, lm_head_box(M, K)}.  The weight is w.tiles (pre-tiled) or, when that is null, the
+// row-major matrix behind w_map.
+int lm_head_box(int M, int K);
+cudaError_t launch_lm_head(const CUtensorMap &x_map, const TiledWeight &w, const CUtensorMap *w_map, int M,
+                           float *tile_max, int *tile_arg, int *n_parts, float *logits, int *status, cudaStream_t st);
+
+cudaError_t launch_argmax_reduce(const float *tile_max, const int *tile_arg, int n_parts, int rows, int *ids_out,
                                  cudaStream_t st);
 
 // Builds the row token ids of a pass from the device state: draft [pending, -1 x D],
@@ -185,11 +220,9 @@ cudaError_t launch_accept_commit(const SeqState &s, int nb, int D, const int *dr
                                  const int *forced, int forced_stride, int max_new, int out_cap,
                                  int *accepted_out, cudaStream_t st);
 
-// Repack rows [0, rows) of a row-major bf16 matrix [rows, K] into the tiled layout at
-// destination row offset dst_row0.
-cudaError_t launch_repack_tiled(const void *src, int rows, int K, void *dst_tiles, int dst_row0, cudaStream_t st);
-// Same, with source row i placed on tile row dst_row0 + (i / group) * stride + i % group
-// (gate and up rows interleaved in 64-row blocks inside each 128-row tile).
+// Repack rows [0, rows) of a row-major bf16 matrix [rows, K] into the tiled layout: source row i
+// on tile row dst_row0 + (i / group) * stride + i % group (gate and up rows interleaved in 64-row
+// blocks inside each 128-row tile; group = rows: contiguous).
 cudaError_t launch_repack_tiled_map(const void *src, int rows, int K, void *dst_tiles, int dst_row0, int group,
                                     int stride, cudaStream_t st);
 
@@ -203,15 +236,23 @@ cudaError_t launch_set_len(int *L, int b, int value, cudaStream_t st);
 cudaError_t launch_prefill_finish(const SeqState &s, int b, int P, const int *first_id, int max_new, int out_cap,
                                   cudaStream_t st);
 
-// y[m, f] = bf16(sum of splits + scale * sum_j bf16(u_j) B[f, j]) for f < N (standalone linear).
-cudaError_t launch_linear_finalize(const Partials &P, int M, int N, int r, float scale, const void *lora_b, void *y,
-                                   cudaStream_t st);
+// B [N, r] -> [N, 32], zero beyond r (standalone linear of many rows whose B has no TMA layout).
+cudaError_t launch_pack_b(const void *b, int N, int r, void *out, cudaStream_t st);
 
 // 2-D bf16 row-major [rows, cols] tensor map, box {64, box_rows}, 128-byte swizzle.
 bool encode_bf16_map(CUtensorMap *map, const void *base, int rows, int cols, int box_rows);
 
 // Per-instantiation kernel attributes (dynamic shared memory), set once before any capture.
 cudaError_t configure_linear_kernels();
+
+// The standalone linear shared by pbd_op_linear and pbd_op_linear_static: scratch is at least
+// 1024 bytes for the status word, `tiles` (N / 128 (+ 1 with an adapter)) * (K / 64) * 16 KiB and
+// `part` 4 * slices * M * (N + r) bytes, all 1024-byte aligned, tiles right behind the first 1024.
+struct LinearScratch {
+    uint8_t *status, *tiles, *part;
+};
+pbd_status run_linear_op(int M, int K, int N, int r, float scale, const void *d_x, const void *d_w, const void *d_a,
+                         const void *d_b, void *d_y, const LinearScratch &ws, cudaStream_t st, const char *who);
 
 // Records the message pbd_op_last_error() returns on this thread.
 void op_record_error(const char *msg);
