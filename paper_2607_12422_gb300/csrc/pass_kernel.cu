@@ -38,6 +38,7 @@
 // is in.
 #include <algorithm>
 #include <cmath>
+#include <numeric>
 #include <vector>
 
 #include "common.cuh"
@@ -1533,7 +1534,11 @@ void mk_build_schedule(const Dims &dm, const PassDesc &pd, const std::vector<int
         const int items = (nsplit[bl] + span - 1) / span;
         merges += items <= grid ? items : 1;
     }
+    // The merges that an o slice waits for are counted per block of the attention width that holds
+    // whole KV groups and whole o slices: a group wider than a slice feeds several slices, and one that
+    // straddles a boundary feeds two.
     const int o_w = mk_slice_atoms(1, K[1]) * KT;  // o slice width
+    const int o_blk = std::lcm(gw, o_w);
     for (int m = 0; m < pd.M; ++m) push(MK_EMBED, 0, 0, m, 0, 0, -1, 0, cl.embed, -1);
     int prev = -1;  // the last layer run so far (skipped layers have no items)
     for (int l = 0; l < pd.nl_run; ++l) {
@@ -1565,17 +1570,13 @@ void mk_build_schedule(const Dims &dm, const PassDesc &pd, const std::vector<int
         for (int bl = 0; bl < pd.nb; ++bl)
             for (int g = 0; g < dm.Hkv; ++g)
                 for (int sp = 0; sp < (nsplit[bl] + span - 1) / span; ++sp)
-                    push(MK_ATTN, 0, l, bl, g, sp, ctr(l, cl.att_in + g), att_in_tgt[g], ctr(l, cl.att_o + g * gw / o_w),
+                    push(MK_ATTN, 0, l, bl, g, sp, ctr(l, cl.att_in + g), att_in_tgt[g], ctr(l, cl.att_o + g * gw / o_blk),
                          -1);
-        // o slice sl reads the heads of the groups g with g * gw / o_w == sl
         for (int r = 0; r < (pd.adapter ? 1 : 0) + n_main[1]; ++r) {
             const int t = pd.adapter ? (r == 0 ? n_main[1] : r - 1) : r;
-            for (int sl = 0; sl < ks[1]; ++sl) {
-                int groups = 0;
-                for (int g = 0; g < dm.Hkv; ++g) groups += (g * gw / o_w == sl) ? 1 : 0;
-                push(MK_LINEAR, 1, l, t, sl, 0, ctr(l, cl.att_o + sl), groups * merges,
+            for (int sl = 0; sl < ks[1]; ++sl)
+                push(MK_LINEAR, 1, l, t, sl, 0, ctr(l, cl.att_o + sl * o_w / o_blk), o_blk / gw * merges,
                      t < n_main[1] ? ctr(l, cl.res_o) : -1, -1);
-            }
         }
         linear(2, ctr(l, cl.res_o), n_main[1] * ks[1]);
         linear(3, -1, 0);
