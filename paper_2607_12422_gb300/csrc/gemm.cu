@@ -54,7 +54,8 @@ __global__ void __launch_bounds__(GM_THREADS, 1) k_gemm(const __grid_constant__ 
     __shared__ GemmState S;
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     constexpr int A_BYTES = TILE_BYTES * (MODE == GEMM_GATE_UP ? 2 : 1);
-    const int stage = A_BYTES + a.bn * 128, nst = a.stages;
+    const int apg = a.stage_atoms, x_off = apg * A_BYTES, x_bytes = a.bn * 128;
+    const int stage = x_off + apg * x_bytes, nst = a.stages;
     const int tiles = a.f_tiles * a.m_tiles;
     const int parts = a.n_slices + (a.delta ? 1 : 0);  // accumulation groups per tile
     if (threadIdx.x == 0) {
@@ -78,6 +79,7 @@ __global__ void __launch_bounds__(GM_THREADS, 1) k_gemm(const __grid_constant__ 
     tc_fence_after();
     const uint32_t tmem = S.tmem_slot;
 
+    pdl_launch();
     // Registers: the block starts with 3 x 128 threads x 168; the producer's warpgroup gives up
     // 128 x 128 of them and the two epilogue warpgroups take 128 x 56 each (40 + 2 x 224 <= 3 x 168),
     // which holds a tile's 128 running sums a thread without spills.
@@ -89,9 +91,34 @@ __global__ void __launch_bounds__(GM_THREADS, 1) k_gemm(const __grid_constant__ 
             int slot = 0, issued = 0;
             uint32_t ph = 1;  // (a fresh barrier counts as having completed the phase before its first)
             bool ok = true;
+            auto weights = [&](uint8_t *st, uint64_t *bar, int ft, int k) {
+                if constexpr (MODE == GEMM_GATE_UP) {
+                    // weight tile t holds gate rows 64t.. then up rows 64t..: two tiles make 128 of each
+                    for (int e = 0; e < apg; ++e)
+                        for (int j = 0; j < 2; ++j) {
+                            const uint8_t *src = a.wt + ((size_t)(2 * ft + j) * a.k_tiles + k + e) * TILE_BYTES;
+                            uint8_t *d = st + e * A_BYTES + j * (TILE_BYTES / 2);
+                            bulk_g2s(d, src, TILE_BYTES / 2, bar, pol);
+                            bulk_g2s(d + TILE_BYTES, src + TILE_BYTES / 2, TILE_BYTES / 2, bar, pol);
+                        }
+                } else if constexpr (TILED) {  // consecutive atoms of a weight tile are contiguous
+                    bulk_g2s(st, a.wt + ((size_t)ft * a.k_tiles + k) * TILE_BYTES, (uint32_t)(apg * TILE_BYTES), bar, pol);
+                } else {
+                    for (int e = 0; e < apg; ++e)
+                        tma_load_2d(st + e * A_BYTES, &a.wmap, (k + e) * KT, ft * TILE_ROWS, bar);
+                }
+            };
+            // pre-tiled weights are a context's own and depend on nothing before this kernel: the first
+            // stages' go out while that still runs (a caller's matrix may be what it writes)
+            const int early = TILED ? min(nst, a.k_tiles / apg) : 0;
+            for (int j = 0; j < early; ++j) {
+                mbar_arrive_expect_tx(&S.full[j], (uint32_t)stage);
+                weights(ring + j * stage, &S.full[j], blockIdx.x % a.f_tiles, j * apg);
+            }
+            pdl_wait();
             for (int t = blockIdx.x; ok && t < tiles; t += gridDim.x) {
                 const int ft = t % a.f_tiles, tok0 = (t / a.f_tiles) * a.bn;
-                for (int k = 0; k < a.k_tiles + (a.delta ? 1 : 0); ++k) {
+                for (int k = 0; k < a.k_tiles + (a.delta ? 1 : 0); k += apg) {
                     if (!mbar_wait(&S.empty[slot], ph, a.status, DEV_TIMEOUT_SLOT, &S.abort)) {
                         ok = false;
                         break;
@@ -100,25 +127,18 @@ __global__ void __launch_bounds__(GM_THREADS, 1) k_gemm(const __grid_constant__ 
                     uint64_t *bar = &S.full[slot];
                     if (++slot == nst) slot = 0, ph ^= 1;
                     ++issued;
-                    mbar_arrive_expect_tx(bar, (uint32_t)stage);
                     if (k == a.k_tiles) {  // the adapter: B rows by u rows
+                        mbar_arrive_expect_tx(bar, (uint32_t)(A_BYTES + x_bytes));
                         tma_load_2d(st, &a.bmap, 0, ft * TILE_ROWS, bar);
-                        tma_load_2d(st + A_BYTES, &a.umap, 0, tok0, bar);
+                        tma_load_2d(st + x_off, &a.umap, 0, tok0, bar);
                         continue;
                     }
-                    if (MODE == GEMM_GATE_UP) {
-                        // weight tile t holds gate rows 64t.. then up rows 64t..: two tiles make 128 of each
-                        for (int j = 0; j < 2; ++j) {
-                            const uint8_t *src = a.wt + ((size_t)(2 * ft + j) * a.k_tiles + k) * TILE_BYTES;
-                            bulk_g2s(st + j * (TILE_BYTES / 2), src, TILE_BYTES / 2, bar, pol);
-                            bulk_g2s(st + TILE_BYTES + j * (TILE_BYTES / 2), src + TILE_BYTES / 2, TILE_BYTES / 2, bar, pol);
-                        }
-                    } else if (TILED) {
-                        bulk_g2s(st, a.wt + ((size_t)ft * a.k_tiles + k) * TILE_BYTES, TILE_BYTES, bar, pol);
-                    } else {
-                        tma_load_2d(st, &a.wmap, k * KT, ft * TILE_ROWS, bar);
+                    if (issued > early) {
+                        mbar_arrive_expect_tx(bar, (uint32_t)stage);
+                        weights(st, bar, ft, k);
                     }
-                    tma_load_2d(st + A_BYTES, &a.xmap, k * KT, tok0, bar);
+                    for (int e = 0; e < apg; ++e)
+                        tma_load_2d(st + x_off + e * x_bytes, &a.xmap, (k + e) * KT, tok0, bar);
                 }
             }
             if (*(volatile int *)&S.abort)  // error path: the copies in flight get a bounded chance to land
@@ -141,27 +161,30 @@ __global__ void __launch_bounds__(GM_THREADS, 1) k_gemm(const __grid_constant__ 
                     const uint32_t d = tmem + (uint32_t)(buf * GM_BUF);
                     const bool dl = s == a.n_slices;
                     const int atoms = dl ? 1 : a.slice_atoms;
-                    for (int k = 0; k < atoms; ++k) {
+                    for (int k = 0; k < atoms; k += apg) {
                         if (!mbar_wait(&S.full[slot], ph, a.status, DEV_TIMEOUT_LOAD, &S.abort)) {
                             ok = false;
                             break;
                         }
                         tc_fence_after();
                         const uint8_t *st = ring + slot * stage;
-                        const uint64_t wd = sw128_kmajor_desc(st), xd = sw128_kmajor_desc(st + A_BYTES);
+                        uint64_t wd = sw128_kmajor_desc(st), xd = sw128_kmajor_desc(st + x_off);
                         if (dl) {  // K = 32: ranks up to 32, zero beyond the rank
 #pragma unroll
                             for (int kk = 0; kk < 2; ++kk)
                                 mma_bf16_ss(d, wd + 2ull * kk, xd + 2ull * kk, idesc, kk != 0 ? 1u : 0u);
                         } else {
-#pragma unroll
-                            for (int kk = 0; kk < KT / 16; ++kk)
-                                mma_bf16_ss(d, wd + 2ull * kk, xd + 2ull * kk, idesc, (k | kk) != 0 ? 1u : 0u);
-                            if (MODE == GEMM_GATE_UP) {
-                                const uint64_t ud = sw128_kmajor_desc(st + TILE_BYTES);
+#pragma unroll 1
+                            for (int e = 0; e < apg; ++e, wd += A_BYTES / 16, xd += x_bytes / 16) {
 #pragma unroll
                                 for (int kk = 0; kk < KT / 16; ++kk)
-                                    mma_bf16_ss(d + a.bn, ud + 2ull * kk, xd + 2ull * kk, idesc, (k | kk) != 0 ? 1u : 0u);
+                                    mma_bf16_ss(d, wd + 2ull * kk, xd + 2ull * kk, idesc, (k | e | kk) != 0 ? 1u : 0u);
+                                if (MODE == GEMM_GATE_UP) {
+                                    const uint64_t ud = wd + TILE_BYTES / 16;
+#pragma unroll
+                                    for (int kk = 0; kk < KT / 16; ++kk)
+                                        mma_bf16_ss(d + a.bn, ud + 2ull * kk, xd + 2ull * kk, idesc, (k | e | kk) != 0 ? 1u : 0u);
+                                }
                             }
                         }
                         mma_commit(&S.empty[slot]);
@@ -177,6 +200,7 @@ __global__ void __launch_bounds__(GM_THREADS, 1) k_gemm(const __grid_constant__ 
         }
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 224;");
+        pdl_wait();  // (the stores below)
         // ---- epilogue: warp w owns TMEM lane quarter w % 4 (32 features) and every other chunk of
         // 16 token columns
         const int q = warp & 3, hh = (warp - 4) >> 2;
@@ -372,11 +396,16 @@ int gemm_pick_bn(int M, int f_tiles, int k_tiles, int max_bn, int ctas) {
 
 template <int MODE, bool TILED>
 static cudaError_t launch_one(GemmArgs &a, int ctas, cudaStream_t st) {
-    const int stage = TILE_BYTES * (MODE == GEMM_GATE_UP ? 2 : 1) + a.bn * 128;
-    a.stages = std::min<int>(GM_MAX_STAGES, (int)((GM_SMEM - sizeof(GemmState) - 2048) / stage));
+    // Atoms per ring stage: a stage costs the issuing threads about 200 ns of waiting, announcing and
+    // committing whatever its size (measured), as long as the MMAs of one atom up to bn = 128; two
+    // atoms share it where at least three stages still fit and slices hold whole stages.
+    const int atom = TILE_BYTES * (MODE == GEMM_GATE_UP ? 2 : 1) + a.bn * 128;
+    const int room = (int)(GM_SMEM - sizeof(GemmState) - 2048);
+    a.stage_atoms = (a.slice_atoms % 2 == 0 && room / (2 * atom) >= 3) ? 2 : 1;
+    const int stage = a.stage_atoms * atom;
+    a.stages = std::min<int>(GM_MAX_STAGES, room / stage);
     const int grid = std::min(ctas, a.f_tiles * a.m_tiles);
-    k_gemm<MODE, TILED><<<grid, GM_THREADS, (size_t)a.stages * stage + 1024, st>>>(a);
-    return cudaGetLastError();
+    return launch_pdl(k_gemm<MODE, TILED>, grid, GM_THREADS, (size_t)a.stages * stage + 1024, st, a);
 }
 
 cudaError_t launch_gemm(GemmMode mode, GemmArgs &a, int ctas, cudaStream_t st) {

@@ -223,6 +223,7 @@ cudaError_t configure_linear_kernels() {
     set((const void *)k_lm_head<64, false>, LmhLayout<64>::TOTAL);
     if (e == cudaSuccess) e = configure_linear_op();
     if (e == cudaSuccess) e = configure_gemm_kernels();
+    if (e == cudaSuccess) e = configure_rows_kernels();
     if (e == cudaSuccess && dev < 64) done[dev] = true;
     return e;
 }

@@ -1,7 +1,7 @@
 // ops.cu -- small kernels around the persistent pass kernel:
 //   k_build_ids       row token ids of a draft / verify / decode pass from the device state
 //   k_accept_commit   longest accepted prefix, emission, KV commit (Section 3, steps 4-5)
-//   k_prefill_finish  cached length and first token after a prompt
+//   k_prefill_finish  cached lengths and first tokens after prompts
 //   k_repack_tiled    row-major bf16 weights -> 128 x 64 tiles in the 128-byte swizzle layout
 //   k_read_kv         paged cache -> contiguous rows (tests of the commit rule)
 //   k_pack_b          adapter B rows padded to 32 columns (standalone linear)
@@ -141,18 +141,22 @@ cudaError_t launch_set_len(int *L, int b, int value, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-__global__ void k_prefill_finish(SeqState s, int b, int P, const int *first_id, int max_new, int out_cap) {
-    const int t = *first_id;
-    s.L[b] = P;
-    s.pending[b] = t;
-    s.out_tokens[(size_t)b * out_cap] = t;
-    s.n_out[b] = 1;
-    s.done[b] = max_new <= 1 ? 1 : 0;
+__global__ void k_prefill_finish(SeqState s, const RowSeg *segs, const int *ro, int n_ro, const int *first_ids,
+                                 int max_new, int out_cap) {
+    for (int r = threadIdx.x; r < n_ro; r += blockDim.x) {
+        const RowSeg sg = segs[ro[r]];
+        const int b = sg.seq, t = first_ids[r];
+        s.L[b] = sg.pos0 + sg.n;
+        s.pending[b] = t;
+        s.out_tokens[(size_t)b * out_cap] = t;
+        s.n_out[b] = 1;
+        s.done[b] = max_new <= 1 ? 1 : 0;
+    }
 }
 
-cudaError_t launch_prefill_finish(const SeqState &s, int b, int P, const int *first_id, int max_new, int out_cap,
-                                  cudaStream_t st) {
-    k_prefill_finish<<<1, 1, 0, st>>>(s, b, P, first_id, max_new, out_cap);
+cudaError_t launch_prefill_finish(const SeqState &s, const RowSeg *segs, const int *ro, int n_ro, const int *first_ids,
+                                  int max_new, int out_cap, cudaStream_t st) {
+    k_prefill_finish<<<1, 64, 0, st>>>(s, segs, ro, n_ro, first_ids, max_new, out_cap);
     return cudaGetLastError();
 }
 

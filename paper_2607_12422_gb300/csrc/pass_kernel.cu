@@ -342,12 +342,6 @@ __device__ __forceinline__ void sum_parts(const MKParams &P, int lin, int m, int
     }
 }
 
-// element (v, k) of a matrix in the 128 x 64 swizzled tile layout
-__device__ __forceinline__ const bf16 *tiled_at(const bf16 *tiles, int K, int v, int k) {
-    const int t = v >> 7, r = v & 127, kt = k >> 6, c = (k & 63) >> 3, e = k & 7;
-    return tiles + ((size_t)t * (K >> 6) + kt) * (TILE_ROWS * KT) + r * KT + ((c ^ (r & 7)) << 3) + e;
-}
-
 // ------------------------------------------------------------------ work items
 
 // token / mask-embedding row -> residual h and its per-tile sums of squares.  A mask row is

@@ -19,7 +19,6 @@ constexpr int PAGE = 16;           // KV page length in tokens
 constexpr int ATT_SPLIT = 128;     // key positions per attention split (position-aligned)
 constexpr int ATT_SUBS_MAX = 2;    // partial results per split at most (its two 64-key halves)
 constexpr int ATT_SPAN_MAX = 2;    // 128-key splits per attention item at most
-constexpr int PREFILL_ROWS = 64;   // rows per prefill chunk
 constexpr int KT = 64;             // K elements per 128-byte swizzle atom row (bf16)
 constexpr int TILE_ROWS = 128;     // output features per tensor-core tile
 constexpr int TILE_BYTES = TILE_ROWS * KT * 2;  // 16 KiB per pre-tiled weight tile
@@ -144,6 +143,48 @@ size_t mk_union_bytes(int bn, int head_dim, int att_span);
 int mk_slice_atoms(int lin, int K);  // 64-wide K atoms per work item of linear `lin`
 cudaError_t launch_pass_kernel(const MKLaunch &L, cudaStream_t st);
 
+// ---- passes over many rows: prompt processing (rows.cu, gemm.cu) ----
+
+// Rows row0 .. row0 + n - 1 of a pass hold positions pos0 .. pos0 + n - 1 of sequence seq.
+struct RowSeg {
+    int row0, seq, pos0, n;
+};
+// One attention work item: rows_attn_tile() (row, head) pairs of a segment and KV head, from pair q0
+// (pair = row in segment * heads per group + head in group).
+struct RowsAttn {
+    int seg, g, q0, pad;
+};
+struct RowsArgs {
+    Dims dm;
+    int M, n_seg;
+    const RowSeg *segs;  // ascending row0, covering rows 0 .. M - 1
+    bf16 *h, *x, *qkv, *q, *attn, *y;
+    KVCache kv;
+    int att_subs;        // partial results per 128-key split (as in the decoding passes)
+    float att_scale;
+    int max_ctas;        // CTAs per launch at most (0: no limit)
+    int *status;
+};
+int rows_attn_tile();
+cudaError_t configure_rows_kernels();
+cudaError_t launch_rows_embed(const RowsArgs &a, const int *ids, const void *embed_tiled, const void *gain,
+                              cudaStream_t st);
+cudaError_t launch_rows_norm(const RowsArgs &a, const void *gain, cudaStream_t st);  // gain null: residual only
+cudaError_t launch_rows_rope(const RowsArgs &a, int layer, const void *q_norm, const void *k_norm,
+                             const float2 *rope_cs, cudaStream_t st);
+cudaError_t launch_rows_attn(const RowsArgs &a, const CUtensorMap &kmap, const CUtensorMap &vmap, int layer,
+                             const RowsAttn *work, int n_work, cudaStream_t st);
+// x_ro[r] = final norm of the last row of segment ro[r]
+cudaError_t launch_rows_final(const RowsArgs &a, const int *ro, int n_ro, const void *gain, void *x_ro, cudaStream_t st);
+
+#ifdef __CUDACC__
+// element (v, k) of a matrix in the 128 x 64 swizzled tile layout
+__device__ __forceinline__ const bf16 *tiled_at(const bf16 *tiles, int K, int v, int k) {
+    const int t = v >> 7, r = v & 127, kt = k >> 6, c = (k & 63) >> 3, e = k & 7;
+    return tiles + ((size_t)t * (K >> 6) + kt) * (TILE_ROWS * KT) + r * KT + ((c ^ (r & 7)) << 3) + e;
+}
+#endif
+
 // ---- launchers (each returns cudaGetLastError()) ----
 
 // Standalone linear of few rows (linear_op.cu), one launch.
@@ -161,7 +202,7 @@ constexpr int LINEAR_OP_MAX_SLICES = 16;  // one cluster
 cudaError_t launch_linear_op(const LinOpArgs &a, cudaStream_t st);
 cudaError_t configure_linear_op();
 
-// Linears of many rows (gemm.cu).  The caller fills everything but m_tiles and stages.
+// Linears of many rows (gemm.cu).  The caller fills everything but the last line.
 enum GemmMode { GEMM_Y = 0, GEMM_GATE_UP = 1, GEMM_HEAD = 2 };
 struct GemmArgs {
     CUtensorMap xmap;        // token rows, box {64, bn}
@@ -180,7 +221,7 @@ struct GemmArgs {
     float *tile_max;         // GEMM_HEAD: per CTA and token the (max, lowest argmax), [grid][M]
     int *tile_arg;
     int *status;
-    int m_tiles, stages;
+    int m_tiles, stages, stage_atoms;
 };
 // ctas: CTAs at most (0: one per SM)
 cudaError_t launch_gemm(GemmMode mode, GemmArgs &a, int ctas, cudaStream_t st);
@@ -229,12 +270,13 @@ cudaError_t launch_repack_tiled_map(const void *src, int rows, int K, void *dst_
 cudaError_t launch_read_kv(const Dims &dm, const KVCache &kv, int layer, int seq, int n, void *k_out, void *v_out,
                            cudaStream_t st);
 
-// L[b] = value (prefill chunks run at L = chunk start).
+// L[b] = value.
 cudaError_t launch_set_len(int *L, int b, int value, cudaStream_t st);
 
-// After the prompt of sequence b: L = P, pending = first token = output token 0.
-cudaError_t launch_prefill_finish(const SeqState &s, int b, int P, const int *first_id, int max_new, int out_cap,
-                                  cudaStream_t st);
+// After the prompts that end in segments ro[0 .. n_ro): L = the segment's end, pending = first token
+// first_ids[r] = output token 0.
+cudaError_t launch_prefill_finish(const SeqState &s, const RowSeg *segs, const int *ro, int n_ro, const int *first_ids,
+                                  int max_new, int out_cap, cudaStream_t st);
 
 // B [N, r] -> [N, 32], zero beyond r (standalone linear of many rows whose B has no TMA layout).
 cudaError_t launch_pack_b(const void *b, int N, int r, void *out, cudaStream_t st);

@@ -92,3 +92,60 @@ def test_lm_head_edges(torch, M, H, V):
     assert (want < max(V // 2, 1)).all()
     plain, none = pbd.pbd_op_lm_head_argmax(x, E)
     assert none is None and torch.equal(plain, ids)
+
+
+@pytest.mark.parametrize("shape,max_seq,start,rounds,ctas", [("tiny", 256, 1, 9, 0), ("qwen2", 420, 40, 21, 0),
+                                                            ("qwen2", 4096, 301, 30, 0), ("grp4", 420, 17, 10, 0),
+                                                            ("qwen2", 420, 130, 14, 20)])
+def test_prefill_equals_decoded_rows_bitwise(torch, shape, max_seq, start, rounds, ctas):
+    """The many-row kernels of the prefill against the pass kernel: K/V of every layer, written by
+    verify rounds that commit 17 random tokens each, equal a prefill of the same tokens, and so do the
+    logits that follow.  Both partitions of an attention split (two halves; whole, at max_seq 4096),
+    heads of 64 and 128, one to four query heads per KV head, last tiles of 1 to 128 rows, few CTAs."""
+    import dataclasses
+    from paper_2607_12422_gb300 import pbd, synth
+    S = synth.TINY if shape == "tiny" else dataclasses.replace(synth.QWEN3_0_6B, n_layers=2, vocab=4096)
+    if shape == "grp4":
+        S = dataclasses.replace(S, n_kv_heads=4, hidden=1280, intermediate=1792)
+    D = 16
+    base, ad = synth.with_random_norm_gains(synth.gen_base_weights(S)), synth.gen_adapter(S)
+    eng = pbd.Engine(S, base, ad, block_D=D, max_batch=1, max_seq_len=max_seq, max_ctas=ctas)
+    rng = np.random.default_rng(start)
+    prompt = rng.integers(0, S.vocab, start).astype(np.int32)
+    eng.pbd_prefill([prompt], max_new=(D + 1) * rounds + 2)
+    for _ in range(rounds):
+        eng.pbd_verify_block(drafts=rng.integers(0, S.vocab, (1, D)).astype(np.int32))
+        eng.pbd_accept_commit(forced_n=[D])
+    L, pend, n_out = (int(z[0]) for z in eng.pbd_get_state())
+    toks = eng.pbd_get_tokens()[0].cpu().numpy()[:n_out]
+    kv = [eng.pbd_read_kv(l, 0, L) for l in range(S.n_layers)]
+    _, lg = eng.pbd_decode_step(want_logits=True)
+    seq = np.concatenate([prompt, toks[:-1]]).astype(np.int32)
+    assert len(seq) == L
+    first = eng.pbd_prefill([seq], max_new=2)
+    assert int(first[0]) == pend
+    for l in range(S.n_layers):
+        k, v = eng.pbd_read_kv(l, 0, L)
+        assert torch.equal(kv[l][0], k) and torch.equal(kv[l][1], v), l
+    _, lg2 = eng.pbd_decode_step(want_logits=True)
+    assert torch.equal(lg, lg2)
+    eng.close()
+
+
+def test_prefill_batch_and_passes_match_single_prompts(torch):
+    """Ragged prompts share passes and a long one spans two (4096 rows each): first tokens and last-layer
+    K/V equal those of each prompt alone."""
+    import dataclasses
+    from paper_2607_12422_gb300 import pbd, synth
+    S = dataclasses.replace(synth.TINY, vocab=1024)
+    base, ad = synth.gen_base_weights(S), synth.gen_adapter(S)
+    rng = np.random.default_rng(4)
+    prompts = [rng.integers(0, S.vocab, n).astype(np.int32) for n in (1, 65, 4100, 300, 17)]
+    eng = pbd.Engine(S, base, ad, block_D=4, max_batch=5, max_seq_len=4200)
+    first = eng.pbd_prefill(prompts, max_new=4).cpu().numpy()
+    kv = [eng.pbd_read_kv(S.n_layers - 1, b, len(p)) for b, p in enumerate(prompts)]
+    for b, p in enumerate(prompts):
+        assert int(eng.pbd_prefill([p], max_new=4)[0]) == first[b], b
+        k, v = eng.pbd_read_kv(S.n_layers - 1, 0, len(p))
+        assert torch.equal(k, kv[b][0]) and torch.equal(v, kv[b][1]), b
+    eng.close()
