@@ -74,8 +74,8 @@ typedef struct {
                                  writes no K/V there); 0 = none.  Bits at or above n_layers must be
                                  clear, and the draft must keep at least one layer (together with
                                  draft_layers) */
-    int32_t max_ctas;         /* CTAs of the persistent pass kernel: 0 = one per SM; otherwise at most
-                                 max_ctas (leaving SMs to other work).  It must be at least the largest
+    int32_t max_ctas;         /* 0 = the whole GPU; otherwise at most max_ctas CTAs at a time (leaving SMs
+                                 to other work): decoding passes then run as the persistent pass kernel.  It must be at least the largest
                                  number of K slices of one linear, whose reductions wait for one
                                  another and so must sit on distinct CTAs: pbd_create fails with
                                  PBD_ERR_INVALID_ARG below that */
@@ -187,17 +187,17 @@ pbd_status pbd_sync(pbd_ctx *ctx);
 pbd_status pbd_bench_rounds(pbd_ctx *ctx, int32_t mode, int32_t warmup, int32_t steps,
                             const int32_t *d_forced_n_seq_opt, double *h_ms, int32_t *h_launches);
 
-/* Times the persistent pass kernel alone (all decoder layers of one pass; the lm_head and the
- * small kernels around it excluded).  On a prefilled context, launches the draft (kind 0),
- * verify (1) or plain-decoding (2) pass kernel `iters` times with CUDA events bracketing each
- * launch; the decoding state is not advanced, so every launch does the same work, and the
+/* Times the decoder layers of one pass alone (the lm_head and the small kernels around them
+ * excluded).  On a prefilled context, runs the layers of the draft (kind 0), verify (1) or
+ * plain-decoding (2) pass `iters` times with CUDA events bracketing each run; the decoding state is not advanced, so every launch does the same work, and the
  * weights it streams (about 0.9 GB for the 0.6B shape) exceed L2.  *h_ms_per_launch receives the
  * mean duration; *h_bytes_per_launch the algorithmic bytes of one launch: every layer weight once
  * (adapter factors too for the draft), the cached K/V read and the block's K/V written. */
 pbd_status pbd_time_pass(pbd_ctx *ctx, int32_t kind, int32_t iters, double *h_ms_per_launch,
                          double *h_bytes_per_launch);
 
-/* Timeline of one pass of the persistent kernel (a profiling aid; the paper's Appendix A.5 profiles
+/* Timeline of one pass of the persistent kernel, which contexts limited by max_ctas (and shapes that do not
+ * fit the kernel chain) decode with; it can be traced on any context (a profiling aid; the paper's Appendix A.5 profiles
  * draft and verify forward latency).  On a prefilled context, runs one draft (kind 0), verify (1)
  * or plain-decoding (2) pass without advancing the state, recording for every work item sixteen
  * %globaltimer stamps in ns: start, inputs complete, main work done, end, then per item kind

@@ -224,6 +224,7 @@ cudaError_t configure_linear_kernels() {
     if (e == cudaSuccess) e = configure_linear_op();
     if (e == cudaSuccess) e = configure_gemm_kernels();
     if (e == cudaSuccess) e = configure_rows_kernels();
+    if (e == cudaSuccess) e = configure_step_kernels();
     if (e == cudaSuccess && dev < 64) done[dev] = true;
     return e;
 }

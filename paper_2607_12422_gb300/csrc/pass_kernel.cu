@@ -41,6 +41,7 @@
 #include <numeric>
 #include <vector>
 
+#include "attn.cuh"
 #include "common.cuh"
 #include "pbd_internal.h"
 
@@ -657,14 +658,7 @@ __device__ __noinline__ void reduce_gu(const MKParams &P, int layer, int tile, i
 
 // ---- attention
 
-// Attention split staging layout in the union buffer: K then V, each DH/64 sub-tiles of
-// [128 keys x 128 bytes] in the 128-byte swizzle layout (16-byte chunk c of key n at
-// (c ^ (n & 7)) * 16), exactly as the tiled TMA writes them.
-constexpr int ATT_SUB_BYTES = ATT_SPLIT * 128;
-
-__device__ __forceinline__ uint32_t sw128(int row, int colb) {
-    return (uint32_t)(row * 128 + ((((colb >> 4) ^ (row & 7)) << 4) | (colb & 15)));
-}
+// Attention split staging in the union buffer: per split K, then V, laid out as attn.cuh describes.
 
 // TMA loads of the pages of one attention item (att_span consecutive 128-key splits), issued by
 // one warp of the compute group (all lanes call): stage 0 = pages entirely below the cached length
@@ -748,7 +742,8 @@ __device__ __noinline__ void attn_split(const MKParams &P, int layer, int bl, in
     for (int unit = cw; unit < n_mt * nsx * subs; unit += CT / 32) {
         const int mt = unit / (nsx * subs), sp = (unit / subs) % nsx, half = unit % subs, kb = half * HALF;
         const int k0 = (sp0 + sp) * ATT_SPLIT;
-        const uint8_t *sK = smem + sp * SPB, *sV = sK + SUBS * ATT_SUB_BYTES;
+        const uint32_t ka = smem_u32(smem + sp * SPB) + attn_k_lane(lane) + kb * 128;
+        const uint32_t va = smem_u32(smem + sp * SPB + SUBS * ATT_SUB_BYTES) + attn_v_lane(lane) + kb * 128;
         const int qv0 = mt * 16 + gq, qv1 = qv0 + 8;
         const bool val0 = qv0 < QV, val1 = qv1 < QV;
         const int i0 = val0 ? qv0 / grp : 0, i1 = val1 ? qv1 / grp : 0;
@@ -779,24 +774,7 @@ __device__ __noinline__ void attn_split(const MKParams &P, int layer, int bl, in
 #pragma unroll 1
         for (int c0 = 0; c0 < kend; c0 += 8 * CN) {
             float sc[CN][4];
-#pragma unroll
-            for (int nt = 0; nt < CN; ++nt) {
-                sc[nt][0] = sc[nt][1] = sc[nt][2] = sc[nt][3] = 0.f;
-                // K fragments of two k-steps per ldmatrix.x4: matrix j = keys n0..n0+7, dims 8j..8j+7
-                // of the 32-dim chunk; thread t addresses row t % 8 of matrix t / 8
-                const int kr = kb + c0 + nt * 8 + (lane & 7);
-#pragma unroll
-                for (int ks = 0; ks < KS; ks += 2) {
-                    const int e = ks * 16 + (lane >> 3) * 8;
-                    const uint32_t addr = smem_u32(sK + (e >> 6) * ATT_SUB_BYTES + sw128(kr, (e & 63) * 2));
-                    uint32_t b0, b1, b2, b3;
-                    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
-                                 : "=r"(b0), "=r"(b1), "=r"(b2), "=r"(b3)
-                                 : "r"(addr));
-                    mma_m16n8k16_bf16(sc[nt], qa[ks], b0, b1);
-                    mma_m16n8k16_bf16(sc[nt], qa[ks + 1], b2, b3);
-                }
-            }
+            attn_scores<DH>(ka + c0 * 128, qa, sc);
             float c0m = -INFINITY, c1m = -INFINITY;
 #pragma unroll
             for (int nt = 0; nt < CN; ++nt)
@@ -834,8 +812,8 @@ __device__ __noinline__ void attn_split(const MKParams &P, int layer, int bl, in
             for (int nt = 0; nt < CN; ++nt)
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {
-                    sc[nt][e] = sc[nt][e] == -INFINITY ? 0.f : __expf(sc[nt][e] - z0);
-                    sc[nt][2 + e] = sc[nt][2 + e] == -INFINITY ? 0.f : __expf(sc[nt][2 + e] - z1);
+                    sc[nt][e] = __expf(sc[nt][e] - z0);  // (0 for a masked score)
+                    sc[nt][2 + e] = __expf(sc[nt][2 + e] - z1);
                     l0 += sc[nt][e];
                     l1 += sc[nt][2 + e];
                 }
@@ -847,7 +825,6 @@ __device__ __noinline__ void attn_split(const MKParams &P, int layer, int bl, in
                 pa[1] = pack_bf162(sc[2 * kstep][2], sc[2 * kstep][3]);
                 pa[2] = pack_bf162(sc[2 * kstep + 1][0], sc[2 * kstep + 1][1]);
                 pa[3] = pack_bf162(sc[2 * kstep + 1][2], sc[2 * kstep + 1][3]);
-                const int vrow = kb + c0 + kstep * 16 + (lane & 7) + ((lane >> 3) & 1) * 8;
                 // V of keys at or past T is set to zero in the fragments: their weights are 0, but
                 // their rows hold whatever the cache or shared memory held (a page's tail beyond the
                 // sequence, or pages not loaded at all), and 0 times an Inf or NaN there would
@@ -860,17 +837,7 @@ __device__ __noinline__ void attn_split(const MKParams &P, int layer, int bl, in
                     ma = (ka < T ? 0x0000FFFFu : 0u) | (ka + 1 < T ? 0xFFFF0000u : 0u);
                     mb = (ka + 8 < T ? 0x0000FFFFu : 0u) | (ka + 9 < T ? 0xFFFF0000u : 0u);
                 }
-#pragma unroll
-                for (int dt = 0; dt < DT; dt += 2) {
-                    const int vcol = dt * 8 + (lane >> 4) * 8;
-                    const uint32_t addr = smem_u32(sV + (vcol >> 6) * ATT_SUB_BYTES + sw128(vrow, (vcol & 63) * 2));
-                    uint32_t r0, r1, r2, r3;
-                    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
-                                 : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
-                                 : "r"(addr));
-                    mma_m16n8k16_bf16(oc[dt], pa, r0 & ma, r1 & mb);
-                    mma_m16n8k16_bf16(oc[dt + 1], pa, r2 & ma, r3 & mb);
-                }
+                attn_pv<DH>(va + (c0 + kstep * 16) * 128, pa, ma, mb, oc);
             }
         }
         stamp_at(sw, 10);

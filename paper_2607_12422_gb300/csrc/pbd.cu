@@ -101,6 +101,15 @@ struct pbd_ctx {
     CounterLayout cl;
     Sched sched[N_PK];
     RowsBuf rows;
+    // decoding passes as kernel chains (steps.cu): whether this generation's pass kinds fit, and
+    // the chain of each kind as a graph, built on a kind's second call of a generation plan
+    void *step_act;  // SiLU(gate) * up rows, bf16
+    bool steps[N_PK] = {false, false, false, false};
+    int nsplit_max = 0;
+    struct StepGraph {
+        cudaGraphExec_t gx = nullptr;
+        int batch = 0, nsplit = 0, calls = 0;
+    } step_graph[N_PK];
     SeqState s;
     CUtensorMap maps[16];    // x_ro, box height 16 (i + 1)
     CUtensorMap kmap, vmap;  // paged K and V caches
@@ -123,6 +132,8 @@ struct pbd_ctx {
         bench_batch[mode] = 0;
     }
     ~pbd_ctx() {
+        for (auto &g : step_graph)
+            if (g.gx) cudaGraphExecDestroy(g.gx);
         drop_bench_graphs(0);
         drop_bench_graphs(1);
     }
@@ -290,6 +301,7 @@ size_t layout(pbd_ctx *c, void *base) {
     c->attn = bp.take(e2 * RA * Hq * d);
     c->act_bytes = sizeof(unsigned long long) * RA * (I / 2);  // tagged words of two bf16
     c->act = bp.take(c->act_bytes);
+    c->step_act = bp.take(e2 * RA * I);
     c->x_ro = bp.take(e2 * c->ro_alloc * H);
     c->ss = (float *)bp.take(sizeof(float) * RA * (H / TILE_ROWS));
     for (int lin = 0; lin < 4; ++lin) {
@@ -550,9 +562,101 @@ pbd_status enqueue_head(pbd_ctx *c, int n_ro, int *ids_out, float *logits) {
     return PBD_OK;
 }
 
+// attention split items per sequence over the whole generation (positions up to P + max_new + 2(D+1))
+std::vector<int> decode_splits(pbd_ctx *c) {
+    std::vector<int> ns(c->batch);
+    for (int b = 0; b < c->batch; ++b) {
+        const int tmax = std::min(c->prompt_lens[b] + c->max_new + 2 * (c->D + 1), c->pages_per_seq * PAGE);
+        ns[b] = std::min(c->n_splits, (tmax + ATT_SPLIT - 1) / ATT_SPLIT);
+    }
+    return ns;
+}
+
+// Builds and uploads the pass kernel's schedule of a pass kind unless this generation has it.
+pbd_status ensure_schedule(pbd_ctx *c, int kind, const PassDesc &pd) {
+    return c->sched[kind].valid ? PBD_OK : upload_schedule(c, kind, pd, decode_splits(c));
+}
+
+// All decoder layers of a pass as a chain of kernels.
+pbd_status enqueue_steps(pbd_ctx *c, const PassDesc &pd, int nsplit) {
+    const pbd_config &k = c->cfg;
+    StepArgs a{};
+    a.dm = c->dm;
+    a.pd = pd;
+    a.L = c->s.L;
+    a.ids = c->ids;
+    a.kv = c->kv;
+    a.h = static_cast<bf16 *>(c->h);
+    a.q = static_cast<bf16 *>(c->q);
+    a.attn = static_cast<bf16 *>(c->attn);
+    a.act = static_cast<bf16 *>(c->step_act);
+    a.ss = c->ss;
+    a.rows_alloc = c->rows_alloc;
+    a.rope_cs = c->rope_cs;
+    a.rope_rows = c->rope_rows;
+    a.att_subs = att_subs_of(c);
+    a.att_scale = (float)(1.0 / std::sqrt((double)k.head_dim));
+    a.o_part = c->o_part;
+    a.ml_part = c->ml_part;
+    a.att_splits_alloc = c->n_splits * a.att_subs;
+    a.status = c->status;
+    CK(launch_step_embed(a, c->w_lm.tiles, c->mask_embed, c->st));
+    for (int l = 0; l < pd.nl_run; ++l) {
+        if (l < 64 && ((pd.skip >> l) & 1u)) continue;
+        for (int lin = 0; lin < 4; ++lin) {
+            StepLin w{};
+            w.tiles = static_cast<const uint8_t *>(c->w[lin][l].tiles);
+            w.K = c->w[lin][l].K;
+            w.n_main = c->w[lin][l].n_main;
+            w.layer = l;
+            w.gain = static_cast<const bf16 *>(lin == 0 ? c->attn_norm : c->mlp_norm) + (size_t)l * k.hidden;
+            w.q_norm = static_cast<const bf16 *>(c->q_norm) + (size_t)l * k.head_dim;
+            w.k_norm = static_cast<const bf16 *>(c->k_norm) + (size_t)l * k.head_dim;
+            w.lora_b = static_cast<const bf16 *>(c->lb[lin]) + (size_t)l * w.n_main * k.lora_rank;
+            CK(launch_step_linear(lin, a, w, c->st));
+            if (lin == 0) CK(launch_step_attn(a, c->kmap, c->vmap, l, nsplit, c->st));
+        }
+    }
+    if (pd.ro_count > 0) CK(launch_step_final(a, c->final_norm, c->x_ro, c->st));
+    return PBD_OK;
+}
+
+// The decoder layers of one pass of a decoding kind: the kernel chain (as a graph from a kind's second
+// call on; inside a capture, or on the legacy stream, launch by launch) or the persistent kernel.
+pbd_status enqueue_layers(pbd_ctx *c, const PassDesc &pd, int kind) {
+    if (!c->steps[kind]) {
+        if (!c->sched[kind].valid) return fail(c, PBD_ERR_STATE, "no schedule for pass kind %d", kind);
+        return enqueue_pass_kernel(c, pd, kind);
+    }
+    if (kind == PK_PREFILL) return enqueue_steps(c, pd, (pd.R + ATT_SPLIT - 1) / ATT_SPLIT);
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    const bool legacy = c->st == nullptr || c->st == cudaStreamLegacy;
+    if (!legacy) CK(cudaStreamIsCapturing(c->st, &cap));
+    pbd_ctx::StepGraph &g = c->step_graph[kind];
+    if (legacy || cap != cudaStreamCaptureStatusNone) return enqueue_steps(c, pd, c->nsplit_max);
+    if (g.batch != c->batch || g.nsplit != c->nsplit_max) {
+        if (g.gx) cudaGraphExecDestroy(g.gx);
+        g = pbd_ctx::StepGraph();
+        g.batch = c->batch;
+        g.nsplit = c->nsplit_max;
+    }
+    if (!g.gx) {
+        if (g.calls++ == 0) return enqueue_steps(c, pd, c->nsplit_max);
+        cudaGraph_t graph = nullptr;
+        CK(cudaStreamBeginCapture(c->st, cudaStreamCaptureModeThreadLocal));
+        const pbd_status s = enqueue_steps(c, pd, c->nsplit_max);
+        cudaError_t e = cudaStreamEndCapture(c->st, &graph);
+        if (s == PBD_OK && e == cudaSuccess) e = cudaGraphInstantiate(&g.gx, graph, 0);
+        if (graph) cudaGraphDestroy(graph);
+        TRY(s);
+        CK(e);
+    }
+    CK(cudaGraphLaunch(g.gx, c->st));
+    return PBD_OK;
+}
+
 pbd_status run_pass(pbd_ctx *c, const PassDesc &pd, int kind, int *ids_out, float *logits) {
-    if (!c->sched[kind].valid) return fail(c, PBD_ERR_STATE, "no schedule for pass kind %d", kind);
-    TRY(enqueue_pass_kernel(c, pd, kind));
+    TRY(enqueue_layers(c, pd, kind));
     return enqueue_head(c, pd.nb * pd.ro_count, ids_out, logits);
 }
 
@@ -708,7 +812,9 @@ pbd_status enqueue_short_prompt(pbd_ctx *c, int P, const int32_t *d_ids) {
     pd.att_span = att_span_of(c);
     const RowSeg seg{0, 0, 0, P};
     const int ro = 0;
-    TRY(upload_schedule(c, PK_PREFILL, pd, std::vector<int>(1, (P + ATT_SPLIT - 1) / ATT_SPLIT)));
+    c->steps[PK_PREFILL] = c->cfg.max_ctas == 0 && step_pass_fits(c->dm, pd, att_subs_of(c), (P + ATT_SPLIT - 1) / ATT_SPLIT);
+    if (!c->steps[PK_PREFILL])
+        TRY(upload_schedule(c, PK_PREFILL, pd, std::vector<int>(1, (P + ATT_SPLIT - 1) / ATT_SPLIT)));
     CK(cudaMemcpyAsync(c->rows.segs, &seg, sizeof seg, cudaMemcpyHostToDevice, c->st));
     CK(cudaMemcpyAsync(c->rows.ro, &ro, sizeof ro, cudaMemcpyHostToDevice, c->st));
     CK(launch_set_len(c->s.L, 0, 0, c->st));
@@ -728,16 +834,6 @@ pbd_status check_device(pbd_ctx *c) {
         return fail(c, PBD_ERR_DEVICE, "device status %d latched by a kernel", code);
     }
     return PBD_OK;
-}
-
-// attention split items per sequence over the whole generation (positions up to P + max_new + 2(D+1))
-std::vector<int> decode_splits(pbd_ctx *c) {
-    std::vector<int> ns(c->batch);
-    for (int b = 0; b < c->batch; ++b) {
-        const int tmax = std::min(c->prompt_lens[b] + c->max_new + 2 * (c->D + 1), c->pages_per_seq * PAGE);
-        ns[b] = std::min(c->n_splits, (tmax + ATT_SPLIT - 1) / ATT_SPLIT);
-    }
-    return ns;
 }
 
 double pass_bytes(pbd_ctx *c, int kind, const std::vector<int> &Ls) {
@@ -923,11 +1019,16 @@ pbd_status pbd_prefill(pbd_ctx *c, int32_t batch, const int32_t *d_prompt_ids, c
     if (d_first_token)
         CK(cudaMemcpyAsync(d_first_token, c->s.pending, sizeof(int) * batch, cudaMemcpyDeviceToDevice, c->st));
     TRY(check_device(c));
-    // schedules of the decode passes of this generation
+    // the decode passes of this generation: kernel chains where they fit, else schedules of the persistent
+    // kernel (which max_ctas limits to fewer CTAs than SMs)
     const std::vector<int> ns = decode_splits(c);
-    TRY(upload_schedule(c, PK_DRAFT, block_pass(c, PK_DRAFT), ns));
-    TRY(upload_schedule(c, PK_VERIFY, block_pass(c, PK_VERIFY), ns));
-    TRY(upload_schedule(c, PK_DECODE, block_pass(c, PK_DECODE), ns));
+    c->nsplit_max = *std::max_element(ns.begin(), ns.end());
+    for (int kind = PK_DRAFT; kind <= PK_DECODE; ++kind) {
+        const PassDesc pd = block_pass(c, kind);
+        c->sched[kind].valid = false;
+        c->steps[kind] = c->cfg.max_ctas == 0 && step_pass_fits(c->dm, pd, att_subs_of(c), c->nsplit_max);
+        if (!c->steps[kind]) TRY(upload_schedule(c, kind, pd, ns));
+    }
     c->phase = PH_READY;
     return PBD_OK;
 }
@@ -1186,15 +1287,17 @@ pbd_status pbd_time_pass(pbd_ctx *c, int32_t kind, int32_t iters, double *h_ms_p
     const PassDesc pd = block_pass(c, kind);
     CK(launch_build_ids(pd, kind == PK_DRAFT ? 0 : (kind == PK_VERIFY ? 1 : 2), c->s.pending, c->draft_ids, c->D,
                         c->ids, c->st));
-    TRY(enqueue_pass_kernel(c, pd, kind));  // warm-up launch
+    for (int i = 0; i < 2; ++i) TRY(enqueue_layers(c, pd, kind));  // warm-up
     std::vector<cudaEvent_t> ev((size_t)iters * 2, nullptr);
     pbd_status s = PBD_OK;
     for (auto &x : ev)
         if (s == PBD_OK && cudaEventCreate(&x) != cudaSuccess) s = fail(c, PBD_ERR_CUDA, "event create");
     for (int i = 0; s == PBD_OK && i < iters; ++i) {
-        cudaError_t e = cudaMemsetAsync(c->cnt, 0, sizeof(int) * (size_t)(c->cl.total + 1), c->st);
+        cudaError_t e = cudaSuccess;
+        if (!c->steps[kind]) e = cudaMemsetAsync(c->cnt, 0, sizeof(int) * (size_t)(c->cl.total + 1), c->st);
         if (e == cudaSuccess) e = cudaEventRecord(ev[2 * i], c->st);
-        if (e == cudaSuccess) e = launch_pass_kernel(make_launch(c, pd, kind), c->st);
+        if (e == cudaSuccess && !c->steps[kind]) e = launch_pass_kernel(make_launch(c, pd, kind), c->st);
+        if (c->steps[kind]) s = enqueue_layers(c, pd, kind);
         if (e == cudaSuccess) e = cudaEventRecord(ev[2 * i + 1], c->st);
         if (e != cudaSuccess) s = fail(c, PBD_ERR_CUDA, "timed launch: %s", cudaGetErrorString(e));
     }
@@ -1242,6 +1345,7 @@ pbd_status pbd_check_stalled_pass(pbd_ctx *c, int32_t *h_device_code) {
     std::vector<int> fill(cta_off.begin(), cta_off.end() - 1);
     for (size_t i = 0; i < items.size(); ++i) dealt[fill[i % c->grid]++] = items[i];
     Sched &sv = c->sched[PK_VERIFY];
+    TRY(ensure_schedule(c, PK_VERIFY, pd));  // (its split counts)
     CK(cudaMemcpyAsync(sv.items, dealt.data(), dealt.size() * sizeof(MKItem), cudaMemcpyHostToDevice, c->st));
     CK(cudaMemcpyAsync(sv.off, cta_off.data(), cta_off.size() * sizeof(int), cudaMemcpyHostToDevice, c->st));
     CK(cudaStreamSynchronize(c->st));
@@ -1251,8 +1355,10 @@ pbd_status pbd_check_stalled_pass(pbd_ctx *c, int32_t *h_device_code) {
     int code = 0;
     CK(cudaMemcpy(&code, c->status, sizeof(int), cudaMemcpyDeviceToHost));
     *h_device_code = code;
-    // the normal verify schedule again; the device code is reported (and cleared) below
-    TRY(upload_schedule(c, PK_VERIFY, pd, ns));
+    // the normal verify schedule again, where verify passes use it; the device code is reported (and cleared)
+    // below
+    c->sched[PK_VERIFY].valid = false;
+    if (!c->steps[PK_VERIFY]) TRY(upload_schedule(c, PK_VERIFY, pd, ns));
     return check_device(c);
 }
 
@@ -1265,6 +1371,7 @@ pbd_status pbd_trace_pass(pbd_ctx *c, int32_t kind, int32_t *h_items, uint64_t *
     std::vector<int> off;
     mk_build_schedule(c->dm, pd, decode_splits(c), c->grid, c->cl, &items, &off);
     if ((int)items.size() > cap) return fail(c, PBD_ERR_CAPACITY, "%zu items exceed cap %d", items.size(), cap);
+    TRY(ensure_schedule(c, kind, pd));
     CK(launch_build_ids(pd, kind == PK_DRAFT ? 0 : (kind == PK_VERIFY ? 1 : 2), c->s.pending, c->draft_ids, c->D,
                         c->ids, c->st));
     CK(cudaMemsetAsync(c->trace, 0, sizeof(unsigned long long) * MK_STAMPS * items.size(), c->st));

@@ -143,6 +143,45 @@ size_t mk_union_bytes(int bn, int head_dim, int att_span);
 int mk_slice_atoms(int lin, int K);  // 64-wide K atoms per work item of linear `lin`
 cudaError_t launch_pass_kernel(const MKLaunch &L, cudaStream_t st);
 
+// ---- decoding passes as a chain of small kernels (steps.cu) ----
+
+struct StepArgs {
+    Dims dm;
+    PassDesc pd;
+    const int *L, *ids;
+    KVCache kv;
+    bf16 *h, *q, *attn, *act;  // [rows_alloc][H], [][Hq d], [][Hq d], [][I]
+    float *ss;                 // [rows_alloc][H / 128] sums of squares of h
+    int rows_alloc;
+    const float2 *rope_cs;
+    int rope_rows;
+    int att_subs;              // partial results per 128-key split
+    float att_scale;
+    float *o_part;             // partial results in memory: [row][head][att_splits_alloc][d],
+    float2 *ml_part;           // [row][head][att_splits_alloc]
+    int att_splits_alloc;
+    int *status;
+    int bn;                    // (set by the launcher) token columns of the MMAs
+};
+struct StepLin {
+    const uint8_t *tiles;      // this layer's weight, pre-tiled, the adapter's rows in the last tile
+    const bf16 *gain, *q_norm, *k_norm, *lora_b;  // this layer's
+    int layer, K, n_main;
+    // set by the launcher
+    CUtensorMap xmap;
+    int k_tiles, katoms, ks, ring_atoms;
+    uint32_t tmem_cols;
+};
+// whether every step of the pass fits a cluster and its shared memory (nsplit: 128-key splits of the
+// longest sequence)
+bool step_pass_fits(const Dims &dm, const PassDesc &pd, int subs, int nsplit);
+cudaError_t launch_step_embed(const StepArgs &a, const void *embed_tiled, const void *mask_embed, cudaStream_t st);
+cudaError_t launch_step_linear(int lin, StepArgs &a, StepLin &w, cudaStream_t st);
+cudaError_t launch_step_attn(const StepArgs &a, const CUtensorMap &kmap, const CUtensorMap &vmap, int layer, int nsplit,
+                             cudaStream_t st);
+cudaError_t launch_step_final(const StepArgs &a, const void *gain, void *x_ro, cudaStream_t st);
+cudaError_t configure_step_kernels();
+
 // ---- passes over many rows: prompt processing (rows.cu, gemm.cu) ----
 
 // Rows row0 .. row0 + n - 1 of a pass hold positions pos0 .. pos0 + n - 1 of sequence seq.
