@@ -105,10 +105,11 @@ struct pbd_ctx {
     // the chain of each kind as a graph, built on a kind's second call of a generation plan
     void *step_act;  // SiLU(gate) * up rows, bf16
     bool steps[N_PK] = {false, false, false, false};
-    int nsplit_max = 0;
+    std::vector<int> nsplit;  // 128-key splits per sequence
     struct StepGraph {
         cudaGraphExec_t gx = nullptr;
-        int batch = 0, nsplit = 0, calls = 0;
+        std::vector<int> nsplit;
+        int calls = 0;
     } step_graph[N_PK];
     SeqState s;
     CUtensorMap maps[16];    // x_ro, box height 16 (i + 1)
@@ -577,9 +578,11 @@ pbd_status ensure_schedule(pbd_ctx *c, int kind, const PassDesc &pd) {
     return c->sched[kind].valid ? PBD_OK : upload_schedule(c, kind, pd, decode_splits(c));
 }
 
-// All decoder layers of a pass as a chain of kernels.
-pbd_status enqueue_steps(pbd_ctx *c, const PassDesc &pd, int nsplit) {
+// All decoder layers of a pass as a chain of kernels; nsplit: 128-key splits per sequence.
+pbd_status enqueue_steps(pbd_ctx *c, const PassDesc &pd, const std::vector<int> &nsplit) {
     const pbd_config &k = c->cfg;
+    StepSplits sp{};
+    for (int b = 0; b < pd.nb; ++b) sp.start[b + 1] = sp.start[b] + nsplit[b];
     StepArgs a{};
     a.dm = c->dm;
     a.pd = pd;
@@ -614,7 +617,7 @@ pbd_status enqueue_steps(pbd_ctx *c, const PassDesc &pd, int nsplit) {
             w.k_norm = static_cast<const bf16 *>(c->k_norm) + (size_t)l * k.head_dim;
             w.lora_b = static_cast<const bf16 *>(c->lb[lin]) + (size_t)l * w.n_main * k.lora_rank;
             CK(launch_step_linear(lin, a, w, c->st));
-            if (lin == 0) CK(launch_step_attn(a, c->kmap, c->vmap, l, nsplit, c->st));
+            if (lin == 0) CK(launch_step_attn(a, c->kmap, c->vmap, l, sp, c->st));
         }
     }
     if (pd.ro_count > 0) CK(launch_step_final(a, c->final_norm, c->x_ro, c->st));
@@ -628,23 +631,22 @@ pbd_status enqueue_layers(pbd_ctx *c, const PassDesc &pd, int kind) {
         if (!c->sched[kind].valid) return fail(c, PBD_ERR_STATE, "no schedule for pass kind %d", kind);
         return enqueue_pass_kernel(c, pd, kind);
     }
-    if (kind == PK_PREFILL) return enqueue_steps(c, pd, (pd.R + ATT_SPLIT - 1) / ATT_SPLIT);
+    if (kind == PK_PREFILL) return enqueue_steps(c, pd, std::vector<int>(1, (pd.R + ATT_SPLIT - 1) / ATT_SPLIT));
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     const bool legacy = c->st == nullptr || c->st == cudaStreamLegacy;
     if (!legacy) CK(cudaStreamIsCapturing(c->st, &cap));
     pbd_ctx::StepGraph &g = c->step_graph[kind];
-    if (legacy || cap != cudaStreamCaptureStatusNone) return enqueue_steps(c, pd, c->nsplit_max);
-    if (g.batch != c->batch || g.nsplit != c->nsplit_max) {
+    if (legacy || cap != cudaStreamCaptureStatusNone) return enqueue_steps(c, pd, c->nsplit);
+    if (g.nsplit != c->nsplit) {
         if (g.gx) cudaGraphExecDestroy(g.gx);
         g = pbd_ctx::StepGraph();
-        g.batch = c->batch;
-        g.nsplit = c->nsplit_max;
+        g.nsplit = c->nsplit;
     }
     if (!g.gx) {
-        if (g.calls++ == 0) return enqueue_steps(c, pd, c->nsplit_max);
+        if (g.calls++ == 0) return enqueue_steps(c, pd, c->nsplit);
         cudaGraph_t graph = nullptr;
         CK(cudaStreamBeginCapture(c->st, cudaStreamCaptureModeThreadLocal));
-        const pbd_status s = enqueue_steps(c, pd, c->nsplit_max);
+        const pbd_status s = enqueue_steps(c, pd, c->nsplit);
         cudaError_t e = cudaStreamEndCapture(c->st, &graph);
         if (s == PBD_OK && e == cudaSuccess) e = cudaGraphInstantiate(&g.gx, graph, 0);
         if (graph) cudaGraphDestroy(graph);
@@ -1022,11 +1024,12 @@ pbd_status pbd_prefill(pbd_ctx *c, int32_t batch, const int32_t *d_prompt_ids, c
     // the decode passes of this generation: kernel chains where they fit, else schedules of the persistent
     // kernel (which max_ctas limits to fewer CTAs than SMs)
     const std::vector<int> ns = decode_splits(c);
-    c->nsplit_max = *std::max_element(ns.begin(), ns.end());
+    c->nsplit = ns;
+    const int longest = *std::max_element(ns.begin(), ns.end());
     for (int kind = PK_DRAFT; kind <= PK_DECODE; ++kind) {
         const PassDesc pd = block_pass(c, kind);
         c->sched[kind].valid = false;
-        c->steps[kind] = c->cfg.max_ctas == 0 && step_pass_fits(c->dm, pd, att_subs_of(c), c->nsplit_max);
+        c->steps[kind] = c->cfg.max_ctas == 0 && step_pass_fits(c->dm, pd, att_subs_of(c), longest);
         if (!c->steps[kind]) TRY(upload_schedule(c, kind, pd, ns));
     }
     c->phase = PH_READY;

@@ -169,16 +169,20 @@ struct StepLin {
     int layer, K, n_main;
     // set by the launcher
     CUtensorMap xmap;
-    int k_tiles, katoms, ks, ring_atoms;
+    int k_tiles, katoms, ks, ring_atoms, push;
     uint32_t tmem_cols;
+};
+// 128-key splits of a pass's sequences end to end: sequence b has start[b] .. start[b + 1) (max_batch <= 64)
+struct StepSplits {
+    int start[65];
 };
 // whether every step of the pass fits a cluster and its shared memory (nsplit: 128-key splits of the
 // longest sequence)
 bool step_pass_fits(const Dims &dm, const PassDesc &pd, int subs, int nsplit);
 cudaError_t launch_step_embed(const StepArgs &a, const void *embed_tiled, const void *mask_embed, cudaStream_t st);
 cudaError_t launch_step_linear(int lin, StepArgs &a, StepLin &w, cudaStream_t st);
-cudaError_t launch_step_attn(const StepArgs &a, const CUtensorMap &kmap, const CUtensorMap &vmap, int layer, int nsplit,
-                             cudaStream_t st);
+cudaError_t launch_step_attn(const StepArgs &a, const CUtensorMap &kmap, const CUtensorMap &vmap, int layer,
+                             const StepSplits &sp, cudaStream_t st);
 cudaError_t launch_step_final(const StepArgs &a, const void *gain, void *x_ro, cudaStream_t st);
 cudaError_t configure_step_kernels();
 

@@ -3,11 +3,10 @@
 // A layer is five kernels: q|k|v (+ QK-norm, RoPE, K/V write), attention, o (+ residual), gate|up (+ SiLU),
 // down (+ residual).  Each is one step of the chain, bound by latency and not by its few megabytes of
 // weights, so the design removes what the chain waits for:
-//   - A linear's K slices (256 wide, gate|up 512) are one thread-block cluster per 128-feature tile.  The
-//     slices' fp32 partial sums stay in shared memory; after a cluster barrier CTA s finishes rows s,
-//     s + slices, ... reading its peers through distributed shared memory.  The attention's key
-//     splits of a (sequence, KV head) are a cluster too, and merge the same way.  No partial sum or
-//     completion counter goes through global memory.
+//   - A linear's K slices (256 wide, gate|up 512) are one thread-block cluster per 128-feature tile.  A
+//     row's fp32 partial sums go through distributed shared memory to the CTA that finishes the row (many
+//     rows: it fetches them).  The attention's key splits of a (sequence, KV head) are a cluster too, as
+//     long as there are few of them, and merge the same way.
 //   - The kernels launch dependent: a CTA sets itself up and requests its weights (or the cached K/V
 //     pages) while the step before it still runs, and waits only for its activations.
 //
@@ -16,9 +15,9 @@
 // CTAs than SMs and for shapes whose slices or partial results do not fit a cluster; rows.cu computes the
 // same for prompts.
 //
-// 0.6B shape, all layers of one pass (the persistent kernel in brackets), us: verify 896 (1136), draft 1159
-// (1287), one-row decoding 720 (945) at 512 tokens of context; 1057 (1430), 1281 (1579), 893 (1196) at 4096;
-// 1823 (3637), 2424 (4080), 1025 (1778) for eight sequences of 420 to 1757 tokens.
+// 0.6B shape, all layers of one pass (the persistent kernel in brackets), us: verify 769 (1136), draft 963
+// (1287), one-row decoding 632 (945) at 512 tokens of context; 899 (1430), 1102 (1579), 750 (1196) at 4096;
+// 1619 (3637), 2059 (4080), 865 (1778) for eight sequences of 420 to 1757 tokens.
 #include <algorithm>
 #include <cmath>
 
@@ -28,8 +27,6 @@
 
 namespace pbd {
 
-constexpr int ST_THREADS = 256;
-constexpr int ST_STAGERS = 192;    // threads that stage a normalised operand (warps 2-7)
 constexpr int ST_HALF = 4;         // 64-wide K atoms per half (256 of K)
 constexpr int ST_RANK = 16;        // adapter rank (8 or 16)
 constexpr int ST_A_BYTES = 2 * ST_RANK * 128;  // adapter rows of one K atom (gate and up: two ranks)
@@ -57,10 +54,37 @@ __device__ __forceinline__ float ld_cluster(uint32_t a) {
     asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
     return v;
 }
-__device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+__device__ __forceinline__ float4 ld_shared_v4(uint32_t a) {
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");
+    return v;
 }
-__device__ __forceinline__ void bar_stagers() { asm volatile("bar.sync 1, 192;" ::: "memory"); }
+__device__ __forceinline__ float2 ld_shared_v2(uint32_t a) {
+    float2 v;
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ float ld_shared(uint32_t a) {
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_cluster(uint32_t a, float v) {
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+}
+__device__ __forceinline__ void st_cluster_v2(uint32_t a, float x, float y) {
+    asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(x), "f"(y) : "memory");
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_sync() {
+    cluster_arrive();
+    cluster_wait();
+}
+template <int N>
+__device__ __forceinline__ void bar_stagers() {
+    asm volatile("bar.sync 1, %0;" ::"n"(N) : "memory");
+}
 
 __device__ __forceinline__ float4 add4(float4 a, float4 b) {
     return make_float4(__fadd_rn(a.x, b.x), __fadd_rn(a.y, b.y), __fadd_rn(a.z, b.z), __fadd_rn(a.w, b.w));
@@ -73,63 +97,96 @@ struct StepLinState {
     uint32_t tmem_slot;
     int abort;
     float rs[256];  // 1/rms of each row (normalised operands)
-    // the adapter's B rows of the tile: row j at chunk j * (r / 8) + j / 4 (16 bytes of padding after
-    // every four rows: a reducing lane reads rows 4l..4l+3)
-    uint4 brows[TILE_ROWS * ST_RANK / 8 + TILE_ROWS / 4];
+    // the adapter's B rows of the tile, transposed and widened: [rank][128] (a reducing lane reads four features
+    // of one rank column at a time)
+    float4 bt[ST_RANK * TILE_ROWS / 4];
 };
 
-// sum over the slices of four features (float4) or of one adapter row, in slice order
-__device__ __forceinline__ float4 sum_slices4(uint32_t a, int ks) {
-    float4 y = ld_cluster_v4(map_cta(a, 0));
-    for (int s0 = 1; s0 < ks; s0 += 4) {
+// Sum over the slices, in slice order, of four features of a row or of one adapter row.  PUSH: the slices lie
+// `stride` bytes apart in this CTA; otherwise slice s at the same address of CTA s.
+__device__ __forceinline__ float4 slice4(uint32_t a, int s, uint32_t stride, bool push) {
+    return push ? ld_shared_v4(a + (uint32_t)s * stride) : ld_cluster_v4(map_cta(a, s));
+}
+__device__ __forceinline__ float4 sum_slices4(uint32_t a, int ks, uint32_t stride, bool push) {
+    float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int s0 = 0; s0 < ks; s0 += 4) {
         float4 v[4];
 #pragma unroll
-        for (int s = 0; s < 4; ++s) v[s] = ld_cluster_v4(map_cta(a, min(s0 + s, ks - 1)));
+        for (int s = 0; s < 4; ++s) v[s] = slice4(a, min(s0 + s, ks - 1), stride, push);
 #pragma unroll
         for (int s = 0; s < 4; ++s)
-            if (s0 + s < ks) y = add4(y, v[s]);
+            if (s0 + s < ks) y = s0 + s == 0 ? v[s] : add4(y, v[s]);
     }
     return y;
 }
-__device__ __forceinline__ float sum_slices(uint32_t a, int ks) {
-    float y = ld_cluster(map_cta(a, 0));
-    for (int s0 = 1; s0 < ks; s0 += 4) {
+__device__ __forceinline__ float sum_slices(uint32_t a, int ks, uint32_t stride, bool push) {
+    float y = 0.f;
+    for (int s0 = 0; s0 < ks; s0 += 4) {
         float v[4];
 #pragma unroll
-        for (int s = 0; s < 4; ++s) v[s] = ld_cluster(map_cta(a, min(s0 + s, ks - 1)));
+        for (int s = 0; s < 4; ++s) {
+            const int t = min(s0 + s, ks - 1);
+            v[s] = push ? ld_shared(a + (uint32_t)t * stride) : ld_cluster(map_cta(a, t));
+        }
 #pragma unroll
         for (int s = 0; s < 4; ++s)
-            if (s0 + s < ks) y = __fadd_rn(y, v[s]);
+            if (s0 + s < ks) y = s0 + s == 0 ? v[s] : __fadd_rn(y, v[s]);
     }
     return y;
 }
 
-// the adapter intermediates u_0 .. u_{r-1} of one row, from lanes base, base + 1, ...
-__device__ __forceinline__ void spread_u(float lane_u, int base, float (&u)[ST_RANK]) {
-#pragma unroll
-    for (int j = 0; j < ST_RANK; ++j) u[j] = __shfl_sync(0xffffffffu, lane_u, base + j);
+// y_f += scale * (u . B_f) for two features f, the products added in rank order: packed fp32 multiplies and
+// adds, each half rounded as __fmul_rn and __fadd_rn round
+struct F2 {
+    unsigned long long v;
+};
+__device__ __forceinline__ F2 f2(float x, float y) {
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(x), "f"(y));
+    return r;
 }
-// u . B[j] over the rank, in order
-__device__ __forceinline__ float lora_dot_s(const float (&u)[ST_RANK], const uint4 *brows, int j, int r) {
-    float a = 0.f;
-    const uint4 *b = brows + j * (r / 8) + (j >> 2);
+__device__ __forceinline__ F2 mul2(F2 a, F2 b) {
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 add2(F2 a, F2 b) {
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(F2 a) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a.v));
+    return r;
+}
+// lane_ua / lane_ub: lane i holds u_i for the first / second pair of features (at fa, fb in the tile)
+__device__ __forceinline__ void add_delta(float (&y)[4], float lane_ua, float lane_ub, int base_b, const float *bt, int fa, int fb,
+                                          int r, float scale) {
+    F2 a = f2(0.f, 0.f), b = a;
 #pragma unroll
-    for (int q = 0; q < ST_RANK / 8; ++q) {
-        if (q * 8 >= r) break;
-        const uint4 w = b[q];
-        const bf16 *e = reinterpret_cast<const bf16 *>(&w);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) a = __fadd_rn(a, __fmul_rn(u[q * 8 + i], bf2f(e[i])));
+    for (int i = 0; i < ST_RANK; ++i) {
+        if (i >= r) break;
+        const float ua = __shfl_sync(0xffffffffu, lane_ua, i), ub = __shfl_sync(0xffffffffu, lane_ub, base_b + i);
+        const float2 ba = *reinterpret_cast<const float2 *>(bt + i * TILE_ROWS + fa);
+        const float2 bb = *reinterpret_cast<const float2 *>(bt + i * TILE_ROWS + fb);
+        a = add2(a, mul2(f2(ua, ua), f2(ba.x, ba.y)));
+        b = add2(b, mul2(f2(ub, ub), f2(bb.x, bb.y)));
     }
-    return a;
+    const F2 s2 = f2(scale, scale);
+    const float2 ya = unpack2(add2(f2(y[0], y[1]), mul2(s2, a))), yb = unpack2(add2(f2(y[2], y[3]), mul2(s2, b)));
+    y[0] = ya.x, y[1] = ya.y, y[2] = yb.x, y[3] = yb.y;
 }
 
 // LIN: 0 q|k|v, 1 o, 2 gate|up, 3 down.  Grid (tiles, slices), cluster (1, slices).
-// Dynamic shared memory: W atoms | adapter atoms (AD) | x atoms; then the partial sums in their place.
-template <int LIN, bool AD, int DH>
-__global__ void __launch_bounds__(ST_THREADS, 1)
+// NT threads: warp 0 streams, warp 1 issues the MMAs, warps 2.. stage a normalised operand, warps 4-7 read the
+// accumulator, all finish rows.  Dynamic shared memory: W atoms | adapter atoms (AD) | x atoms | partial sums
+// (or those in the operands' place).
+template <int LIN, bool AD, int DH, int NT>
+__global__ void __maxnreg__(NT == 256 ? 104 : 128)
     k_step_linear(const __grid_constant__ StepArgs a, const __grid_constant__ StepLin w) {
     constexpr bool NORM = LIN == 0 || LIN == 2;  // the operand is RMSNorm(h)
+    constexpr int STAGERS = NT - 64;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     __shared__ StepLinState S;
@@ -160,6 +217,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = S.tmem_slot;
+    cluster_arrive();  // (this CTA's shared memory exists: its peers wait for that before they write there)
     pdl_launch();  // (after the allocation: a later kernel's CTA never holds TMEM that this one waits for)
 
     if (warp == 0 && elect_one()) {
@@ -233,10 +291,14 @@ __global__ void __launch_bounds__(ST_THREADS, 1)
                 gv[hf] = __ldg(reinterpret_cast<const uint4 *>(w.gain + (size_t)(slice * w.katoms + hf * ST_HALF) * KT) + c);
         if (AD) {
             const int cpr = r / 8;
-            for (int q = ct; q < TILE_ROWS * cpr; q += ST_STAGERS) {
-                const int j = q / cpr, e = q % cpr;
+            float *bt = reinterpret_cast<float *>(S.bt);
+            for (int q = ct; q < TILE_ROWS * cpr; q += STAGERS) {
+                const int j = q % TILE_ROWS, e = q / TILE_ROWS;
                 const int f = LIN == 2 ? (j < 64 ? tile * 64 + j : dm.I + tile * 64 + (j - 64)) : ft + j;
-                S.brows[j * cpr + (j >> 2) + e] = __ldg(reinterpret_cast<const uint4 *>(w.lora_b + (size_t)f * r) + e);
+                const uint4 v = __ldg(reinterpret_cast<const uint4 *>(w.lora_b + (size_t)f * r) + e);
+                const bf16 *x = reinterpret_cast<const bf16 *>(&v);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) bt[(e * 8 + i) * TILE_ROWS + j] = bf2f(x[i]);
             }
         }
         pdl_wait();
@@ -245,18 +307,26 @@ __global__ void __launch_bounds__(ST_THREADS, 1)
             // (as build_b in pass_kernel.cu)
             uint8_t *col = sX + (size_t)(c >> 3) * x_atom;
             auto chunk = [&](int at, int m) { return col + at * x_atom + m * 128 + (((c & 7) ^ (m & 7)) << 4); };
+            const bool both = halves == 2 && ra > ST_HALF;  // room for both halves at once
+            auto copy = [&](int hf) {
+                const bf16 *src = a.h + (size_t)(slice * w.katoms + hf * ST_HALF) * KT + c * 8;
+#pragma unroll 1
+                for (int m = ct >> 5; m < M; m += STAGERS / 32) cp_async16(chunk((hf * ST_HALF) % ra, m), src + (size_t)m * dm.H);
+                cp_async_commit();
+            };
+            copy(0);
+            if (both) copy(1);
             bool ok = true;
             for (int hf = 0; hf < halves; ++hf) {
                 const int at = (hf * ST_HALF) % ra;
-                if (hf == 1 && ra == ST_HALF && !mbar_wait(&S.hdone, 0, a.status, DEV_TIMEOUT_MMA, &S.abort)) ok = false;
-                if (!ok) break;
-                const bf16 *src = a.h + (size_t)(slice * w.katoms + hf * ST_HALF) * KT + c * 8;
-#pragma unroll 1
-                for (int m = ct >> 5; m < M; m += ST_STAGERS / 32) cp_async16(chunk(at, m), src + (size_t)m * dm.H);
-                cp_async_commit();
+                if (hf == 1 && !both) {
+                    if (!mbar_wait(&S.hdone, 0, a.status, DEV_TIMEOUT_MMA, &S.abort)) ok = false;
+                    if (!ok) break;
+                    copy(1);
+                }
                 if (hf == 0) {
                     const int nt = dm.H / TILE_ROWS;
-                    for (int m = ct; m < M; m += ST_STAGERS) {
+                    for (int m = ct; m < M; m += STAGERS) {
                         const float2 *s = reinterpret_cast<const float2 *>(a.ss + (size_t)m * nt);
                         float sum = 0.f;
                         for (int t0 = 0; t0 < nt; t0 += 8) {
@@ -273,11 +343,14 @@ __global__ void __launch_bounds__(ST_THREADS, 1)
                         S.rs[m] = __fdiv_rn(1.0f, __fsqrt_rn(__fadd_rn(__fdiv_rn(sum, (float)dm.H), dm.eps)));
                     }
                 }
-                cp_async_wait_all();
-                if (hf == 0) bar_stagers();
+                if (hf == 0 && both)
+                    cp_async_wait_1();
+                else
+                    cp_async_wait_all();
+                if (hf == 0) bar_stagers<STAGERS>();
                 const __nv_bfloat162 *g2 = reinterpret_cast<const __nv_bfloat162 *>(&gv[hf]);
 #pragma unroll 1
-                for (int m = ct >> 5; m < M; m += ST_STAGERS / 32) {
+                for (int m = ct >> 5; m < M; m += STAGERS / 32) {
                     uint4 *p = reinterpret_cast<uint4 *>(chunk(at, m));
                     uint4 val = *p;
                     __nv_bfloat162 *v2 = reinterpret_cast<__nv_bfloat162 *>(&val);
@@ -290,44 +363,86 @@ __global__ void __launch_bounds__(ST_THREADS, 1)
                     *p = val;
                 }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                bar_stagers();
+                bar_stagers<STAGERS>();
                 if (ct == 0) mbarrier_arrive_one(&S.xfull[hf]);
             }
         }
     }
     __syncwarp();
 
-    // ---- partial sums into shared memory (every MMA has read its operands): warps 4-7, one TMEM lane quarter
-    // (32 features) each
-    float *part = reinterpret_cast<float *>(base), *part_u = part + M * TILE_ROWS;
-    if (warp >= 4) {
+    // what the warp's first row needs besides its sums, on its way early
+    const int m_first = slice + warp * w.ks;
+    int pos1 = 0, page1 = 0;
+    float4 rope1[2] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
+    uint2 h1 = make_uint2(0, 0);
+    auto row_pos = [&](int m) { return a.L[a.pd.b0 + m / a.pd.R] + m % a.pd.R; };
+    auto row_page = [&](int m, int pos) {
+        return pos / PAGE < a.kv.pages_per_seq ? a.kv.page_table[(a.pd.b0 + m / a.pd.R) * a.kv.pages_per_seq + pos / PAGE] : -1;
+    };
+    auto row_rope = [&](int pos, float4 (&c)[2]) {
+        const float4 *p = reinterpret_cast<const float4 *>(a.rope_cs + (size_t)(pos < a.rope_rows ? pos : 0) * (DH / 2) +
+                                                           (4 * (lane % (DH / 4))) % (DH / 2));
+        c[0] = __ldg(p);
+        c[1] = __ldg(p + 1);
+    };
+    if (warp < 2) pdl_wait();  // (the warps that have not yet)
+    if (m_first < M) {
+        if (LIN == 0) {
+            pos1 = row_pos(m_first);
+            if (kind > 0) page1 = row_page(m_first, pos1);
+            if (kind < 2) row_rope(pos1, rope1);
+        } else if (LIN != 2) {
+            h1 = __ldcg(reinterpret_cast<const uint2 *>(a.h + (size_t)m_first * dm.H + ft) + lane);
+        }
+    }
+
+    // ---- partial sums: warps 4-7 (and 8-11), a TMEM lane quarter (32 features) each.  PUSH: row m straight to CTA
+    // m % slices, which finishes it, as [slice][row / slices][features] behind its ring.  Otherwise (many
+    // rows) into the ring's place, every MMA having read its operands, for the peers to read.
+    const bool push = w.push != 0;
+    const int rpo = (M + w.ks - 1) / w.ks;  // rows per CTA
+    float *part = reinterpret_cast<float *>(push ? sX + ra * x_atom : base);
+    float *part_u = part + (push ? w.ks * rpo : M) * TILE_ROWS;
+    const uint32_t pa = smem_u32(part), pu = smem_u32(part_u);
+    cluster_wait();
+    constexpr int MOVERS = NT / 128 > 2 ? 2 : 1;  // warps per lane quarter
+    if ((warp >= 4 && warp < 4 + 4 * MOVERS) || (AD && warp == 0)) {
         const bool have = mbar_wait(&S.done, 0, a.status, DEV_TIMEOUT_MMA, &S.abort) && !*(volatile int *)&S.abort;
         tc_fence_after();
-        const int q = warp - 4, row = q * 32 + lane;
-        const uint32_t tq = tmem + ((uint32_t)(q * 32) << 16);
-        for (int c0 = 0; have && c0 < M; c0 += 16) {
+        // the features' warps take every MOVERS-th chunk of 16 columns (rows of the pass); warp 0 the adapter's
+        const bool ad = AD && warp == 0;
+        const int row = ad ? lane : (warp & 3) * 32 + lane, width = ad ? ru : TILE_ROWS, first = ad ? 0 : (warp - 4) >> 2;
+        const uint32_t col = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (ad ? (uint32_t)a.bn : 0u);
+        float *local = ad ? part_u : part;
+        const uint32_t remote = ad ? pu : pa;
+        const bool mine = !ad || lane < ru;
+#pragma unroll 1
+        for (int c0 = first * 16; have && c0 < M; c0 += ad ? 16 : 16 * MOVERS) {
             uint32_t v[16];
-            tmem_ld_16cols(tq + (uint32_t)c0, v);
+            tmem_ld_16cols(col + (uint32_t)c0, v);
             tmem_ld_wait();
+            if (push) {
+                int to = c0 % w.ks, at = slice * rpo + c0 / w.ks;  // destination CTA and row there
 #pragma unroll
-            for (int j = 0; j < 16; ++j)
-                if (c0 + j < M) part[(c0 + j) * TILE_ROWS + row] = __uint_as_float(v[j]);
-            if (AD && q == 0) {
-                tmem_ld_16cols(tq + (uint32_t)(a.bn + c0), v);
-                tmem_ld_wait();
+                for (int j = 0; j < 16; ++j) {
+                    if (c0 + j >= M) break;
+                    if (mine) st_cluster(map_cta(remote + (uint32_t)(at * width + row) * 4u, to), __uint_as_float(v[j]));
+                    if (++to == w.ks) to = 0, ++at;
+                }
+            } else {
 #pragma unroll
                 for (int j = 0; j < 16; ++j)
-                    if (c0 + j < M && lane < ru) part_u[(c0 + j) * ru + lane] = __uint_as_float(v[j]);
+                    if (c0 + j < M && mine) local[(c0 + j) * width + row] = __uint_as_float(v[j]);
             }
         }
         tc_fence_before();
     }
+    __syncwarp();
     cluster_sync();
     if (warp == 0) tmem_dealloc(tmem, w.tmem_cols);
-    if (warp < 2) pdl_wait();  // (the warps that have not yet; the stores below)
 
     // ---- rows slice, slice + slices, ...: one warp per row
-    const uint32_t pa = smem_u32(part), pu = smem_u32(part_u) + 4u * (lane < ru ? lane : 0);
+    const uint32_t st4 = (uint32_t)(rpo * TILE_ROWS) * 4u, stu = (uint32_t)(rpo * ru) * 4u;  // slice strides (PUSH)
     float gn[4] = {0.f, 0.f, 0.f, 0.f};  // QK-norm gain of the lane's four features
     constexpr int LPH = DH / 4;          // lanes per head
     const int e0 = 4 * (lane % LPH);
@@ -337,52 +452,51 @@ __global__ void __launch_bounds__(ST_THREADS, 1)
         const float2 y = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&raw.y));
         gn[0] = x.x, gn[1] = x.y, gn[2] = y.x, gn[3] = y.y;
     }
-    for (int m = slice + warp * w.ks; m < M; m += w.ks * (ST_THREADS / 32)) {
-        float u[ST_RANK], u2[ST_RANK];  // the row's adapter intermediates (gate|up: gate's and up's)
-        if (AD) {
-            const float lu = rbf(sum_slices(pu + (uint32_t)(m * ru) * 4u, w.ks));  // lane j: u_j
-            spread_u(lu, 0, u);
-            if (LIN == 2) spread_u(lu, r, u2);
-        }
+    for (int m = slice + warp * w.ks; m < M; m += w.ks * (NT / 32)) {
+        const int at = push ? m / w.ks : m;
+        float lu = 0.f;  // lane i: the row's adapter intermediate u_i (gate|up: gate's, then up's)
+        if (AD) lu = rbf(sum_slices(pu + (uint32_t)(at * ru + (lane < ru ? lane : 0)) * 4u, w.ks, stu, push));
+        const float *bt = reinterpret_cast<const float *>(S.bt);
         if constexpr (LIN == 2) {
             // gate rows 2l, 2l + 1 and up rows 64 + 2l, 64 + 2l + 1 -> act features 64 tile + 2l, + 2l + 1
             float g[2], up[2];
             {
                 float2 gs = make_float2(0.f, 0.f), us = gs;
-                const uint32_t ga = pa + (uint32_t)(m * TILE_ROWS + 2 * lane) * 4u;
+                const uint32_t ga = pa + (uint32_t)(at * TILE_ROWS + 2 * lane) * 4u;
                 for (int s = 0; s < w.ks; ++s) {
-                    const float2 x = ld_cluster_v2(map_cta(ga, s)), y = ld_cluster_v2(map_cta(ga + 256u, s));
+                    const uint32_t p = push ? ga + (uint32_t)s * st4 : map_cta(ga, s);
+                    const float2 x = push ? ld_shared_v2(p) : ld_cluster_v2(p), y = push ? ld_shared_v2(p + 256u) : ld_cluster_v2(p + 256u);
                     gs = s == 0 ? x : make_float2(__fadd_rn(gs.x, x.x), __fadd_rn(gs.y, x.y));
                     us = s == 0 ? y : make_float2(__fadd_rn(us.x, y.x), __fadd_rn(us.y, y.y));
                 }
                 g[0] = gs.x, g[1] = gs.y, up[0] = us.x, up[1] = us.y;
             }
+            if (AD) {
+                float y[4] = {g[0], g[1], up[0], up[1]};
+                add_delta(y, lu, lu, r, bt, 2 * lane, 64 + 2 * lane, r, dm.lora_scale);
+                g[0] = y[0], g[1] = y[1], up[0] = y[2], up[1] = y[3];
+            }
             float o[2];
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
-                if (AD) {
-                    g[e] = __fadd_rn(g[e], __fmul_rn(dm.lora_scale, lora_dot_s(u, S.brows, 2 * lane + e, r)));
-                    up[e] = __fadd_rn(up[e], __fmul_rn(dm.lora_scale, lora_dot_s(u2, S.brows, 64 + 2 * lane + e, r)));
-                }
                 const float gt = rbf(g[e]);
                 o[e] = __fmul_rn(__fdiv_rn(gt, __fadd_rn(1.0f, expf(-gt))), rbf(up[e]));
             }
             *reinterpret_cast<uint32_t *>(a.act + (size_t)m * dm.I + tile * 64 + 2 * lane) = pack_bf162(o[0], o[1]);
         } else {
-            uint2 hraw = make_uint2(0, 0);
+            uint2 hraw = h1;
             uint2 *hp = reinterpret_cast<uint2 *>(a.h + (size_t)m * dm.H + ft) + lane;
-            if (LIN == 1 || LIN == 3) hraw = __ldcg(hp);
-            const float4 y4 = sum_slices4(pa + (uint32_t)(m * TILE_ROWS + 4 * lane) * 4u, w.ks);
+            if ((LIN == 1 || LIN == 3) && m != m_first) hraw = __ldcg(hp);
+            const float4 y4 = sum_slices4(pa + (uint32_t)(at * TILE_ROWS + 4 * lane) * 4u, w.ks, st4, push);
             float y[4] = {y4.x, y4.y, y4.z, y4.w};
+            if (AD) add_delta(y, lu, lu, 0, bt, 4 * lane, 4 * lane + 2, r, dm.lora_scale);
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                if (AD) y[e] = __fadd_rn(y[e], __fmul_rn(dm.lora_scale, lora_dot_s(u, S.brows, 4 * lane + e, r)));
-                y[e] = rbf(y[e]);
-            }
+            for (int e = 0; e < 4; ++e) y[e] = rbf(y[e]);
             if constexpr (LIN == 0) {
-                const int b = a.pd.b0 + m / a.pd.R, pos = a.L[b] + m % a.pd.R, pg = pos / PAGE;
+                const int pos = m == m_first ? pos1 : row_pos(m);
+                const int page = kind == 0 ? 0 : (m == m_first ? page1 : row_page(m, pos));
                 const int head = (ft - (kind == 0 ? 0 : (kind == 1 ? qw : qw + kvw))) / DH + lane / LPH;
-                bool bad = kind > 0 && pg >= a.kv.pages_per_seq;
+                bool bad = page < 0;
                 if (kind < 2) {
                     bad = bad || pos >= a.rope_rows;
                     float ssq = __fmul_rn(y[0], y[0]);
@@ -391,8 +505,9 @@ __global__ void __launch_bounds__(ST_THREADS, 1)
 #pragma unroll
                     for (int off = LPH / 2; off >= 1; off >>= 1) ssq = __fadd_rn(ssq, __shfl_xor_sync(0xffffffffu, ssq, off));
                     const float rs = __fdiv_rn(1.0f, __fsqrt_rn(__fadd_rn(__fdiv_rn(ssq, (float)DH), dm.eps)));
-                    const float4 *c4 = reinterpret_cast<const float4 *>(a.rope_cs + (size_t)(bad ? 0 : pos) * (DH / 2) + (e0 % (DH / 2)));
-                    const float4 ca = __ldg(c4), cb = __ldg(c4 + 1);
+                    float4 rope[2] = {rope1[0], rope1[1]};
+                    if (m != m_first) row_rope(pos, rope);
+                    const float4 ca = rope[0], cb = rope[1];
                     const float cs[4] = {ca.x, ca.z, cb.x, cb.z}, sn[4] = {ca.y, ca.w, cb.y, cb.w};
 #pragma unroll
                     for (int j = 0; j < 4; ++j) y[j] = rbf(__fmul_rn(gn[j], rbf(__fmul_rn(y[j], rs))));
@@ -411,11 +526,9 @@ __global__ void __launch_bounds__(ST_THREADS, 1)
                     continue;
                 }
                 bf16 *dst = a.q + ((size_t)m * dm.Hq + head) * DH + e0;
-                if (kind > 0) {
-                    const int page = a.kv.page_table[b * a.kv.pages_per_seq + pg];
+                if (kind > 0)
                     dst = static_cast<bf16 *>(kind == 1 ? a.kv.k : a.kv.v) +
                           ((((size_t)w.layer * a.kv.n_pages + page) * dm.Hkv + head) * PAGE + (pos % PAGE)) * DH + e0;
-                }
                 *reinterpret_cast<uint2 *>(dst) = make_uint2(pack_bf162(y[0], y[1]), pack_bf162(y[2], y[3]));
             } else {
                 const __nv_bfloat162 *h2 = reinterpret_cast<const __nv_bfloat162 *>(&hraw);
@@ -432,29 +545,28 @@ __global__ void __launch_bounds__(ST_THREADS, 1)
             }
         }
     }
-    cluster_sync();  // no CTA leaves while another still reads its partials
+    if (!push) cluster_sync();  // no CTA leaves while another still reads its partials
 }
 
 // ------------------------------------------------------------------ attention step
 //
-// Grid (CTAs per group, KV heads, sequences).  CTA `rank` of a (sequence, KV head) takes splits rank,
-// rank + cs, ... of 128 keys, up to two staged at a time; units of one 16-row query tile against one split
-// (or 64-key half of it) go to the warps, as in attn_split (pass_kernel.cu).
+// Grid (splits, KV heads, sequences): a CTA takes one 128-key split of a (sequence, KV head); units of one
+// 16-row query tile against the split (or a 64-key half of it) go to the warps, as in attn_split
+// (pass_kernel.cu), and each leaves a partial result (m, l, O) per row.
 //
-// CLUSTER: the group's CTAs are a cluster.  The partial results (m, l, O) stay in shared memory, and
-// after the cluster barrier the CTAs merge rows rank, rank + cs, ... in key order.  Otherwise (more
-// splits than a portable cluster has CTAs, or more groups than the GPU holds clusters of: then clusters
-// wait for one another's SMs) every split is a CTA of its own, the partial results go to memory and
+// CLUSTER: the group's CTAs are a cluster (a power of two of them, so some may have no split).  A row's
+// partial results go straight to the shared memory of CTA row % CTAs, which merges them in key order
+// after the cluster barrier.  Otherwise (more splits than a portable cluster has CTAs, or more groups
+// than the GPU holds clusters of: then clusters wait for one another's SMs) they go to memory and
 // k_step_merge merges them.
-constexpr int SA_WARPS = 8;   // compute warps of a cluster's CTA (two splits' units)
+//
+// A step of ~6.5 us is bound by its warps' latency, not by K/V bytes (17 rows at 512 tokens: scores, softmax and PV
+// 2.4 us, exchange 1.4, merge 1.3).  The q rows lie in shared memory and each MMA group's fragments are
+// loaded before its MMAs; with all of q's fragments in registers the compiler had too few left to batch
+// those loads (verify pass 779 us against 769; 4096 tokens 934 against 899).
+constexpr int SA_WARPS = 6;   // compute warps of a cluster's CTA: the units of 17 rows with two heads a group
 constexpr int SG_WARPS = 4;   // compute warps of a single split's CTA
 constexpr int SA_STATS = 4;   // partial results per row at most: 32 x this
-
-template <int DH>
-struct SaLayout {
-    static constexpr int SPB = 2 * (DH / 64) * ATT_SUB_BYTES;  // K, then V of a split
-    static constexpr int PITCH = DH + 4;                       // floats per partial row
-};
 
 // Merge of one row's nv partial results in key order, relative to the row's overall maximum (attn_combine in
 // pass_kernel.cu): lane l gathers the statistics of partials l, l + 32, ... and the outputs 4l..4l+3.
@@ -503,254 +615,248 @@ __device__ __forceinline__ void merge_row(int nv, int lane, FS stat, FO out, bf1
 }
 
 template <int DH, bool BLK, bool CLUSTER>
-__global__ void __launch_bounds__(32 * (CLUSTER ? SA_WARPS : SG_WARPS) + 32, CLUSTER ? 1 : 2)
+__global__ void __launch_bounds__(32 * (CLUSTER ? SA_WARPS : SG_WARPS) + 32, CLUSTER ? 1 : 3)
     k_step_attn(const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap vmap,
-                const __grid_constant__ StepArgs a, int layer, int bufs, int parts) {
-    using LY = SaLayout<DH>;
-    constexpr int WARPS = CLUSTER ? SA_WARPS : SG_WARPS;
-    constexpr int KS = DH / 16, DT = DH / 8, SUBS = DH / 64, NP = ATT_SPLIT / PAGE;
+                const __grid_constant__ StepArgs a, int layer, int parts, const __grid_constant__ StepSplits sp) {
+    constexpr int WARPS = CLUSTER ? SA_WARPS : SG_WARPS, PITCH = DH + 4, QP = ATT_Q_PITCH(DH);
+    constexpr int DT = DH / 8, SUBS = DH / 64, NP = ATT_SPLIT / PAGE;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    __shared__ uint64_t full[2], empty[2];
-    __shared__ int s_abort;
+    __shared__ uint64_t full;
     const Dims &dm = a.dm;
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
-    const int rank = blockIdx.x, cs = gridDim.x, g = blockIdx.y, bl = blockIdx.z;
+    // (without clusters the sequences' splits lie end to end along x)
+    int bl = blockIdx.z;
+    if (!CLUSTER)
+        while (blockIdx.x >= sp.start[bl + 1]) ++bl;
+    const int split = blockIdx.x - (CLUSTER ? 0 : sp.start[bl]), cs = gridDim.x, g = blockIdx.y;
     const int b = a.pd.b0 + bl, R = a.pd.R, grp = dm.Hq / dm.Hkv, RH = R * grp;
-    const int sub_sh = a.att_subs - 1, HALF = ATT_SPLIT >> sub_sh;          // one or two partial results per split
-    float *po = reinterpret_cast<float *>(base + bufs * LY::SPB);           // [parts][RH][PITCH]
-    float2 *pml = reinterpret_cast<float2 *>(po + (size_t)parts * RH * LY::PITCH);  // [parts][RH]
+    const int sub_sh = a.att_subs - 1, HALF = ATT_SPLIT >> sub_sh;  // one or two partial results per split
+    // CLUSTER: the partial results of the rows that this CTA merges
+    const int cs_sh = __ffs(cs) - 1, rpo = (RH + cs - 1) / cs;           // (cs is a power of two there)
+    const uint32_t sq = smem_u32(base + 2 * SUBS * ATT_SUB_BYTES);       // q rows (16 a tile), QP bytes each
+    const uint32_t po = sq + (uint32_t)((RH + 15) / 16 * 16 * QP);       // [parts][rpo][PITCH]
+    const uint32_t pml = po + (uint32_t)(parts * rpo * PITCH) * 4u;      // [parts][rpo] (m, l)
     if (threadIdx.x == 0) {
-        for (int i = 0; i < 2; ++i) {
-            mbar_init(&full[i], 1);
-            mbar_init(&empty[i], WARPS);
-        }
-        s_abort = 0;
+        mbar_init(&full, 1);
         fence_mbarrier_init();
         prefetch_tensormap(&kmap);
         prefetch_tensormap(&vmap);
     }
     __syncthreads();
+    if (CLUSTER) cluster_arrive();  // (this CTA's shared memory exists: its peers wait for that before they write there)
     pdl_launch();
     // the cached length was set by a kernel that finished before this pass began
-    const int L = a.L[b], T = L + R, nsp = (T + ATT_SPLIT - 1) / ATT_SPLIT;
-    const int mine = rank < nsp ? (nsp - 1 - rank) / cs + 1 : 0;  // splits of this CTA
+    const int L = a.L[b], T = L + R, nsp = (T + ATT_SPLIT - 1) / ATT_SPLIT, k0 = split * ATT_SPLIT;
+    const bool active = split < nsp;
 
     if (warp == WARPS) {
-        // ---- producer warp: lane p the page p of a split.  Pages entirely below L hold earlier passes' keys
-        // and are requested at once; the block's own after the wait (their page ids are read before it).
-        auto page_of = [&](int j) {
-            const int s = rank + j * cs, p = s * NP + lane;
-            return lane < NP && p * PAGE < T && p < a.kv.pages_per_seq ? a.kv.page_table[(size_t)b * a.kv.pages_per_seq + p] : -1;
-        };
-        auto request = [&](int j, int buf, int page, bool cached) {
-            const int kp = (rank + j * cs) * ATT_SPLIT + lane * PAGE;
-            const unsigned mask = __ballot_sync(0xffffffffu, page >= 0 && (kp + PAGE <= L) == cached);
-            const uint32_t bytes = (uint32_t)__popc(mask) * 2u * SUBS * PAGE * 128u;
-            if (lane == 0) {
-                if (!cached)
-                    mbar_arrive_expect_tx(&full[buf], bytes);
-                else if (bytes)
-                    mbar_expect_tx(&full[buf], bytes);
-            }
-            __syncwarp();
+        // ---- producer warp: lane p the page p of the split.  Pages entirely below L hold earlier passes' keys and
+        // are requested at once; the block's own after the wait.
+        if (active) {
+            const int pg = split * NP + lane, kp = k0 + lane * PAGE;
+            const int page = lane < NP && kp < T && pg < a.kv.pages_per_seq ? a.kv.page_table[(size_t)b * a.kv.pages_per_seq + pg] : -1;
+            auto request = [&](bool cached) {
+                const unsigned mask = __ballot_sync(0xffffffffu, page >= 0 && (kp + PAGE <= L) == cached);
+                const uint32_t bytes = (uint32_t)__popc(mask) * 2u * SUBS * PAGE * 128u;
+                if (lane == 0) {
+                    if (!cached)
+                        mbar_arrive_expect_tx(&full, bytes);
+                    else if (bytes)
+                        mbar_expect_tx(&full, bytes);
+                }
+                __syncwarp();
 #pragma unroll 1
-            for (int c0 = 0; c0 < NP * 2 * SUBS; c0 += 32) {
-                const int cp = c0 + lane, p = cp / (2 * SUBS), q = cp % (2 * SUBS);
-                const int pg = __shfl_sync(0xffffffffu, page, p & 31);
-                if (p < NP && ((mask >> p) & 1u))
-                    tma_load_2d(base + buf * LY::SPB + q * ATT_SUB_BYTES + p * PAGE * 128, q / SUBS ? &vmap : &kmap,
-                                (q % SUBS) * 64, ((layer * a.kv.n_pages + pg) * dm.Hkv + g) * PAGE, &full[buf]);
-            }
-        };
-        const int p0 = mine > 0 ? page_of(0) : -1, p1 = mine > 1 && bufs > 1 ? page_of(1) : -1;
-        if (mine > 0) request(0, 0, p0, true);
-        if (mine > 1 && bufs > 1) request(1, 1, p1, true);
-        pdl_wait();
-        fence_proxy_async_global();
-        int j = 0;
-        for (; j < mine; ++j) {
-            const int buf = bufs > 1 ? j & 1 : 0;
-            int page = j == 0 ? p0 : p1;
-            if (j >= bufs) {
-                page = page_of(j);
-                if (!mbar_wait(&empty[buf], ((bufs > 1 ? j >> 1 : j) - 1) & 1, a.status, DEV_TIMEOUT_SLOT, &s_abort)) break;
-                request(j, buf, page, true);
-            }
-            request(j, buf, page, false);
+                for (int c0 = 0; c0 < NP * 2 * SUBS; c0 += 32) {
+                    const int cp = c0 + lane, p = cp / (2 * SUBS), q = cp % (2 * SUBS);
+                    const int phys = __shfl_sync(0xffffffffu, page, p & 31);
+                    if (p < NP && ((mask >> p) & 1u))
+                        tma_load_2d(base + q * ATT_SUB_BYTES + p * PAGE * 128, q / SUBS ? &vmap : &kmap, (q % SUBS) * 64,
+                                    ((layer * a.kv.n_pages + phys) * dm.Hkv + g) * PAGE, &full);
+                }
+            };
+            request(true);
+            pdl_wait();
+            fence_proxy_async_global();
+            request(false);
+            mbar_wait(&full, 0, nullptr, 0, nullptr);  // (the copies land before this CTA's memory goes)
         }
-        if (*(volatile int *)&s_abort)  // error path: the copies in flight get a bounded chance to land
-            for (int h = j > bufs ? j - bufs : 0; h < j; ++h)
-                mbar_wait(&full[bufs > 1 ? h & 1 : 0], (bufs > 1 ? h >> 1 : h) & 1, nullptr, 0, nullptr);
+        if (CLUSTER) cluster_wait();
     } else {
-        pdl_wait();
-        const int gq = lane >> 2, tq = lane & 3, n_mt = (RH + 15) / 16;
+        const int gq = lane >> 2, tq = lane & 3, n_units = ((RH + 15) / 16) << sub_sh;
         const float scale = a.att_scale;
-        const uint32_t koff = attn_k_lane(lane), voff = attn_v_lane(lane);
-        uint32_t ph = 0;
-        for (int j0 = 0; j0 < mine; j0 += bufs, ph ^= 1) {
-            const int nsx = min(bufs, mine - j0);
-            bool landed = true;
-            for (int i = 0; i < nsx; ++i)
-                landed = landed && mbar_wait(&full[i], ph, a.status, DEV_TIMEOUT_LOAD, &s_abort);
-            if (!landed) break;
-#pragma unroll 1
-            for (int unit = warp; unit < ((n_mt * nsx) << sub_sh); unit += WARPS) {
-                // (nsx is 1 or 2)
-                const int half = unit & sub_sh, us = unit >> sub_sh, sp = us & (nsx - 1), mt = us >> (nsx - 1), kb = half * HALF;
-                const int k0 = (rank + (j0 + sp) * cs) * ATT_SPLIT;
-                const uint32_t ka = smem_u32(base + sp * LY::SPB) + koff + kb * 128;
-                const uint32_t va = smem_u32(base + sp * LY::SPB + SUBS * ATT_SUB_BYTES) + voff + kb * 128;
-                const int qv0 = mt * 16 + gq, qv1 = qv0 + 8;
-                const bool val0 = qv0 < RH, val1 = qv1 < RH;
-                const int i0 = val0 ? qv0 / grp : 0, i1 = val1 ? qv1 / grp : 0;
-                uint32_t qa[KS][4];
-                {
-                    const bf16 *q0 = a.q + ((size_t)(bl * R + i0) * dm.Hq + g * grp + (val0 ? qv0 % grp : 0)) * DH + 2 * tq;
-                    const bf16 *q1 = a.q + ((size_t)(bl * R + i1) * dm.Hq + g * grp + (val1 ? qv1 % grp : 0)) * DH + 2 * tq;
-#pragma unroll
-                    for (int ks = 0; ks < KS; ++ks) {
-                        qa[ks][0] = val0 ? __ldcg(reinterpret_cast<const unsigned *>(q0 + ks * 16)) : 0u;
-                        qa[ks][1] = val1 ? __ldcg(reinterpret_cast<const unsigned *>(q1 + ks * 16)) : 0u;
-                        qa[ks][2] = val0 ? __ldcg(reinterpret_cast<const unsigned *>(q0 + ks * 16 + 8)) : 0u;
-                        qa[ks][3] = val1 ? __ldcg(reinterpret_cast<const unsigned *>(q1 + ks * 16 + 8)) : 0u;
-                    }
-                }
-                // last visible key of each row (the draft's mask rows see the whole block)
-                const int lim0 = val0 ? ((BLK && i0 >= 1) ? T - 1 : L + i0) : -1;
-                const int lim1 = val1 ? ((BLK && i1 >= 1) ? T - 1 : L + i1) : -1;
-                float m0 = -INFINITY, m1 = -INFINITY, l0 = 0.f, l1 = 0.f;
-                float oc[DT][4];
-#pragma unroll
-                for (int dt = 0; dt < DT; ++dt) oc[dt][0] = oc[dt][1] = oc[dt][2] = oc[dt][3] = 0.f;
-                const int kend = min(HALF, T - (k0 + kb));
-#pragma unroll 1
-                for (int c0 = 0; c0 < kend; c0 += 32) {
-                    float sc[4][4];
-                    attn_scores<DH>(ka + c0 * 128, qa, sc);
-                    float c0m = -INFINITY, c1m = -INFINITY;
-#pragma unroll
-                    for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-                        for (int e = 0; e < 2; ++e) {
-                            const int kp = k0 + kb + c0 + nt * 8 + 2 * tq + e;
-                            sc[nt][e] = kp <= lim0 ? __fmul_rn(sc[nt][e], scale) : -INFINITY;
-                            sc[nt][2 + e] = kp <= lim1 ? __fmul_rn(sc[nt][2 + e], scale) : -INFINITY;
-                            c0m = fmaxf(c0m, sc[nt][e]);
-                            c1m = fmaxf(c1m, sc[nt][2 + e]);
-                        }
-                    c0m = fmaxf(c0m, __shfl_xor_sync(0xffffffffu, c0m, 1));
-                    c0m = fmaxf(c0m, __shfl_xor_sync(0xffffffffu, c0m, 2));
-                    c1m = fmaxf(c1m, __shfl_xor_sync(0xffffffffu, c1m, 1));
-                    c1m = fmaxf(c1m, __shfl_xor_sync(0xffffffffu, c1m, 2));
-                    const float n0 = fmaxf(m0, c0m), n1 = fmaxf(m1, c1m);
-                    if (__any_sync(0xffffffffu, (n0 != m0 && m0 != -INFINITY) || (n1 != m1 && m1 != -INFINITY))) {
-                        const float a0 = m0 == -INFINITY ? 0.f : __expf(m0 - n0), a1 = m1 == -INFINITY ? 0.f : __expf(m1 - n1);
-                        l0 = __fmul_rn(l0, a0);
-                        l1 = __fmul_rn(l1, a1);
-#pragma unroll
-                        for (int dt = 0; dt < DT; ++dt) {
-                            oc[dt][0] = __fmul_rn(oc[dt][0], a0);
-                            oc[dt][1] = __fmul_rn(oc[dt][1], a0);
-                            oc[dt][2] = __fmul_rn(oc[dt][2], a1);
-                            oc[dt][3] = __fmul_rn(oc[dt][3], a1);
-                        }
-                    }
-                    const float z0 = n0 == -INFINITY ? 0.f : n0, z1 = n1 == -INFINITY ? 0.f : n1;
-                    m0 = n0;
-                    m1 = n1;
-#pragma unroll
-                    for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-                        for (int e = 0; e < 2; ++e) {
-                            sc[nt][e] = __expf(sc[nt][e] - z0);  // (0 for a masked score)
-                            sc[nt][2 + e] = __expf(sc[nt][2 + e] - z1);
-                            l0 += sc[nt][e];
-                            l1 += sc[nt][2 + e];
-                        }
-#pragma unroll
-                    for (int kstep = 0; kstep < 2; ++kstep) {
-                        uint32_t pa[4];
-                        pa[0] = pack_bf162(sc[2 * kstep][0], sc[2 * kstep][1]);
-                        pa[1] = pack_bf162(sc[2 * kstep][2], sc[2 * kstep][3]);
-                        pa[2] = pack_bf162(sc[2 * kstep + 1][0], sc[2 * kstep + 1][1]);
-                        pa[3] = pack_bf162(sc[2 * kstep + 1][2], sc[2 * kstep + 1][3]);
-                        // V of keys at or past T is zero in the fragments (see attn_split)
-                        const int kst = k0 + kb + c0 + kstep * 16;
-                        uint32_t ma = 0xFFFFFFFFu, mb = 0xFFFFFFFFu;
-                        if (kst + 16 > T) {
-                            const int kf = kst + 2 * tq;
-                            ma = (kf < T ? 0x0000FFFFu : 0u) | (kf + 1 < T ? 0xFFFF0000u : 0u);
-                            mb = (kf + 8 < T ? 0x0000FFFFu : 0u) | (kf + 9 < T ? 0xFFFF0000u : 0u);
-                        }
-                        attn_pv<DH>(va + (c0 + kstep * 16) * 128, pa, ma, mb, oc);
-                    }
-                }
-                l0 += __shfl_xor_sync(0xffffffffu, l0, 1);
-                l0 += __shfl_xor_sync(0xffffffffu, l0, 2);
-                l1 += __shfl_xor_sync(0xffffffffu, l1, 1);
-                l1 += __shfl_xor_sync(0xffffffffu, l1, 2);
-                auto store = [&](bool val, int qv, int i, float m, float l, int e) {
-                    if (!val) return;
-                    float *dst;
-                    if constexpr (CLUSTER) {
-                        const int row = (((j0 + sp) << sub_sh) + half) * RH + qv;
-                        dst = po + (size_t)row * LY::PITCH + 2 * tq;
-                        if (tq == 0) pml[row] = make_float2(m, l);
-                    } else {
-                        const size_t row = ((size_t)(bl * R + i) * dm.Hq + g * grp + qv % grp) * a.att_splits_alloc +
-                                           (((size_t)rank << sub_sh) + half);
-                        dst = a.o_part + row * DH + 2 * tq;
-                        if (tq == 0) a.ml_part[row] = make_float2(m, l);
-                    }
-#pragma unroll
-                    for (int dt = 0; dt < DT; ++dt)
-                        *reinterpret_cast<float2 *>(dst + dt * 8) = make_float2(oc[dt][e], oc[dt][e + 1]);
-                };
-                store(val0, qv0, i0, m0, l0, 0);
-                store(val1, qv1, i1, m1, l1, 2);
+        const uint32_t ka = smem_u32(base) + attn_k_lane(lane);
+        const uint32_t va = smem_u32(base + SUBS * ATT_SUB_BYTES) + attn_v_lane(lane), qoff = attn_q_lane<DH>(lane);
+        pdl_wait();
+        // the group's q rows through L2 while the block's pages land
+        if (active) {
+            for (int q = threadIdx.x; q < RH * (DH / 8); q += 32 * WARPS) {
+                const int qv = q / (DH / 8), c = q % (DH / 8);
+                cp_async16_at(sq + (uint32_t)(qv * QP + c * 16),
+                              a.q + ((size_t)(bl * R + qv / grp) * dm.Hq + g * grp + qv % grp) * DH + c * 8);
             }
-            __syncwarp();
-            if (lane == 0)
-                for (int i = 0; i < nsx; ++i) mbarrier_arrive_one(&empty[i]);
+            cp_async_commit();
+            cp_async_wait_all();
+            asm volatile("bar.sync 1, %0;" ::"n"(32 * WARPS) : "memory");
+        }
+        if (CLUSTER) cluster_wait();
+        bool landed = false;
+#pragma unroll 1
+        for (int unit = warp; active && unit < n_units; unit += WARPS) {
+            const int half = unit & sub_sh, mt = unit >> sub_sh, kb = half * HALF;
+            const int qv0 = mt * 16 + gq, qv1 = qv0 + 8;
+            const bool val0 = qv0 < RH, val1 = qv1 < RH;
+            const int i0 = val0 ? qv0 / grp : 0, i1 = val1 ? qv1 / grp : 0;
+            if (!landed && !(landed = mbar_wait(&full, 0, a.status, DEV_TIMEOUT_LOAD, nullptr))) break;
+            // last visible key of each row (the draft's mask rows see the whole block)
+            const int lim0 = val0 ? ((BLK && i0 >= 1) ? T - 1 : L + i0) : -1;
+            const int lim1 = val1 ? ((BLK && i1 >= 1) ? T - 1 : L + i1) : -1;
+            float m0 = -INFINITY, m1 = -INFINITY, l0 = 0.f, l1 = 0.f;
+            float oc[DT][4];
+#pragma unroll
+            for (int dt = 0; dt < DT; ++dt) oc[dt][0] = oc[dt][1] = oc[dt][2] = oc[dt][3] = 0.f;
+            const int kend = min(HALF, T - (k0 + kb));
+#pragma unroll 1
+            for (int c0 = 0; c0 < kend; c0 += 32) {
+                float sc[4][4];
+                attn_scores_sq<DH>(ka + (kb + c0) * 128, sq + (uint32_t)(mt * 16 * QP) + qoff, sc);
+                float c0m = -INFINITY, c1m = -INFINITY;
+#pragma unroll
+                for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const int kp = k0 + kb + c0 + nt * 8 + 2 * tq + e;
+                        sc[nt][e] = kp <= lim0 ? __fmul_rn(sc[nt][e], scale) : -INFINITY;
+                        sc[nt][2 + e] = kp <= lim1 ? __fmul_rn(sc[nt][2 + e], scale) : -INFINITY;
+                        c0m = fmaxf(c0m, sc[nt][e]);
+                        c1m = fmaxf(c1m, sc[nt][2 + e]);
+                    }
+                c0m = fmaxf(c0m, __shfl_xor_sync(0xffffffffu, c0m, 1));
+                c0m = fmaxf(c0m, __shfl_xor_sync(0xffffffffu, c0m, 2));
+                c1m = fmaxf(c1m, __shfl_xor_sync(0xffffffffu, c1m, 1));
+                c1m = fmaxf(c1m, __shfl_xor_sync(0xffffffffu, c1m, 2));
+                const float n0 = fmaxf(m0, c0m), n1 = fmaxf(m1, c1m);
+                if (__any_sync(0xffffffffu, (n0 != m0 && m0 != -INFINITY) || (n1 != m1 && m1 != -INFINITY))) {
+                    const float a0 = m0 == -INFINITY ? 0.f : __expf(m0 - n0), a1 = m1 == -INFINITY ? 0.f : __expf(m1 - n1);
+                    l0 = __fmul_rn(l0, a0);
+                    l1 = __fmul_rn(l1, a1);
+#pragma unroll
+                    for (int dt = 0; dt < DT; ++dt) {
+                        oc[dt][0] = __fmul_rn(oc[dt][0], a0);
+                        oc[dt][1] = __fmul_rn(oc[dt][1], a0);
+                        oc[dt][2] = __fmul_rn(oc[dt][2], a1);
+                        oc[dt][3] = __fmul_rn(oc[dt][3], a1);
+                    }
+                }
+                const float z0 = n0 == -INFINITY ? 0.f : n0, z1 = n1 == -INFINITY ? 0.f : n1;
+                m0 = n0;
+                m1 = n1;
+#pragma unroll
+                for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        sc[nt][e] = __expf(sc[nt][e] - z0);  // (0 for a masked score)
+                        sc[nt][2 + e] = __expf(sc[nt][2 + e] - z1);
+                        l0 += sc[nt][e];
+                        l1 += sc[nt][2 + e];
+                    }
+#pragma unroll
+                for (int kstep = 0; kstep < 2; ++kstep) {
+                    uint32_t pa[4];
+                    pa[0] = pack_bf162(sc[2 * kstep][0], sc[2 * kstep][1]);
+                    pa[1] = pack_bf162(sc[2 * kstep][2], sc[2 * kstep][3]);
+                    pa[2] = pack_bf162(sc[2 * kstep + 1][0], sc[2 * kstep + 1][1]);
+                    pa[3] = pack_bf162(sc[2 * kstep + 1][2], sc[2 * kstep + 1][3]);
+                    // V of keys at or past T is zero in the fragments (see attn_split)
+                    const int kst = k0 + kb + c0 + kstep * 16;
+                    uint32_t ma = 0xFFFFFFFFu, mb = 0xFFFFFFFFu;
+                    if (kst + 16 > T) {
+                        const int kf = kst + 2 * tq;
+                        ma = (kf < T ? 0x0000FFFFu : 0u) | (kf + 1 < T ? 0xFFFF0000u : 0u);
+                        mb = (kf + 8 < T ? 0x0000FFFFu : 0u) | (kf + 9 < T ? 0xFFFF0000u : 0u);
+                    }
+                    attn_pv<DH>(va + (kb + c0 + kstep * 16) * 128, pa, ma, mb, oc);
+                }
+            }
+            l0 += __shfl_xor_sync(0xffffffffu, l0, 1);
+            l0 += __shfl_xor_sync(0xffffffffu, l0, 2);
+            l1 += __shfl_xor_sync(0xffffffffu, l1, 1);
+            l1 += __shfl_xor_sync(0xffffffffu, l1, 2);
+            const int part = (split << sub_sh) + half;
+            auto store = [&](bool val, int qv, int i, float m, float l, int e) {
+                if (!val) return;
+                if constexpr (CLUSTER) {
+                    const int row = part * rpo + (qv >> cs_sh), to = qv & (cs - 1);
+                    const uint32_t dst = map_cta(po + (uint32_t)(row * PITCH + 2 * tq) * 4u, to);
+                    if (tq == 0) st_cluster_v2(map_cta(pml + (uint32_t)row * 8u, to), m, l);
+#pragma unroll
+                    for (int dt = 0; dt < DT; ++dt) st_cluster_v2(dst + dt * 32, oc[dt][e], oc[dt][e + 1]);
+                } else {
+                    const size_t row = ((size_t)(bl * R + i) * dm.Hq + g * grp + qv % grp) * a.att_splits_alloc + part;
+                    float *dst = a.o_part + row * DH + 2 * tq;
+                    if (tq == 0) a.ml_part[row] = make_float2(m, l);
+#pragma unroll
+                    for (int dt = 0; dt < DT; ++dt) *reinterpret_cast<float2 *>(dst + dt * 8) = make_float2(oc[dt][e], oc[dt][e + 1]);
+                }
+            };
+            store(val0, qv0, i0, m0, l0, 0);
+            store(val1, qv1, i1, m1, l1, 2);
         }
     }
     if constexpr (CLUSTER) {
         __syncwarp();
         cluster_sync();
-        if (warp < SA_WARPS) {
-            const int cs_sh = __ffs(cs) - 1;  // (a power of two)
-            const uint32_t poa = smem_u32(po), pma = smem_u32(pml);
-            for (int qv = rank + warp * cs; qv < RH; qv += cs * SA_WARPS) {
-                // partial p: split p >> sub_sh, the (split / cs)-th of CTA split % cs
-                auto at = [&](uint32_t first, int p, uint32_t bytes) {
-                    const int sp = p >> sub_sh;
-                    return map_cta(first + (uint32_t)((((sp >> cs_sh) << sub_sh) + (p & sub_sh)) * RH + qv) * bytes, sp & (cs - 1));
-                };
+        if (warp < SA_WARPS)
+            for (int qv = split + warp * cs; qv < RH; qv += cs * SA_WARPS)
                 merge_row<DH>(
-                    nsp << sub_sh, lane, [&](int p) { return ld_cluster_v2(at(pma, p, 8u)); },
-                    [&](int p, int c) { return ld_cluster_v4(at(poa, p, LY::PITCH * 4u) + (uint32_t)c * 4u); },
+                    nsp << sub_sh, lane, [&](int p) { return ld_shared_v2(pml + (uint32_t)(p * rpo + (qv >> cs_sh)) * 8u); },
+                    [&](int p, int c) { return ld_shared_v4(po + (uint32_t)((p * rpo + (qv >> cs_sh)) * PITCH + c) * 4u); },
                     a.attn + ((size_t)(bl * R + qv / grp) * dm.Hq + g * grp + qv % grp) * DH);
-            }
-        }
-        cluster_sync();  // no CTA leaves while another still reads its partials
     }
 }
 
-// One warp per (row, query head): merge of the partial results in memory.
+// Merge of the partial results in memory (as merge_row): a block per (row, query head), a thread per
+// dimension, so that up to 32 partial outputs are on their way at once.
 template <int DH>
-__global__ void __launch_bounds__(256) k_step_merge(const __grid_constant__ StepArgs a) {
-    const int lane = threadIdx.x & 31, un = blockIdx.x * 8 + (threadIdx.x >> 5);
-    const int m = un / a.dm.Hq;
+__global__ void __launch_bounds__(DH) k_step_merge(const __grid_constant__ StepArgs a) {
+    constexpr int OB = 32;
+    const int lane = threadIdx.x & 31, m = blockIdx.x / a.dm.Hq;
     pdl_launch();
-    const int T = m < a.pd.M ? a.L[a.pd.b0 + m / a.pd.R] + a.pd.R : 0;
+    const int nv = (a.L[a.pd.b0 + m / a.pd.R] + a.pd.R + ATT_SPLIT - 1) / ATT_SPLIT * a.att_subs;
+    const size_t row = (size_t)blockIdx.x * a.att_splits_alloc;
+    const float *op = a.o_part + row * DH + threadIdx.x;
     pdl_wait();
-    if (m >= a.pd.M) return;
-    const size_t row = (size_t)un * a.att_splits_alloc;
-    merge_row<DH>(
-        (T + ATT_SPLIT - 1) / ATT_SPLIT * a.att_subs, lane, [&](int p) { return __ldcg(a.ml_part + row + p); },
-        [&](int p, int c) { return __ldcg(reinterpret_cast<const float4 *>(a.o_part + (row + p) * DH + c)); },
-        a.attn + (size_t)un * DH);
+    float2 st[SA_STATS];
+    float o[OB];
+#pragma unroll
+    for (int i = 0; i < SA_STATS; ++i)
+        st[i] = 32 * i + lane < nv ? __ldcg(a.ml_part + row + 32 * i + lane) : make_float2(-INFINITY, 0.f);
+#pragma unroll
+    for (int u = 0; u < OB; ++u) o[u] = u < nv ? __ldcg(op + (size_t)u * DH) : 0.f;
+    float mx = -INFINITY;
+#pragma unroll
+    for (int i = 0; i < SA_STATS; ++i)
+        if (st[i].y > 0.f) mx = fmaxf(mx, st[i].x);
+#pragma unroll
+    for (int off = 16; off >= 1; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+    float num = 0.f, den = 0.f;
+#pragma unroll
+    for (int i = 0; i < SA_STATS; ++i) {
+        if (32 * i >= nv) break;
+        if (i > 0)
+#pragma unroll
+            for (int u = 0; u < OB; ++u) o[u] = 32 * i + u < nv ? __ldcg(op + (size_t)(32 * i + u) * DH) : 0.f;
+        const float wl = __expf(st[i].x - mx);
+#pragma unroll
+        for (int u = 0; u < OB; ++u) {
+            if (32 * i + u >= nv) break;
+            const float wt = __shfl_sync(0xffffffffu, wl, u), l = __shfl_sync(0xffffffffu, st[i].y, u);
+            if (!(l > 0.f)) continue;  // the row saw no key in this partial result
+            den = __fadd_rn(den, __fmul_rn(wt, l));
+            num = __fadd_rn(num, __fmul_rn(wt, o[u]));
+        }
+    }
+    a.attn[(size_t)blockIdx.x * DH + threadIdx.x] = f2bf(__fdiv_rn(num, den));
 }
 
 // ------------------------------------------------------------------ ends of the pass
@@ -812,37 +918,41 @@ __global__ void __launch_bounds__(256) k_step_final(const __grid_constant__ Step
 
 // ------------------------------------------------------------------ host side
 
-constexpr int ST_SMEM = 220 * 1024;   // dynamic shared memory of one CTA at most
+constexpr int ST_SMEM = 216 * 1024;   // dynamic shared memory of one CTA at most
 constexpr int ST_MAX_CLUSTER = 16;
+// Rows up to which partial sums are pushed: a pushed row costs a scalar remote store per thread (~40 ns), pulling
+// costs a remote round trip and a second cluster barrier (~0.8 us) once (17 rows: verify pass 896 us pulled, 799
+// pushed; 136 rows: 1823 pulled, 2032 pushed).
+constexpr int ST_PUSH_ROWS = 32;
 
 static int step_bn(int M) { return std::max(32, (M + 15) / 16 * 16); }
 
-static int lin_smem(int bn, int ra, bool ad) { return ra * (TILE_BYTES + (ad ? ST_A_BYTES : 0) + bn * 128) + 1024; }
-
-// ring atoms of a linear with katoms per slice (0: does not fit)
-static int lin_ring(int bn, int M, int katoms, bool ad, int ru) {
+// Ring atoms of a linear with katoms per slice (0: does not fit), whether its partial sums have room behind the
+// ring (push), and the dynamic shared memory.
+static int lin_ring(int bn, int M, int katoms, int ks, bool ad, int ru, int *push, size_t *smem) {
     for (int ra : {katoms, ST_HALF}) {
-        const int room = lin_smem(bn, ra, ad) - 1024;
-        if (room + 1024 <= ST_SMEM && (int)sizeof(float) * M * (TILE_ROWS + ru) <= room) return ra;
+        const int ring = ra * (TILE_BYTES + (ad ? ST_A_BYTES : 0) + bn * 128);
+        const int behind = (int)sizeof(float) * ks * ((M + ks - 1) / ks) * (TILE_ROWS + ru);
+        if (ring + 1024 > ST_SMEM) continue;
+        *push = M <= ST_PUSH_ROWS && ring + behind + 1024 <= ST_SMEM ? 1 : 0;
+        *smem = (size_t)ring + (*push ? behind : 0) + 1024;
+        if (*push || (int)sizeof(float) * M * (TILE_ROWS + ru) <= ring) return ra;
     }
     return 0;
 }
 
-static int attn_smem(const Dims &dm, int R, int bufs, int parts) {
-    const int rh = R * (dm.Hq / dm.Hkv);
-    return bufs * 2 * (dm.d / 64) * ATT_SUB_BYTES + parts * rh * ((dm.d + 4) * 4 + 8) + 1024;
+static int attn_smem(const Dims &dm, int R, int parts, int rows) {
+    return 2 * (dm.d / 64) * ATT_SUB_BYTES + (R * (dm.Hq / dm.Hkv) + 15) / 16 * 16 * ATT_Q_PITCH(dm.d) + parts * rows * ((dm.d + 4) * 4 + 8) + 1024;
 }
 
-// The attention's form: cs CTAs of a cluster per (sequence, KV head) with bufs staged splits and `parts` partial
-// results each, or cs = 0: one CTA per split and a merge kernel.  Clusters while each split gets its own
-// CTA in a portable cluster, the partial results fit, and every cluster has its SMs at once.
-static int attn_cluster(const Dims &dm, const PassDesc &pd, int subs, int nsplit, int *bufs, int *parts) {
+// The attention's form: the CTAs of a cluster per (sequence, KV head), a split each, or 0: one CTA per split and
+// a merge kernel.  Clusters while a portable one has a CTA for each split, the partial results of the rows
+// that a CTA merges fit, and every cluster has its SMs at once.
+static int attn_cluster(const Dims &dm, const PassDesc &pd, int subs, int nsplit, size_t *smem) {
     int c = 1;
     while (c < nsplit && c < 8) c *= 2;
-    *bufs = std::min(2, (nsplit + c - 1) / c);
-    *parts = (nsplit + c - 1) / c * subs;
-    const bool ok = c >= nsplit && pd.nb * dm.Hkv * c <= gemm_ctas() && attn_smem(dm, pd.R, *bufs, *parts) <= ST_SMEM;
-    return ok ? c : 0;
+    *smem = attn_smem(dm, pd.R, nsplit * subs, (pd.R * (dm.Hq / dm.Hkv) + c - 1) / c);
+    return c >= nsplit && pd.nb * dm.Hkv * c <= gemm_ctas() && *smem <= (size_t)ST_SMEM ? c : 0;
 }
 
 bool step_pass_fits(const Dims &dm, const PassDesc &pd, int subs, int nsplit) {
@@ -851,10 +961,13 @@ bool step_pass_fits(const Dims &dm, const PassDesc &pd, int subs, int nsplit) {
     if (pd.M > 256 || dm.r > ST_RANK) return false;
     for (int lin = 0; lin < 4; ++lin) {
         const int ka = mk_slice_atoms(lin, K[lin]);
-        if (K[lin] / (ka * KT) > ST_MAX_CLUSTER) return false;
-        if (lin_ring(bn, pd.M, ka, pd.adapter, pd.adapter ? (lin == 2 ? 2 : 1) * dm.r : 0) == 0) return false;
+        const int ks = K[lin] / (ka * KT), ru = pd.adapter ? (lin == 2 ? 2 : 1) * dm.r : 0;
+        int push;
+        size_t smem;
+        if (ks > ST_MAX_CLUSTER || lin_ring(bn, pd.M, ka, ks, pd.adapter, ru, &push, &smem) == 0) return false;
     }
-    return nsplit * subs <= 32 * SA_STATS;  // (statistics a merging warp holds)
+    // (statistics a merging warp holds; a split's pages and the group's q rows)
+    return nsplit * subs <= 32 * SA_STATS && attn_smem(dm, pd.R, 0, 0) <= ST_SMEM;
 }
 
 template <typename... P, typename... A>
@@ -877,12 +990,16 @@ static cudaError_t launch_step(void (*kernel)(P...), dim3 grid, dim3 cluster, in
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
-template <int DH>
+// More threads for more rows: staging and finishing rows are loops over them (136 rows, 0.6B
+// shape: verify pass 1763 us with 256 threads, 1619 with 512; at 17 rows the wider CTA starts later).
+static int lin_threads(int M) { return M <= 64 ? 256 : 512; }
+
+template <int DH, int NT>
 static cudaError_t launch_lin(int lin, bool ad, dim3 grid, size_t smem, const StepArgs &a, const StepLin &w, cudaStream_t st) {
     const dim3 cl(1, grid.y);
-#define STEP_LIN(L)                                                                                                      \
-    return ad ? launch_step(k_step_linear<L, true, DH>, grid, cl, ST_THREADS, smem, st, a, w)                            \
-              : launch_step(k_step_linear<L, false, DH>, grid, cl, ST_THREADS, smem, st, a, w)
+#define STEP_LIN(L)                                                                                              \
+    return ad ? launch_step(k_step_linear<L, true, DH, NT>, grid, cl, NT, smem, st, a, w)                        \
+              : launch_step(k_step_linear<L, false, DH, NT>, grid, cl, NT, smem, st, a, w)
     switch (lin) {
         case 0: STEP_LIN(0);
         case 1: STEP_LIN(1);
@@ -898,7 +1015,8 @@ cudaError_t launch_step_linear(int lin, StepArgs &a, StepLin &w, cudaStream_t st
     w.k_tiles = w.K / KT;
     w.katoms = mk_slice_atoms(lin, w.K);
     w.ks = w.k_tiles / w.katoms;
-    w.ring_atoms = lin_ring(a.bn, a.pd.M, w.katoms, ad, ad ? (lin == 2 ? 2 : 1) * a.dm.r : 0);
+    size_t smem = 0;
+    w.ring_atoms = lin_ring(a.bn, a.pd.M, w.katoms, w.ks, ad, ad ? (lin == 2 ? 2 : 1) * a.dm.r : 0, &w.push, &smem);
     if (w.ring_atoms == 0 || w.ks > ST_MAX_CLUSTER) return cudaErrorInvalidValue;
     w.tmem_cols = 32;
     while ((int)w.tmem_cols < (ad ? 2 : 1) * a.bn) w.tmem_cols <<= 1;
@@ -906,30 +1024,33 @@ cudaError_t launch_step_linear(int lin, StepArgs &a, StepLin &w, cudaStream_t st
         if (!encode_bf16_map(&w.xmap, lin == 1 ? (const void *)a.attn : (const void *)a.act, a.rows_alloc, w.K, a.bn))
             return cudaErrorInvalidValue;
     const dim3 grid(w.n_main / TILE_ROWS, w.ks);
-    const size_t smem = lin_smem(a.bn, w.ring_atoms, ad);
-    return a.dm.d == 128 ? launch_lin<128>(lin, ad, grid, smem, a, w, st) : launch_lin<64>(lin, ad, grid, smem, a, w, st);
+    if (lin_threads(a.pd.M) == 256)
+        return a.dm.d == 128 ? launch_lin<128, 256>(lin, ad, grid, smem, a, w, st) : launch_lin<64, 256>(lin, ad, grid, smem, a, w, st);
+    return a.dm.d == 128 ? launch_lin<128, 512>(lin, ad, grid, smem, a, w, st) : launch_lin<64, 512>(lin, ad, grid, smem, a, w, st);
 }
 
 template <int DH, bool BLK>
-static cudaError_t launch_attn(const StepArgs &a, const CUtensorMap &kmap, const CUtensorMap &vmap, int layer, int nsplit,
-                               cudaStream_t st) {
-    int bufs, parts;
-    const int cs = attn_cluster(a.dm, a.pd, a.att_subs, nsplit, &bufs, &parts);
+static cudaError_t launch_attn(const StepArgs &a, const CUtensorMap &kmap, const CUtensorMap &vmap, int layer,
+                               const StepSplits &sp, cudaStream_t st) {
+    int nsplit = 0;
+    for (int b = 0; b < a.pd.nb; ++b) nsplit = std::max(nsplit, sp.start[b + 1] - sp.start[b]);
+    size_t smem;
+    const int cs = attn_cluster(a.dm, a.pd, a.att_subs, nsplit, &smem);
     if (cs > 0)
-        return launch_step(k_step_attn<DH, BLK, true>, dim3(cs, a.dm.Hkv, a.pd.nb), dim3(cs), 32 * SA_WARPS + 32,
-                           attn_smem(a.dm, a.pd.R, bufs, parts), st, kmap, vmap, a, layer, bufs, parts);
-    cudaError_t e = launch_step(k_step_attn<DH, BLK, false>, dim3(nsplit, a.dm.Hkv, a.pd.nb), dim3(1), 32 * SG_WARPS + 32,
-                                attn_smem(a.dm, a.pd.R, 1, 0), st, kmap, vmap, a, layer, 1, 0);
+        return launch_step(k_step_attn<DH, BLK, true>, dim3(cs, a.dm.Hkv, a.pd.nb), dim3(cs), 32 * SA_WARPS + 32, smem, st,
+                           kmap, vmap, a, layer, nsplit * a.att_subs, sp);
+    cudaError_t e = launch_step(k_step_attn<DH, BLK, false>, dim3(sp.start[a.pd.nb], a.dm.Hkv), dim3(1), 32 * SG_WARPS + 32,
+                                attn_smem(a.dm, a.pd.R, 0, 0), st, kmap, vmap, a, layer, 0, sp);
     if (e != cudaSuccess) return e;
-    return launch_pdl(k_step_merge<DH>, (a.pd.M * a.dm.Hq + 7) / 8, 256, 0, st, a);
+    return launch_pdl(k_step_merge<DH>, a.pd.M * a.dm.Hq, DH, 0, st, a);
 }
 
-cudaError_t launch_step_attn(const StepArgs &a, const CUtensorMap &kmap, const CUtensorMap &vmap, int layer, int nsplit,
-                             cudaStream_t st) {
+cudaError_t launch_step_attn(const StepArgs &a, const CUtensorMap &kmap, const CUtensorMap &vmap, int layer,
+                             const StepSplits &sp, cudaStream_t st) {
     const bool blk = a.pd.mask_mode == MASK_BLOCK_DRAFT;
     if (a.dm.d == 128)
-        return blk ? launch_attn<128, true>(a, kmap, vmap, layer, nsplit, st) : launch_attn<128, false>(a, kmap, vmap, layer, nsplit, st);
-    return blk ? launch_attn<64, true>(a, kmap, vmap, layer, nsplit, st) : launch_attn<64, false>(a, kmap, vmap, layer, nsplit, st);
+        return blk ? launch_attn<128, true>(a, kmap, vmap, layer, sp, st) : launch_attn<128, false>(a, kmap, vmap, layer, sp, st);
+    return blk ? launch_attn<64, true>(a, kmap, vmap, layer, sp, st) : launch_attn<64, false>(a, kmap, vmap, layer, sp, st);
 }
 
 cudaError_t launch_step_embed(const StepArgs &a, const void *embed_tiled, const void *mask_embed, cudaStream_t st) {
@@ -947,16 +1068,24 @@ cudaError_t configure_step_kernels() {
     auto set = [&](const void *f) {
         if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, ST_SMEM);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        // an SM changes its split of shared memory and L1 only when it is empty: with one split for all steps a
+        // step's CTAs can start beside the one before
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     };
-#define STEP_SET(L)                               \
-    set((const void *)k_step_linear<L, true, 128>);  \
-    set((const void *)k_step_linear<L, false, 128>); \
-    set((const void *)k_step_linear<L, true, 64>);   \
-    set((const void *)k_step_linear<L, false, 64>)
-    STEP_SET(0);
-    STEP_SET(1);
-    STEP_SET(2);
-    STEP_SET(3);
+#define STEP_SET(L, NT)                                  \
+    set((const void *)k_step_linear<L, true, 128, NT>);  \
+    set((const void *)k_step_linear<L, false, 128, NT>); \
+    set((const void *)k_step_linear<L, true, 64, NT>);   \
+    set((const void *)k_step_linear<L, false, 64, NT>)
+    STEP_SET(0, 256);
+    STEP_SET(1, 256);
+    STEP_SET(2, 256);
+    STEP_SET(3, 256);
+    STEP_SET(0, 512);
+    STEP_SET(1, 512);
+    STEP_SET(2, 512);
+    STEP_SET(3, 512);
 #undef STEP_SET
 #define STEP_SET(DH, BLK)                            \
     set((const void *)k_step_attn<DH, BLK, true>);   \
@@ -966,6 +1095,10 @@ cudaError_t configure_step_kernels() {
     STEP_SET(64, true);
     STEP_SET(64, false);
 #undef STEP_SET
+    for (const void *f : {(const void *)k_step_merge<128>, (const void *)k_step_merge<64>, (const void *)k_step_embed,
+                          (const void *)k_step_final})
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     return e;
 }
 

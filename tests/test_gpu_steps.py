@@ -1,0 +1,98 @@
+"""Decoding passes as kernel chains against the persistent pass kernel (which max_ctas selects), bit for
+bit: draft, verify and plain-decoding logits, accepted lengths and cached K/V, over block sizes, batch
+sizes, head layouts, context lengths (one cluster per group; partial results in memory), draft variants
+and adapter ranks."""
+import dataclasses
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def torch():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    return torch
+
+
+def _shape(name):
+    from paper_2607_12422_gb300 import synth
+    two = dataclasses.replace(synth.QWEN3_0_6B, n_layers=2, vocab=2048)
+    return {
+        "tiny": synth.TINY,
+        "qwen2": two,
+        "grp4": dataclasses.replace(two, n_kv_heads=4, hidden=768, intermediate=1280),
+        "grp1-d64": dataclasses.replace(synth.TINY, n_q_heads=8, n_kv_heads=8, hidden=512, intermediate=512, vocab=1024),
+        "r8": dataclasses.replace(two, lora_rank=8, lora_alpha=16.0),
+    }[name]
+
+
+CASES = [
+    # shape, D, prompt lengths, max_seq, engine options
+    ("tiny", 16, (64,), 256, {}),
+    ("tiny", 1, (1,), 64, {}),
+    ("qwen2", 16, (512,), 640, {}),
+    ("qwen2", 32, (200,), 320, {}),
+    ("qwen2", 64, (30,), 256, {}),
+    ("qwen2", 4, (1100,), 1400, {}),
+    ("qwen2", 16, (128, 127, 129), 400, {}),
+    ("qwen2", 16, (700, 40, 333, 512, 90, 1, 600, 257), 900, {}),
+    ("qwen2", 31, (50, 60, 70, 80, 90, 100, 110, 120), 320, {}),  # 256 rows
+    ("qwen2", 16, (300,), 400, dict(draft_layers=1)),
+    ("qwen2", 16, (300, 20), 400, dict(draft_skip=1, denoise_steps=2, anchored=False)),
+    ("grp4", 16, (333, 40), 500, {}),
+    ("grp1-d64", 8, (150, 33), 300, {}),
+    ("r8", 16, (140,), 300, {}),
+]
+
+
+@pytest.mark.parametrize("shape,D,lens,max_seq,opt", CASES, ids=lambda v: str(v).replace(" ", "")[:40])
+def test_kernel_chain_equals_persistent_kernel(torch, shape, D, lens, max_seq, opt):
+    from paper_2607_12422_gb300 import pbd, synth
+    S = _shape(shape)
+    base, ad = synth.with_random_norm_gains(synth.gen_base_weights(S)), synth.gen_adapter(S)
+    rng = np.random.default_rng(D + sum(lens))
+    prompts = [rng.integers(0, S.vocab, n).astype(np.int32) for n in lens]
+    rounds = 3
+    drafts = rng.integers(0, S.vocab, (rounds, len(lens), D)).astype(np.int32)
+    forced = rng.integers(0, D + 1, (rounds, len(lens))).astype(np.int32)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    got = []
+    for ctas in (0, sms):
+        eng = pbd.Engine(S, base, ad, block_D=D, max_batch=len(lens), max_seq_len=max_seq, max_ctas=ctas, **opt)
+        out = [eng.pbd_prefill(prompts, max_new=rounds * (D + 1) + 4)]
+        for r in range(rounds):  # (the third round replays the chains as graphs)
+            d_ids, d_lg = eng.pbd_draft_block(want_logits=True)
+            v_ids, v_lg = eng.pbd_verify_block(drafts=drafts[r], want_logits=True)
+            out += [d_ids, d_lg, v_ids, v_lg, eng.pbd_accept_commit(forced_n=forced[r])]
+        for _ in range(3):
+            out += list(eng.pbd_decode_step(want_logits=True))
+        L = [int(x) for x in eng.pbd_get_state()[0]]
+        for b in range(len(lens)):
+            for l in range(S.n_layers):
+                out += list(eng.pbd_read_kv(l, b, L[b]))
+        got.append((L, [t.clone() for t in out]))
+        eng.close()
+    assert got[0][0] == got[1][0]
+    for i, (x, y) in enumerate(zip(got[0][1], got[1][1])):
+        assert torch.equal(x, y), i
+
+
+def test_graphs_follow_the_generation(torch):
+    """One engine, generations of other batch and prompt sizes in turn: chains and their graphs are those of the
+    current generation, not of the one before."""
+    from paper_2607_12422_gb300 import pbd, synth
+    S = _shape("qwen2")
+    base, ad = synth.gen_base_weights(S), synth.gen_adapter(S)
+    rng = np.random.default_rng(2)
+    eng = pbd.Engine(S, base, ad, block_D=8, max_batch=3, max_seq_len=900)
+    for lens in ((40,), (700, 30, 300), (40,), (300, 30), (820,)):
+        prompts = [rng.integers(0, S.vocab, n).astype(np.int32) for n in lens]
+        spec, _ = eng.pbd_generate(prompts, 24, mode=0)
+        eng.pbd_prefill(prompts, max_new=24)
+        toks = [eng.pbd_decode_step()[0].clone() for _ in range(23)]
+        assert torch.equal(spec[:, 1:], torch.stack(toks, 1)), lens
+    eng.close()
