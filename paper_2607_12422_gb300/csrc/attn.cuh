@@ -1,5 +1,5 @@
-// attn.cuh -- tensor-core steps of the attention, shared by the pass kernel and the many-row kernel (their
-// results must agree bit for bit).
+// attn.cuh -- tensor-core steps of the attention, shared by the pass kernel and the decoding chain (their
+// results must agree bit for bit, and with rows.cu's).
 //
 // Staged K and V: DH / 64 sub-tiles of [128 keys x 128 bytes] in the 128-byte swizzle layout (16-byte
 // chunk c of key n at (c ^ (n & 7)) * 16), as the tiled TMA writes them, 1024-byte aligned.  The key

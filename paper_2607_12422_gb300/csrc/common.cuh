@@ -115,23 +115,42 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
     return ok != 0;
 }
 
+__device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
 // Bounded wait on one phase of an mbarrier.  Returns false (and latches `code`) after
-// WAIT_LIMIT_NS, or as soon as *abort is set by another thread of the CTA.
+// WAIT_LIMIT_NS, or as soon as *abort is set by another thread of the CTA.  The clock is not read
+// before a first stretch of polls has failed: a read of the global timer holds a warp up for as long as
+// most waits last.
 __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, int *status, int code,
                                           volatile int *abort) {
     const uint32_t a = smem_u32(bar);
-    if (mbar_try_wait(a, parity)) return true;
-    const uint64_t t0 = globaltimer_ns();
-    for (;;) {
-        for (int i = 0; i < 32; ++i)
-            if (mbar_try_wait(a, parity)) return true;
-        if (abort && *abort) return false;
-        if (globaltimer_ns() - t0 > WAIT_LIMIT_NS) {
-            latch_error(status, code);
-            if (abort) *abort = 1;
-            return false;
+    bool ok = false;
+#pragma unroll 1
+    for (int i = 0; i < 256 && !ok; ++i) ok = mbar_try_wait(a, parity);
+    if (!ok) {
+        const uint64_t t0 = globaltimer_ns();
+        for (;;) {
+#pragma unroll 1
+            for (int i = 0; i < 32 && !ok; ++i) ok = mbar_try_wait(a, parity);
+            if (ok || (abort && *abort)) break;
+            if (globaltimer_ns() - t0 > WAIT_LIMIT_NS) {
+                latch_error(status, code);
+                if (abort) *abort = 1;
+                break;
+            }
         }
     }
+    return ok;
 }
 
 // ------------------------------------------------------------------ TMA
@@ -235,6 +254,21 @@ __device__ __forceinline__ uint64_t sw128_kmajor_desc(const void *smem_tile) {
     return d;
 }
 
+// The same for an operand with N contiguous (MN-major; bit 16 of the instruction descriptor for B): a row of 128
+// bytes is 64 values of one k, 8 of them an atom.  Leading byte offset: to the next 64 of N; stride byte
+// offset: to the next 8 of K (1024 B).
+__device__ __forceinline__ uint64_t sw128_mnmajor_desc(const void *smem_tile, uint32_t next64) {
+    const uint64_t addr = smem_u32(smem_tile);
+    uint64_t d = 0;
+    d |= (addr >> 4) & 0x3FFFull;
+    d |= (uint64_t)(next64 >> 4) << 16;
+    d |= (uint64_t)(1024 >> 4) << 32;
+    d |= 1ull << 46;
+    d |= 2ull << 61;
+    return d;
+}
+constexpr uint32_t IDESC_B_MN = 1u << 16;
+
 // Instruction descriptor for kind::f16 with bf16 A/B, fp32 accumulator, both K-major.
 //   bits 4-5: D format (1 = f32); 7-9: A format (1 = bf16); 10-12: B format (1 = bf16);
 //   bit 15/16: A/B major (0 = K); 17-22: N >> 3; 24-28: M >> 4.
@@ -250,6 +284,16 @@ __device__ __forceinline__ void mma_bf16_ss(uint32_t tmem_d, uint64_t adesc, uin
         "setp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
         "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+
+// The same with A in tensor memory: lane = row, a 32-bit column two of its bf16 values along K (8 columns a step).
+__device__ __forceinline__ void mma_bf16_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(tmem_d),
+        "r"(tmem_a), "l"(bdesc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
 
@@ -298,6 +342,56 @@ __device__ __forceinline__ float warp_max(float v, int *lane_of) {
     asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(m) : "f"(v));
     *lane_of = __ffs(__ballot_sync(0xffffffffu, v == m)) - 1;
     return m;
+}
+
+// Each thread of the warp writes 16 / 32 consecutive 32-bit columns of its TMEM lane.
+__device__ __forceinline__ void tmem_st_16cols(uint32_t taddr, const uint32_t (&v)[16]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+        "%16};" ::"r"(taddr),
+        "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]), "r"(v[9]),
+        "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15])
+        : "memory");
+}
+__device__ __forceinline__ void tmem_st_32cols(uint32_t taddr, const uint32_t (&v)[32]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};" ::"r"(taddr),
+        "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]), "r"(v[9]),
+        "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]), "r"(v[16]), "r"(v[17]), "r"(v[18]),
+        "r"(v[19]), "r"(v[20]), "r"(v[21]), "r"(v[22]), "r"(v[23]), "r"(v[24]), "r"(v[25]), "r"(v[26]), "r"(v[27]),
+        "r"(v[28]), "r"(v[29]), "r"(v[30]), "r"(v[31])
+        : "memory");
+}
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
+// ------------------------------------------------------------------ packed fp32
+
+// Two floats; each half is rounded as __fadd_rn and __fmul_rn round.  A product that is then added to is made
+// by mul2: of mul.rn.f32x2 and add.rn.f32x2 the compiler makes one fused operation, with another last bit.
+struct F2 {
+    unsigned long long v;
+};
+__device__ __forceinline__ F2 f2(float x, float y) {
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ F2 mulp2(F2 a, F2 b) {
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 mul2(float s, float x, float y) { return f2(__fmul_rn(s, x), __fmul_rn(s, y)); }
+__device__ __forceinline__ F2 add2(F2 a, F2 b) {
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(F2 a) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a.v));
+    return r;
 }
 
 // ------------------------------------------------------------------ legacy warp MMA (attention)

@@ -229,299 +229,427 @@ __global__ void __launch_bounds__(RW_THREADS) k_rows_rope(const __grid_constant_
 
 // ------------------------------------------------------------------ attention
 //
-// One CTA: 128 (row, head) pairs of one sequence's segment and KV head, 16 per compute warp, against
-// the cached keys up to the last row's position, in the pass kernel's partition: 128-key splits, each
-// one or two partial results of HALF keys computed in 32-key chunks with a running maximum, combined
-// in key order relative to the row's overall maximum.  The pass kernel stores the partial
-// results and merges them afterwards; here a first sweep over the keys finds the overall maximum
-// (scores only), and the second sweep computes each partial result and adds it to the row's sums
-// at once, in registers.  One more QK^T per key replaces 520 bytes of partial results written
-// and read back per (row, head, partial).
+// One CTA: 128 (row, head) pairs of one sequence's segment and KV head against the cached keys up to the last
+// row's position, in the pass kernel's partition: 128-key splits, each one or two partial results of HALF
+// keys computed in 32-key chunks with a running maximum, combined in key order relative to the row's
+// overall maximum.  The pass kernel stores the partial results and merges them afterwards; here a first
+// sweep over the keys finds the overall maximum (scores only), and the second sweep computes each partial
+// result and adds it to the row's sums at once, in registers.  One more QK^T per key replaces 520 bytes
+// of partial results written and read back per (row, head, partial).
 //
-// Warp 8 streams units of 128 keys of K (first sweep) or K, then V (second) into a ring: one tiled
-// TMA per 16-token page and 64-dim half.
+// Scores and P V are tcgen05 MMAs: over one K range and in one order of K steps their fp32 sums came out bit for bit
+// as mma.sync's (0 of 1.3 M sums differed, over normal, wide-range and probability operands), so the results
+// stay the decoding passes'.  Columns of tensor memory: scores of 64-key units [0, 256) in the first
+// sweep (four buffers) and [0, 128) in the second (two), P over the scores that it came from (bf16, the A
+// operand), the partial result [128, 256).
 //
-// Bound: latency of legacy mma.sync in two warps per SM quarter (4096 rows: 352 us a layer; 497 us with
-// the scores' MMAs in one chain after another and swizzled addresses computed per fragment; 387 us
-// as two CTAs of four warps).  The tcgen05 tensor core is not used because its summation order
-// differs from the decoding pass's.
-constexpr int RA_WARPS = 8;
-constexpr int RA_THREADS = 32 * RA_WARPS + 128;  // the producer's warpgroup has one warp with work
-constexpr int RA_UNITS = 4;
+// Roles: warps 0-3 one thread per pair (scores to probabilities, running rescale, sums); warp 4 streams K, then K
+// and V, one tiled TMA per 16-token page and 64-dim half; warp 5 issues the MMAs.  One tile keeps the tensor core
+// waiting for the softmax and the other way round, so two CTAs share an SM.  The first sweep runs from the
+// last unit to the first: the scores of units 0 and 1 are then still there for the second.
+//
+// Bound: a 32-key chunk is a chain of ~1600 cycles (scores out of tensor memory and to probabilities 620, waits
+// 180, rescale or merge 500, P back and handed over 190); two CTAs fill 56% of the issue slots and 28% of
+// the tensor core's time.  4096 rows of the 0.6B shape: 165 us a layer; 352 with mma.sync, whose own rate
+// would take 176.  725 rows: 34 us against 41.
+constexpr int RA_PAIRS = 128;
+constexpr int RA_KEYS = 64;      // keys of a unit
+constexpr int RA_RING = 4;       // units of K or V in flight
+constexpr int RA_THREADS = 256;  // (the second warpgroup has two warps with work)
 
 template <int DH>
 struct RaLayout {
-    static constexpr int SUB = ATT_SPLIT * 128;  // 128 keys x 64 dims, 128-byte swizzle
+    static constexpr int SUB = RA_KEYS * 128;  // 64 keys x 64 dims, 128-byte swizzle
     static constexpr int UNIT = (DH / 64) * SUB;
-    static constexpr int TOTAL = RA_UNITS * UNIT + 1024;
+    static constexpr int QSUB = RA_PAIRS * 128;
+    static constexpr int Q = (DH / 64) * QSUB;
+    static constexpr int TOTAL = Q + RA_RING * UNIT + 1024;
+};
+
+// ring units of an item of nu units of keys
+__device__ __forceinline__ int ra_units(int nu) { return 2 * nu + max(nu - 2, 0); }
+
+struct RaState {
+    uint64_t full[RA_RING], empty[RA_RING];  // ring
+    uint64_t qfull, qfree;                     // q's place filled, given up
+    uint64_t sfull1[4], sempty[4], sfull2[2];  // scores: first sweep, second sweep
+    uint64_t pfull, pvdone;                    // P of a chunk stored, its P V done
+    uint64_t fin;
+    uint32_t tmem_slot;
+    int abort;
 };
 
 template <int DH>
-__global__ void __launch_bounds__(RA_THREADS, 1)
+__global__ void __launch_bounds__(RA_THREADS, 2)
     k_rows_attn(const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap vmap,
                 const __grid_constant__ RowsArgs a, int layer, const RowsAttn *__restrict__ work, int n_work) {
     using LY = RaLayout<DH>;
-    constexpr int KS = DH / 16, DT = DH / 8, SUBS = DH / 64;
+    constexpr int KS = DH / 16, SUBS = DH / 64;
     extern __shared__ uint8_t smem_raw[];
-    uint8_t *ring = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    __shared__ uint64_t full[RA_UNITS], empty[RA_UNITS];
-    __shared__ int s_abort;
+    uint8_t *sQ = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint8_t *ring = sQ + LY::Q;
+    __shared__ RaState S;
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const Dims &dm = a.dm;
     const int grp = dm.Hq / dm.Hkv;
     if (threadIdx.x == 0) {
-        for (int i = 0; i < RA_UNITS; ++i) {
-            mbar_init(&full[i], 1);
-            mbar_init(&empty[i], RA_WARPS);
+        for (int i = 0; i < RA_RING; ++i) {
+            mbar_init(&S.full[i], 1);
+            mbar_init(&S.empty[i], 1);
         }
-        s_abort = 0;
+        mbar_init(&S.qfull, RA_PAIRS);
+        mbar_init(&S.qfree, RA_PAIRS);
+        for (int i = 0; i < 4; ++i) {
+            mbar_init(&S.sfull1[i], 1);
+            mbar_init(&S.sempty[i], RA_PAIRS / 32);
+        }
+        mbar_init(&S.sfull2[0], 1);
+        mbar_init(&S.sfull2[1], 1);
+        mbar_init(&S.pfull, RA_PAIRS / 32);
+        mbar_init(&S.pvdone, 1);
+        mbar_init(&S.fin, 1);
+        S.abort = 0;
         fence_mbarrier_init();
         prefetch_tensormap(&kmap);
         prefetch_tensormap(&vmap);
     }
+    if (warp == 4) tmem_alloc(&S.tmem_slot, 256);
+    tc_fence_before();
     __syncthreads();
-    pdl_begin();
-    int slot = 0;
-    // registers: the producer's warpgroup gives up 128 x 128 of the launch's 3 x 128 x 168, the two
-    // compute warpgroups take 128 x 56 each
-    if (warp >= RA_WARPS) {
+    tc_fence_after();
+    const uint32_t tmem = S.tmem_slot, tmem_o = tmem + 128;
+    // (the work list was uploaded before the pass's first kernel)
+    if (warp < 6 && blockIdx.x < n_work) {
+        const RowsAttn *wk = work + blockIdx.x;
+        asm volatile("prefetch.global.L1 [%0];" ::"l"(wk));
+        asm volatile("prefetch.global.L1 [%0];" ::"l"(a.segs + wk->seg));
+    }
+    pdl_begin();  // (after the allocation: a later kernel's CTA never holds TMEM that this one waits for)
+    // an item's last visible key; keys of later pages are not loaded
+    auto last_key = [&](const RowsAttn &wk, const RowSeg &sg) { return sg.pos0 + min(sg.n - 1, (wk.q0 + RA_PAIRS - 1) / grp); };
+    const int HALF = ATT_SPLIT / a.att_subs;
+
+    // registers: of the launch's 2 x 128 x 128 the second warpgroup keeps 128 x 40, the first takes 128 x 216
+    if (warp >= 4) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
-        if (warp > RA_WARPS) return;
-        // ---- producer warp: a lane per page and half
-        uint32_t ph = 1;
-        int issued = 0;
+        if (warp == 4) {
+            // ---- producer warp: a lane per page and half
+            int issued = 0;
+            bool ok = true;
+            // this pass's own K/V were written by generic stores of an earlier kernel
+            fence_proxy_async_global();
+            for (int w = blockIdx.x; ok && w < n_work; w += gridDim.x) {
+                const RowsAttn wk = work[w];
+                const RowSeg sg = a.segs[wk.seg];
+                const int last = last_key(wk, sg), nu = last / RA_KEYS + 1;
+                for (int i = 0; i < ra_units(nu); ++i) {  // K of every unit, last to first; then V 0, V 1, K 2, V 2, K 3, V 3 ...
+                    const int j = i - nu, slot = issued % RA_RING;
+                    const bool v = j == 0 || (j > 0 && (j & 1));
+                    const int u = j < 0 ? nu - 1 - i : (v ? (j + 1) >> 1 : (j >> 1) + 1);
+                    if (!mbar_wait(&S.empty[slot], ((issued / RA_RING) & 1) ^ 1, a.status, DEV_TIMEOUT_SLOT, &S.abort)) ok = false;
+                    if (!(ok = __all_sync(0xffffffffu, ok))) break;
+                    const int npg = min(RA_KEYS / PAGE, last / PAGE - u * (RA_KEYS / PAGE) + 1);
+                    if (lane == 0) mbar_arrive_expect_tx(&S.full[slot], (uint32_t)(npg * SUBS * PAGE * 128));
+                    __syncwarp();
+                    if (lane < npg * SUBS) {
+                        const int p = lane / SUBS, sub = lane % SUBS;
+                        const int page = a.kv.page_table[sg.seq * a.kv.pages_per_seq + u * (RA_KEYS / PAGE) + p];
+                        tma_load_2d(ring + slot * LY::UNIT + sub * LY::SUB + p * PAGE * 128, v ? &vmap : &kmap, sub * 64,
+                                    ((layer * a.kv.n_pages + page) * dm.Hkv + wk.g) * PAGE, &S.full[slot]);
+                    }
+                    ++issued;
+                }
+            }
+            if (*(volatile int *)&S.abort)  // error path: the copies in flight get a bounded chance to land
+                for (int h = issued > RA_RING ? issued - RA_RING : 0; h < issued; ++h)
+                    mbar_wait(&S.full[h % RA_RING], (h / RA_RING) & 1, nullptr, 0, nullptr);
+        } else if (warp == 5 && elect_one()) {
+            // ---- MMA warp
+            const uint32_t ids = idesc_bf16_f32(128, RA_KEYS), ido = idesc_bf16_f32(128, DH) | IDESC_B_MN;
+            const uint64_t qd = sw128_kmajor_desc(sQ);
+            int used = 0;  // ring units
+            uint32_t ph = 0;  // phase bits: 0-3 sempty, 4 pfull, 5 qfull
+            bool ok = true;
+            auto wait = [&](uint64_t *bar, int bit) {
+                ok = ok && mbar_wait(bar, (ph >> bit) & 1u, a.status, DEV_TIMEOUT_MMA, &S.abort);
+                ph ^= 1u << bit;
+                return ok;
+            };
+            auto unit = [&]() {  // the next ring unit, once it has landed
+                const int slot = used % RA_RING;
+                ok = ok && mbar_wait(&S.full[slot], (used / RA_RING) & 1, a.status, DEV_TIMEOUT_LOAD, &S.abort);
+                ++used;
+                return slot;
+            };
+            auto scores = [&](uint32_t col, uint64_t *bar) {
+                const int slot = unit();
+                if (!ok) return;
+                tc_fence_after();
+                const uint64_t kd = sw128_kmajor_desc(ring + slot * LY::UNIT);
+#pragma unroll
+                for (int ks = 0; ks < KS; ++ks)
+                    mma_bf16_ss(tmem + col, qd + (uint64_t)((ks >> 2) * LY::QSUB / 16 + 2 * (ks & 3)),
+                                kd + (uint64_t)((ks >> 2) * LY::SUB / 16 + 2 * (ks & 3)), ids, ks != 0);
+                mma_commit(&S.empty[slot]);
+                mma_commit(bar);
+            };
+            for (int w = blockIdx.x; ok && w < n_work; w += gridDim.x) {
+                const RowsAttn wk = work[w];
+                const RowSeg sg = a.segs[wk.seg];
+                const int last = last_key(wk, sg), nu = last / RA_KEYS + 1;
+                if (!wait(&S.qfull, 5)) break;
+                for (int u = nu - 1; ok && u >= 0; --u) {
+                    if (u + 4 < nu) wait(&S.sempty[u & 3], u & 3);
+                    scores((u & 3) * RA_KEYS, &S.sfull1[u & 3]);
+                }
+                for (int u = 0; ok && u < min(nu, 4); ++u) wait(&S.sempty[u & 3], u & 3);
+                for (int u = 0; ok && u < nu; ++u) {
+                    int vslot = 0;
+                    for (int cc = 0; cc < 2; ++cc) {
+                        const int k = u * RA_KEYS + cc * 32;
+                        if (k > last) break;
+                        // (every thread of the softmax saw the P V before this one done: the other scores'
+                        // columns are free)
+                        if (!wait(&S.pfull, 4)) break;
+                        if (cc == 0) vslot = unit();
+                        if (!ok) break;
+                        tc_fence_after();
+                        const uint64_t vd = sw128_mnmajor_desc(ring + vslot * LY::UNIT, LY::SUB);
+#pragma unroll
+                        for (int j = 0; j < 2; ++j)
+                            if (k + j * PAGE <= last)
+                                mma_bf16_ts(tmem_o, tmem + (u & 1) * RA_KEYS + cc * 32 + j * 8,
+                                            vd + (uint64_t)((cc * 2 + j) * PAGE * 128 >> 4), ido, j != 0 || (k & (HALF - 1)) != 0);
+                        mma_commit(&S.pvdone);
+                        if (cc == 0 && u >= 1 && u + 1 < nu) scores(((u + 1) & 1) * RA_KEYS, &S.sfull2[(u + 1) & 1]);
+                    }
+                    if (ok) mma_commit(&S.empty[vslot]);
+                }
+            }
+            mma_commit(&S.fin);  // also on the error path: every MMA issued completes before TMEM goes
+            mbar_wait(&S.fin, 0, nullptr, 0, nullptr);
+        }
+    } else {
+        // ---- softmax: thread t the pair q0 + t (tensor memory lane t)
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 216;");
+        const uint32_t tl = tmem + ((uint32_t)(warp * 32) << 16), to = tl + 128;
+        const float scale = a.att_scale;
+        uint32_t ph = 0;  // phase bits: 0-3 sfull1, 4-5 sfull2, 6 pvdone, 7 qfree
+        int units = 0;    // ring units before this item's
+        auto wait = [&](uint64_t *bar, int bit) {
+            bool ok = false;
+            for (int t = 0; t < 4096 && !ok; ++t) ok = mbar_test_wait(smem_u32(bar), (ph >> bit) & 1u);
+            if (!ok) ok = mbar_wait(bar, (ph >> bit) & 1u, a.status, DEV_TIMEOUT_MMA, &S.abort);
+            ph ^= 1u << bit;
+            return __all_sync(0xffffffffu, ok) != 0;
+        };
         bool ok = true;
-        // this pass's own K/V were written by generic stores of an earlier kernel
-        fence_proxy_async_global();
         for (int w = blockIdx.x; ok && w < n_work; w += gridDim.x) {
             const RowsAttn wk = work[w];
             const RowSeg sg = a.segs[wk.seg];
-            const int last = sg.pos0 + min(sg.n - 1, (wk.q0 + 16 * RA_WARPS - 1) / grp);  // last visible key
-            const int ns = last / ATT_SPLIT + 1;
-            for (int u = 0; u < 3 * ns; ++u) {  // K of every split, then K and V of every split
-                const int s = u < ns ? u : (u - ns) >> 1;
-                const bool v = u >= ns && ((u - ns) & 1);
-                if (!mbar_wait(&empty[slot], ph, a.status, DEV_TIMEOUT_SLOT, &s_abort)) {
-                    ok = false;
-                    break;
+            const int last = last_key(wk, sg), nu = last / RA_KEYS + 1, T = sg.pos0 + sg.n, QV = sg.n * grp;
+            if (w != blockIdx.x && !(ok = wait(&S.qfree, 7))) break;  // (the last item's sums were staged there)
+            for (int q = threadIdx.x; q < RA_PAIRS * (DH / 8); q += RA_PAIRS) {
+                const int r = q / (DH / 8), c = q % (DH / 8), qv = wk.q0 + r;
+                if (qv < QV)
+                    cp_async16(sQ + (c >> 3) * LY::QSUB + r * 128 + (((c & 7) ^ (r & 7)) << 4),
+                               a.q + ((size_t)(sg.row0 + qv / grp) * dm.Hq + wk.g * grp + qv % grp) * DH + c * 8);
+            }
+            cp_async_commit();
+            cp_async_wait_all();
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            mbarrier_arrive_one(&S.qfull);
+            const int qv = wk.q0 + threadIdx.x;
+            const bool val = qv < QV;
+            const int i = val ? qv / grp : 0, h = wk.g * grp + (val ? qv % grp : 0);
+            const int lim = val ? sg.pos0 + i : -1;  // last visible key
+            // the warp's last visible key (-1: no pairs), and the last key that all its pairs see
+            const int wq0 = wk.q0 + warp * 32;
+            const int wlast = wq0 < QV ? sg.pos0 + min(sg.n - 1, (wq0 + 31) / grp) : -1;
+            const int wall = wq0 + 31 < QV ? sg.pos0 + wq0 / grp : -1;
+            // first sweep: the largest score (the scale is positive and rounding is monotonic, so the
+            // largest scaled score is the scaled largest score)
+            float x = -INFINITY;
+            for (int u = nu - 1; u >= 0; --u) {
+                if (!(ok = wait(&S.sfull1[u & 3], u & 3))) break;
+                tc_fence_after();
+                const int k0 = u * RA_KEYS;
+#pragma unroll 1
+                for (int k = k0; k < k0 + RA_KEYS && k <= wlast; k += 32) {
+                    uint32_t v[32];
+                    tmem_ld_32cols(tl + (u & 3) * RA_KEYS + (k - k0), v);
+                    tmem_ld_wait();
+                    float y[4] = {x, x, x, x};
+                    if (k + 31 <= wall) {
+#pragma unroll
+                        for (int e = 0; e < 32; ++e) y[e & 3] = fmaxf(y[e & 3], __uint_as_float(v[e]));
+                    } else {
+#pragma unroll
+                        for (int e = 0; e < 32; ++e) y[e & 3] = fmaxf(y[e & 3], k + e <= lim ? __uint_as_float(v[e]) : -INFINITY);
+                    }
+                    x = fmaxf(fmaxf(y[0], y[1]), fmaxf(y[2], y[3]));
                 }
-                const int npg = min(ATT_SPLIT / PAGE, last / PAGE - s * (ATT_SPLIT / PAGE) + 1);
-                if (lane == 0) mbar_arrive_expect_tx(&full[slot], (uint32_t)(npg * SUBS * PAGE * 128));
+                tc_fence_before();
                 __syncwarp();
-                if (lane < npg * SUBS) {
-                    const int p = lane / SUBS, sub = lane % SUBS;
-                    const int page = a.kv.page_table[sg.seq * a.kv.pages_per_seq + s * (ATT_SPLIT / PAGE) + p];
-                    tma_load_2d(ring + (size_t)slot * LY::UNIT + sub * LY::SUB + p * PAGE * 128, v ? &vmap : &kmap, sub * 64,
-                                ((layer * a.kv.n_pages + page) * dm.Hkv + wk.g) * PAGE, &full[slot]);
-                }
-                ++issued;
-                if (++slot == RA_UNITS) slot = 0, ph ^= 1;
+                if (lane == 0) mbarrier_arrive_one(&S.sempty[u & 3]);
+                __syncwarp();
             }
+            if (!ok) break;
+            x = __fmul_rn(x, scale);
+            // second sweep: partial results in key order, added with their weights relative to x
+            F2 num[DH / 2];
+            float den = 0.f;
+#pragma unroll
+            for (int d = 0; d < DH / 2; ++d) num[d] = f2(0.f, 0.f);
+            // running maximum and sum of the partial result; l[j]: the keys 2j, 2j + 1 (mod 8)
+            float m = -INFINITY, l[4] = {0.f, 0.f, 0.f, 0.f};
+            // (the last iteration only merges)
+#pragma unroll 1
+            for (int k = 0;; k += 32) {
+                const int u = k / RA_KEYS;
+                const uint32_t cols = tl + (u & 1) * RA_KEYS + (k & 32);
+                const bool more = k <= last, first = !more || (k & (HALF - 1)) == 0;
+                const float pm = m, pl = __fadd_rn(__fadd_rn(l[0], l[1]), __fadd_rn(l[2], l[3]));
+                bool grow = false;
+                float sc = 0.f;
+                uint32_t p[16];
+                if (more) {
+                    if (u >= 2 && (k & 32) == 0 && !(ok = wait(&S.sfull2[u & 1], 4 + (u & 1)))) break;
+                    tc_fence_after();
+                    uint32_t v[32];
+                    tmem_ld_32cols(cols, v);
+                    if (first) {
+                        m = -INFINITY;
+                        l[0] = l[1] = l[2] = l[3] = 0.f;
+                    }
+                    tmem_ld_wait();
+                    if (k + 31 > wall)
+#pragma unroll
+                        for (int e = 0; e < 32; ++e)
+                            if (k + e > lim) v[e] = 0xff800000u;  // -infinity (the scale is positive)
+                    float cm[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+                    for (int e = 0; e < 32; e += 2) {
+                        const float y0 = __fmul_rn(__uint_as_float(v[e]), scale), y1 = __fmul_rn(__uint_as_float(v[e + 1]), scale);
+                        v[e] = __float_as_uint(y0);
+                        v[e + 1] = __float_as_uint(y1);
+                        cm[(e >> 1) & 3] = fmaxf(fmaxf(cm[(e >> 1) & 3], y0), y1);
+                    }
+                    const float n = fmaxf(m, fmaxf(fmaxf(cm[0], cm[1]), fmaxf(cm[2], cm[3])));
+                    grow = __any_sync(0xffffffffu, n != m && m != -INFINITY);
+                    sc = m == -INFINITY ? 0.f : __expf(m - n);
+                    if (grow)
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) l[j] = __fmul_rn(l[j], sc);
+                    const float z = n == -INFINITY ? 0.f : n;
+                    m = n;
+#pragma unroll
+                    for (int e = 0; e < 32; e += 2) {
+                        const float p0 = __expf(__uint_as_float(v[e]) - z), p1 = __expf(__uint_as_float(v[e + 1]) - z);  // (0 if masked)
+                        l[(e >> 1) & 3] += p0;
+                        l[(e >> 1) & 3] += p1;
+                        p[e >> 1] = pack_bf162(p0, p1);
+                    }
+                }
+                if (k > 0) {
+                    if (!(ok = wait(&S.pvdone, 6))) break;
+                    tc_fence_after();
+                    if (first) {
+                        // the finished partial result joins the row's sums
+                        const float wt = __expf(pm - x);
+                        if (pl > 0.f) den = __fadd_rn(den, __fmul_rn(wt, pl));
+#pragma unroll
+                        for (int d0 = 0; d0 < DH; d0 += 32) {
+                            uint32_t o[32];
+                            tmem_ld_32cols(to + d0, o);
+                            tmem_ld_wait();
+                            if (pl > 0.f)  // (else the pair saw no key in this partial result)
+#pragma unroll
+                                for (int d = 0; d < 16; ++d)
+                                    num[d0 / 2 + d] = add2(num[d0 / 2 + d], mul2(wt, __uint_as_float(o[2 * d]), __uint_as_float(o[2 * d + 1])));
+                            __syncwarp();
+                        }
+                    } else if (grow) {
+#pragma unroll 1
+                        for (int d0 = 0; d0 < DH; d0 += 32) {
+                            uint32_t o[32];
+                            tmem_ld_32cols(to + d0, o);
+                            tmem_ld_wait();
+#pragma unroll
+                            for (int d = 0; d < 32; d += 2) {
+                                const float2 y = unpack2(mulp2(f2(__uint_as_float(o[d]), __uint_as_float(o[d + 1])), f2(sc, sc)));
+                                o[d] = __float_as_uint(y.x);
+                                o[d + 1] = __float_as_uint(y.y);
+                            }
+                            tmem_st_32cols(to + d0, o);
+                        }
+                    }
+                }
+                if (!more) break;
+                tmem_st_16cols(cols, p);
+                tmem_st_wait();
+                // V of keys at or past T in the last page: whatever the page held, so zero (0 x NaN)
+                if (warp == 0 && k + 32 > last && T % PAGE && T < (last / PAGE + 1) * PAGE) {
+                    const int vu = units + nu + max(2 * u - 1, 0);
+                    uint8_t *vs = ring + (vu % RA_RING) * LY::UNIT;
+                    ok = mbar_wait(&S.full[vu % RA_RING], (vu / RA_RING) & 1, a.status, DEV_TIMEOUT_LOAD, &S.abort);
+                    if (!(ok = __all_sync(0xffffffffu, ok))) break;
+                    const int r0 = T - u * RA_KEYS, nr = (last / PAGE + 1) * PAGE - T;
+                    for (int e = lane; e < nr * SUBS * 8; e += 32)
+                        *reinterpret_cast<uint4 *>(vs + (e / (nr * 8)) * LY::SUB + (r0 + (e / 8) % nr) * 128 + (e % 8) * 16) =
+                            make_uint4(0, 0, 0, 0);
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbarrier_arrive_one(&S.pfull);
+                __syncwarp();
+            }
+            if (!ok) break;
+            tc_fence_before();
+            units += ra_units(nu);
+            // Quotients, in a loop out of shared memory (q's place: every MMA has read it) to keep the code short: a short
+            // prompt's time is that of fetching it.  The result is the bf16 of the fp32 quotient x / den.
+            // The products of x with two numbers around 1 / den bracket that quotient (rounding is
+            // monotonic), so where both give one bf16 value it is the result; else (1 in 10^4) it is
+            // divided.  __fdiv_rn for all took 5 us a tile: its rare-case branches keep divisions from overlapping.
+            constexpr int NC = LY::Q / (RA_PAIRS * 16);  // float4 per pair that fit
+            float4 *stage = reinterpret_cast<float4 *>(sQ) + threadIdx.x;
+            bf16 *dst = a.attn + ((size_t)(sg.row0 + i) * dm.Hq + h) * DH;
+            const bool plain = den > 1e-30f && den < 1e30f;
+            const float rc = __frcp_rn(den), rlo = __fmul_rn(rc, 1.f - 0x1p-22f), rhi = __fmul_rn(rc, 1.f + 0x1p-22f);
+#pragma unroll
+            for (int d0 = 0; d0 < DH; d0 += 4 * NC) {
+#pragma unroll
+                for (int c = 0; c < NC; ++c) {
+                    const float2 y0 = unpack2(num[d0 / 2 + 2 * c]), y1 = unpack2(num[d0 / 2 + 2 * c + 1]);
+                    stage[c * RA_PAIRS] = make_float4(y0.x, y0.y, y1.x, y1.y);
+                }
+                if (val)
+#pragma unroll 1
+                    for (int c = 0; c < NC; c += 2) {
+                        const float4 y0 = stage[c * RA_PAIRS], y1 = stage[(c + 1) * RA_PAIRS];
+                        const float y[8] = {y0.x, y0.y, y0.z, y0.w, y1.x, y1.y, y1.z, y1.w};
+                        uint32_t o[4];
+                        bool same = plain;
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            o[e] = pack_bf162(__fmul_rn(y[2 * e], rlo), __fmul_rn(y[2 * e + 1], rlo));
+                            same = same && o[e] == pack_bf162(__fmul_rn(y[2 * e], rhi), __fmul_rn(y[2 * e + 1], rhi));
+                        }
+                        if (!same)
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) o[e] = pack_bf162(__fdiv_rn(y[2 * e], den), __fdiv_rn(y[2 * e + 1], den));
+                        *reinterpret_cast<uint4 *>(dst + d0 + 4 * c) = make_uint4(o[0], o[1], o[2], o[3]);
+                    }
+            }
+            mbarrier_arrive_one(&S.qfree);
         }
-        if (*(volatile int *)&s_abort)  // error path: the copies in flight get a bounded chance to land
-            for (int h = issued > RA_UNITS ? issued - RA_UNITS : 0; h < issued; ++h)
-                mbar_wait(&full[h % RA_UNITS], (h / RA_UNITS) & 1, nullptr, 0, nullptr);
-        return;
+        tc_fence_before();
     }
-    // ---- compute warps
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 224;");
-    const int gq = lane >> 2, tq = lane & 3;
-    const float scale = a.att_scale;
-    const int HALF = ATT_SPLIT / a.att_subs;
-    const uint32_t koff = attn_k_lane(lane), voff = attn_v_lane(lane);
-    uint32_t ph = 0;
-    for (int w = blockIdx.x; w < n_work; w += gridDim.x) {
-        const RowsAttn wk = work[w];
-        const RowSeg sg = a.segs[wk.seg];
-        const int last = sg.pos0 + min(sg.n - 1, (wk.q0 + 16 * RA_WARPS - 1) / grp);
-        const int ns = last / ATT_SPLIT + 1, T = sg.pos0 + sg.n, QV = sg.n * grp;
-        const int qv0 = wk.q0 + warp * 16 + gq, qv1 = qv0 + 8;
-        const bool val0 = qv0 < QV, val1 = qv1 < QV;
-        const int i0 = val0 ? qv0 / grp : 0, i1 = val1 ? qv1 / grp : 0;
-        const int h0 = wk.g * grp + (val0 ? qv0 % grp : 0), h1 = wk.g * grp + (val1 ? qv1 % grp : 0);
-        const int lim0 = val0 ? sg.pos0 + i0 : -1, lim1 = val1 ? sg.pos0 + i1 : -1;  // last visible keys
-        // the warp's last visible key (-1: no rows), and the last key that all its rows see
-        const int wq0 = wk.q0 + warp * 16;
-        const int wlast = wq0 < QV ? sg.pos0 + min(sg.n - 1, (wq0 + 15) / grp) : -1;
-        const int wall = wq0 + 15 < QV ? sg.pos0 + wq0 / grp : -1;
-        uint32_t qa[KS][4];
-        {
-            const bf16 *q0 = a.q + ((size_t)(sg.row0 + i0) * dm.Hq + h0) * DH + 2 * tq;
-            const bf16 *q1 = a.q + ((size_t)(sg.row0 + i1) * dm.Hq + h1) * DH + 2 * tq;
-#pragma unroll
-            for (int ks = 0; ks < KS; ++ks) {
-                qa[ks][0] = val0 ? *reinterpret_cast<const unsigned *>(q0 + ks * 16) : 0u;
-                qa[ks][1] = val1 ? *reinterpret_cast<const unsigned *>(q1 + ks * 16) : 0u;
-                qa[ks][2] = val0 ? *reinterpret_cast<const unsigned *>(q0 + ks * 16 + 8) : 0u;
-                qa[ks][3] = val1 ? *reinterpret_cast<const unsigned *>(q1 + ks * 16 + 8) : 0u;
-            }
-        }
-        // first sweep: each row's largest score (the scale is positive and rounding is monotonic, so the
-        // largest scaled score is the scaled largest score)
-        float x0 = -INFINITY, x1 = -INFINITY;
-        for (int s = 0; s < ns; ++s) {
-            if (!mbar_wait(&full[slot], ph, a.status, DEV_TIMEOUT_LOAD, &s_abort)) return;
-            const uint32_t kaddr = smem_u32(ring + (size_t)slot * LY::UNIT) + koff;
-            const int k0 = s * ATT_SPLIT;
-#pragma unroll 1
-            for (int c0 = 0; c0 < ATT_SPLIT && k0 + c0 <= wlast; c0 += 32) {
-                float sc[4][4];
-                attn_scores<DH>(kaddr + c0 * 128, qa, sc);
-                if (k0 + c0 + 31 <= wall) {
-#pragma unroll
-                    for (int nt = 0; nt < 4; ++nt) {
-                        x0 = fmaxf(x0, fmaxf(sc[nt][0], sc[nt][1]));
-                        x1 = fmaxf(x1, fmaxf(sc[nt][2], sc[nt][3]));
-                    }
-                } else {
-#pragma unroll
-                    for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-                        for (int e = 0; e < 2; ++e) {
-                            const int kp = k0 + c0 + nt * 8 + 2 * tq + e;
-                            x0 = fmaxf(x0, kp <= lim0 ? sc[nt][e] : -INFINITY);
-                            x1 = fmaxf(x1, kp <= lim1 ? sc[nt][2 + e] : -INFINITY);
-                        }
-                }
-            }
-            __syncwarp();
-            if (lane == 0) mbarrier_arrive_one(&empty[slot]);
-            if (++slot == RA_UNITS) slot = 0, ph ^= 1;
-        }
-        x0 = fmaxf(x0, __shfl_xor_sync(0xffffffffu, x0, 1));
-        x0 = fmaxf(x0, __shfl_xor_sync(0xffffffffu, x0, 2));
-        x1 = fmaxf(x1, __shfl_xor_sync(0xffffffffu, x1, 1));
-        x1 = fmaxf(x1, __shfl_xor_sync(0xffffffffu, x1, 2));
-        x0 = __fmul_rn(x0, scale);
-        x1 = __fmul_rn(x1, scale);
-        // second sweep: partial results in key order, added with their weights relative to x0 / x1
-        float num[DT][4], den0 = 0.f, den1 = 0.f;
-#pragma unroll
-        for (int dt = 0; dt < DT; ++dt) num[dt][0] = num[dt][1] = num[dt][2] = num[dt][3] = 0.f;
-        for (int s = 0; s < ns; ++s) {
-            const int kslot = slot;
-            if (!mbar_wait(&full[slot], ph, a.status, DEV_TIMEOUT_LOAD, &s_abort)) return;
-            if (++slot == RA_UNITS) slot = 0, ph ^= 1;
-            const int vslot = slot;
-            if (!mbar_wait(&full[slot], ph, a.status, DEV_TIMEOUT_LOAD, &s_abort)) return;
-            if (++slot == RA_UNITS) slot = 0, ph ^= 1;
-            const uint32_t kaddr = smem_u32(ring + (size_t)kslot * LY::UNIT) + koff;
-            const uint32_t vaddr = smem_u32(ring + (size_t)vslot * LY::UNIT) + voff;
-            const int k0 = s * ATT_SPLIT;
-#pragma unroll 1
-            for (int kb = 0; kb < ATT_SPLIT && k0 + kb <= wlast; kb += HALF) {
-                float m0 = -INFINITY, m1 = -INFINITY, l0 = 0.f, l1 = 0.f;
-                float oc[DT][4];
-#pragma unroll
-                for (int dt = 0; dt < DT; ++dt) oc[dt][0] = oc[dt][1] = oc[dt][2] = oc[dt][3] = 0.f;
-#pragma unroll 1
-                for (int c0 = kb; c0 < kb + HALF && k0 + c0 <= wlast; c0 += 32) {
-                    float sc[4][4];
-                    attn_scores<DH>(kaddr + c0 * 128, qa, sc);
-                    const bool all = k0 + c0 + 31 <= wall;  // (uniform) no key to mask
-                    float c0m = -INFINITY, c1m = -INFINITY;
-#pragma unroll
-                    for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-                        for (int e = 0; e < 2; ++e) {
-                            const int kp = k0 + c0 + nt * 8 + 2 * tq + e;
-                            sc[nt][e] = all || kp <= lim0 ? __fmul_rn(sc[nt][e], scale) : -INFINITY;
-                            sc[nt][2 + e] = all || kp <= lim1 ? __fmul_rn(sc[nt][2 + e], scale) : -INFINITY;
-                            c0m = fmaxf(c0m, sc[nt][e]);
-                            c1m = fmaxf(c1m, sc[nt][2 + e]);
-                        }
-                    c0m = fmaxf(c0m, __shfl_xor_sync(0xffffffffu, c0m, 1));
-                    c0m = fmaxf(c0m, __shfl_xor_sync(0xffffffffu, c0m, 2));
-                    c1m = fmaxf(c1m, __shfl_xor_sync(0xffffffffu, c1m, 1));
-                    c1m = fmaxf(c1m, __shfl_xor_sync(0xffffffffu, c1m, 2));
-                    const float n0 = fmaxf(m0, c0m), n1 = fmaxf(m1, c1m);
-                    if (__any_sync(0xffffffffu, (n0 != m0 && m0 != -INFINITY) || (n1 != m1 && m1 != -INFINITY))) {
-                        const float a0 = m0 == -INFINITY ? 0.f : __expf(m0 - n0), a1 = m1 == -INFINITY ? 0.f : __expf(m1 - n1);
-                        l0 = __fmul_rn(l0, a0);
-                        l1 = __fmul_rn(l1, a1);
-#pragma unroll
-                        for (int dt = 0; dt < DT; ++dt) {
-                            oc[dt][0] = __fmul_rn(oc[dt][0], a0);
-                            oc[dt][1] = __fmul_rn(oc[dt][1], a0);
-                            oc[dt][2] = __fmul_rn(oc[dt][2], a1);
-                            oc[dt][3] = __fmul_rn(oc[dt][3], a1);
-                        }
-                    }
-                    const float z0 = n0 == -INFINITY ? 0.f : n0, z1 = n1 == -INFINITY ? 0.f : n1;
-                    m0 = n0;
-                    m1 = n1;
-#pragma unroll
-                    for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-                        for (int e = 0; e < 2; ++e) {
-                            sc[nt][e] = __expf(sc[nt][e] - z0);  // (0 for a masked score)
-                            sc[nt][2 + e] = __expf(sc[nt][2 + e] - z1);
-                            l0 += sc[nt][e];
-                            l1 += sc[nt][2 + e];
-                        }
-#pragma unroll
-                    for (int kstep = 0; kstep < 2; ++kstep) {
-                        uint32_t pa[4];
-                        pa[0] = pack_bf162(sc[2 * kstep][0], sc[2 * kstep][1]);
-                        pa[1] = pack_bf162(sc[2 * kstep][2], sc[2 * kstep][3]);
-                        pa[2] = pack_bf162(sc[2 * kstep + 1][0], sc[2 * kstep + 1][1]);
-                        pa[3] = pack_bf162(sc[2 * kstep + 1][2], sc[2 * kstep + 1][3]);
-                        // V of keys at or past T: whatever the page or the ring held, so zero (see attn_split)
-                        const int kst = k0 + c0 + kstep * 16;
-                        uint32_t ma = 0xFFFFFFFFu, mb = 0xFFFFFFFFu;
-                        if (kst + 16 > T) {
-                            const int ka = kst + 2 * tq;
-                            ma = (ka < T ? 0x0000FFFFu : 0u) | (ka + 1 < T ? 0xFFFF0000u : 0u);
-                            mb = (ka + 8 < T ? 0x0000FFFFu : 0u) | (ka + 9 < T ? 0xFFFF0000u : 0u);
-                        }
-                        // (pages past the CTA's last visible key were not loaded)
-                        const int lastpg = (last / PAGE + 1) * PAGE;
-                        if (kst >= lastpg) ma = mb = 0u;
-                        attn_pv<DH>(vaddr + (c0 + kstep * 16) * 128, pa, ma, mb, oc);
-                    }
-                }
-                l0 += __shfl_xor_sync(0xffffffffu, l0, 1);
-                l0 += __shfl_xor_sync(0xffffffffu, l0, 2);
-                l1 += __shfl_xor_sync(0xffffffffu, l1, 1);
-                l1 += __shfl_xor_sync(0xffffffffu, l1, 2);
-                if (l0 > 0.f) {  // (else the row saw no key in this partial result)
-                    const float wt = __expf(m0 - x0);
-                    den0 = __fadd_rn(den0, __fmul_rn(wt, l0));
-#pragma unroll
-                    for (int dt = 0; dt < DT; ++dt) {
-                        num[dt][0] = __fadd_rn(num[dt][0], __fmul_rn(wt, oc[dt][0]));
-                        num[dt][1] = __fadd_rn(num[dt][1], __fmul_rn(wt, oc[dt][1]));
-                    }
-                }
-                if (l1 > 0.f) {
-                    const float wt = __expf(m1 - x1);
-                    den1 = __fadd_rn(den1, __fmul_rn(wt, l1));
-#pragma unroll
-                    for (int dt = 0; dt < DT; ++dt) {
-                        num[dt][2] = __fadd_rn(num[dt][2], __fmul_rn(wt, oc[dt][2]));
-                        num[dt][3] = __fadd_rn(num[dt][3], __fmul_rn(wt, oc[dt][3]));
-                    }
-                }
-            }
-            __syncwarp();
-            if (lane == 0) {
-                mbarrier_arrive_one(&empty[kslot]);
-                mbarrier_arrive_one(&empty[vslot]);
-            }
-        }
-        if (val0) {
-            bf16 *dst = a.attn + ((size_t)(sg.row0 + i0) * dm.Hq + h0) * DH + 2 * tq;
-#pragma unroll
-            for (int dt = 0; dt < DT; ++dt)
-                *reinterpret_cast<uint32_t *>(dst + dt * 8) = pack_bf162(__fdiv_rn(num[dt][0], den0), __fdiv_rn(num[dt][1], den0));
-        }
-        if (val1) {
-            bf16 *dst = a.attn + ((size_t)(sg.row0 + i1) * dm.Hq + h1) * DH + 2 * tq;
-#pragma unroll
-            for (int dt = 0; dt < DT; ++dt)
-                *reinterpret_cast<uint32_t *>(dst + dt * 8) = pack_bf162(__fdiv_rn(num[dt][2], den1), __fdiv_rn(num[dt][3], den1));
-        }
-    }
+    __syncwarp();
+    __syncthreads();
+    if (warp == 4) tmem_dealloc(tmem, 256);
 }
 
 // final RMSNorm of read-out row r: the last row of segment ro[r]
@@ -553,11 +681,16 @@ __global__ void __launch_bounds__(RW_THREADS) k_rows_final(const __grid_constant
 
 // ------------------------------------------------------------------ host side
 
+template <int DH>
+static cudaError_t configure_rows_attn() {
+    const void *f = (const void *)k_rows_attn<DH>;
+    const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, RaLayout<DH>::TOTAL);
+    return e != cudaSuccess ? e : cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+}
+
 cudaError_t configure_rows_kernels() {
-    cudaError_t e = cudaFuncSetAttribute(k_rows_attn<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, RaLayout<128>::TOTAL);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_rows_attn<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, RaLayout<64>::TOTAL);
-    return e;
+    const cudaError_t e = configure_rows_attn<128>();
+    return e != cudaSuccess ? e : configure_rows_attn<64>();
 }
 
 static int warp_blocks(long warps, int max_ctas) {
@@ -565,7 +698,7 @@ static int warp_blocks(long warps, int max_ctas) {
     return (int)std::min<long>(b, max_ctas > 0 ? max_ctas : 1 << 30);
 }
 
-int rows_attn_tile() { return 16 * RA_WARPS; }
+int rows_attn_tile() { return RA_PAIRS; }
 
 cudaError_t launch_rows_embed(const RowsArgs &a, const int *ids, const void *embed_tiled, const void *gain, cudaStream_t st) {
     return launch_pdl(k_rows_embed, warp_blocks(a.M, a.max_ctas), RW_THREADS, 0, st, a, ids,

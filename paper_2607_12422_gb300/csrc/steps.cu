@@ -135,31 +135,7 @@ __device__ __forceinline__ float sum_slices(uint32_t a, int ks, uint32_t stride,
     return y;
 }
 
-// y_f += scale * (u . B_f) for two features f, the products added in rank order: packed fp32 multiplies and
-// adds, each half rounded as __fmul_rn and __fadd_rn round
-struct F2 {
-    unsigned long long v;
-};
-__device__ __forceinline__ F2 f2(float x, float y) {
-    F2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(x), "f"(y));
-    return r;
-}
-__device__ __forceinline__ F2 mul2(F2 a, F2 b) {
-    F2 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
-    return r;
-}
-__device__ __forceinline__ F2 add2(F2 a, F2 b) {
-    F2 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
-    return r;
-}
-__device__ __forceinline__ float2 unpack2(F2 a) {
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a.v));
-    return r;
-}
+// y_f += scale * (u . B_f) for two pairs of features f, the products added in rank order.
 // lane_ua / lane_ub: lane i holds u_i for the first / second pair of features (at fa, fb in the tile)
 __device__ __forceinline__ void add_delta(float (&y)[4], float lane_ua, float lane_ub, int base_b, const float *bt, int fa, int fb,
                                           int r, float scale) {
@@ -170,11 +146,11 @@ __device__ __forceinline__ void add_delta(float (&y)[4], float lane_ua, float la
         const float ua = __shfl_sync(0xffffffffu, lane_ua, i), ub = __shfl_sync(0xffffffffu, lane_ub, base_b + i);
         const float2 ba = *reinterpret_cast<const float2 *>(bt + i * TILE_ROWS + fa);
         const float2 bb = *reinterpret_cast<const float2 *>(bt + i * TILE_ROWS + fb);
-        a = add2(a, mul2(f2(ua, ua), f2(ba.x, ba.y)));
-        b = add2(b, mul2(f2(ub, ub), f2(bb.x, bb.y)));
+        a = add2(a, mul2(ua, ba.x, ba.y));
+        b = add2(b, mul2(ub, bb.x, bb.y));
     }
-    const F2 s2 = f2(scale, scale);
-    const float2 ya = unpack2(add2(f2(y[0], y[1]), mul2(s2, a))), yb = unpack2(add2(f2(y[2], y[3]), mul2(s2, b)));
+    const float2 da = unpack2(a), db = unpack2(b);
+    const float2 ya = unpack2(add2(f2(y[0], y[1]), mul2(scale, da.x, da.y))), yb = unpack2(add2(f2(y[2], y[3]), mul2(scale, db.x, db.y)));
     y[0] = ya.x, y[1] = ya.y, y[2] = yb.x, y[3] = yb.y;
 }
 

@@ -96,7 +96,7 @@ def test_lm_head_edges(torch, M, H, V):
 
 @pytest.mark.parametrize("shape,max_seq,start,rounds,ctas", [("tiny", 256, 1, 9, 0), ("qwen2", 420, 40, 21, 0),
                                                             ("qwen2", 4096, 301, 30, 0), ("grp4", 420, 17, 10, 0),
-                                                            ("qwen2", 420, 130, 14, 20)])
+                                                            ("qwen2", 420, 130, 14, 20), ("tiny", 600, 130, 25, 4)])
 def test_prefill_equals_decoded_rows_bitwise(torch, shape, max_seq, start, rounds, ctas):
     """The many-row kernels of the prefill against the pass kernel: K/V of every layer, written by
     verify rounds that commit 17 random tokens each, equal a prefill of the same tokens, and so do the
