@@ -51,9 +51,12 @@ struct Bump {
 // Buffers of a pass over many prompt rows (rows.cu).
 constexpr int ROWS_MAX = 4096;                   // rows per pass at most,
 constexpr size_t ROWS_BYTES = (size_t)256 << 20; // or as many as this holds
-// A single prompt of at most this many tokens goes through the persistent pass kernel instead, which is
-// the faster of the two for one operand tile of rows (0.6B shape, 17 tokens: 2.0 against 2.4 ms; 64
+// A single prompt of few tokens is one decoding pass instead: its rows are too few for the many-row kernels' serial
+// K loops.  As a kernel chain it is the faster of the two up to 128 tokens (0.6B shape: 33 tokens 1.36 against
+// 2.09 ms, 64 1.57 / 2.07, 96 1.69 / 2.08, 128 1.94 / 2.12, 160 2.24 / 2.15); on the persistent kernel,
+// where the chain does not run, only for one operand tile of rows (17 tokens: 2.0 against 2.4 ms; 64
 // tokens: 3.2 against 2.5 ms).
+constexpr int CHAIN_PROMPT = 128;
 constexpr int SHORT_PROMPT = 32;
 struct RowsBuf {
     int cap = 0, work_cap = 0;
@@ -223,7 +226,7 @@ size_t layout(pbd_ctx *c, void *base) {
     const int nl = k.n_layers, H = k.hidden, d = k.head_dim, Hq = k.n_q_heads, Hkv = k.n_kv_heads;
     const int I = k.intermediate, V = k.vocab, r = k.lora_rank, D = k.block_D;
     c->D = D;
-    c->rows_alloc = ((std::max(k.max_batch * (D + 1), SHORT_PROMPT) + 31) / 32) * 32;
+    c->rows_alloc = ((std::max(k.max_batch * (D + 1), CHAIN_PROMPT) + 31) / 32) * 32;
     c->ro_alloc = k.max_batch * (D + 1);
     c->out_cap = k.max_seq_len;
     // a truncated last round can leave L up to D past the budget, and every later pass still
@@ -802,8 +805,8 @@ pbd_status enqueue_prompts(pbd_ctx *c, const int32_t *d_ids) {
     return rows > 0 ? flush() : PBD_OK;
 }
 
-// One prompt of at most SHORT_PROMPT tokens as one pass of the persistent kernel.
-pbd_status enqueue_short_prompt(pbd_ctx *c, int P, const int32_t *d_ids) {
+// One prompt as a single decoding pass over its P rows.
+PassDesc prompt_pass(pbd_ctx *c, int P) {
     PassDesc pd{};
     pd.nb = 1;
     pd.R = pd.M = P;
@@ -812,6 +815,19 @@ pbd_status enqueue_short_prompt(pbd_ctx *c, int P, const int32_t *d_ids) {
     pd.ro_count = 1;
     pd.nl_run = c->cfg.n_layers;
     pd.att_span = att_span_of(c);
+    return pd;
+}
+
+// Whether a lone prompt goes that way: up to CHAIN_PROMPT rows as a kernel chain, up to SHORT_PROMPT on the persistent
+// kernel.
+bool short_prompt(pbd_ctx *c, int P) {
+    const bool chain = c->cfg.max_ctas == 0 && P <= CHAIN_PROMPT &&
+                       step_pass_fits(c->dm, prompt_pass(c, P), att_subs_of(c), (P + ATT_SPLIT - 1) / ATT_SPLIT);
+    return chain || P <= SHORT_PROMPT;
+}
+
+pbd_status enqueue_short_prompt(pbd_ctx *c, int P, const int32_t *d_ids) {
+    const PassDesc pd = prompt_pass(c, P);
     const RowSeg seg{0, 0, 0, P};
     const int ro = 0;
     c->steps[PK_PREFILL] = c->cfg.max_ctas == 0 && step_pass_fits(c->dm, pd, att_subs_of(c), (P + ATT_SPLIT - 1) / ATT_SPLIT);
@@ -1014,7 +1030,7 @@ pbd_status pbd_prefill(pbd_ctx *c, int32_t batch, const int32_t *d_prompt_ids, c
     c->batch = batch;
     c->max_new = max_new;
     c->prompt_lens.assign(h_prompt_lens, h_prompt_lens + batch);
-    if (batch == 1 && h_prompt_lens[0] <= SHORT_PROMPT)
+    if (batch == 1 && short_prompt(c, h_prompt_lens[0]))
         TRY(enqueue_short_prompt(c, h_prompt_lens[0], d_prompt_ids));
     else
         TRY(enqueue_prompts(c, d_prompt_ids));

@@ -96,3 +96,23 @@ def test_graphs_follow_the_generation(torch):
         toks = [eng.pbd_decode_step()[0].clone() for _ in range(23)]
         assert torch.equal(spec[:, 1:], torch.stack(toks, 1)), lens
     eng.close()
+
+
+@pytest.mark.parametrize("shape,P", [("qwen2", 33), ("qwen2", 127), ("qwen2", 128), ("qwen2", 129), ("tiny", 100)])
+def test_prompt_of_few_tokens_equals_the_many_row_kernels(torch, shape, P):
+    """A lone prompt up to the chain's limit is one decoding pass; in a batch it goes through the many-row
+    kernels: the same first token and K/V, bit for bit."""
+    from paper_2607_12422_gb300 import pbd, synth
+    S = _shape(shape)
+    base, ad = synth.with_random_norm_gains(synth.gen_base_weights(S)), synth.gen_adapter(S)
+    eng = pbd.Engine(S, base, ad, block_D=8, max_batch=2, max_seq_len=256)
+    p = np.random.default_rng(P).integers(0, S.vocab, P).astype(np.int32)
+    first = int(eng.pbd_prefill([p], max_new=4)[0])
+    kv = [eng.pbd_read_kv(l, 0, P) for l in range(S.n_layers)]
+    both = eng.pbd_prefill([p, p], max_new=4)
+    assert first == int(both[0]) == int(both[1])
+    for l in range(S.n_layers):
+        for b in (0, 1):
+            k, v = eng.pbd_read_kv(l, b, P)
+            assert torch.equal(kv[l][0], k) and torch.equal(kv[l][1], v), (l, b)
+    eng.close()
