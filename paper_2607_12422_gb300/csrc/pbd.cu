@@ -843,9 +843,9 @@ pbd_status enqueue_short_prompt(pbd_ctx *c, int P, const int32_t *d_ids) {
 }
 
 pbd_status check_device(pbd_ctx *c) {
-    CK(cudaStreamSynchronize(c->st));
     int code = 0;
-    CK(cudaMemcpy(&code, c->status, sizeof(int), cudaMemcpyDeviceToHost));
+    CK(cudaMemcpyAsync(&code, c->status, sizeof(int), cudaMemcpyDeviceToHost, c->st));
+    CK(cudaStreamSynchronize(c->st));
     if (code != 0) {
         CK(cudaMemsetAsync(c->status, 0, sizeof(int), c->st));  // reported once; the context stays usable
         CK(cudaStreamSynchronize(c->st));
