@@ -144,9 +144,9 @@ def source_hash(path):
 
 
 def traffic_for(kernel_src):
-    """DRAM bytes per launch from the committed ncu summary, if the kernel source is unchanged since
+    """DRAM bytes per pass from the committed ncu summary, if the kernel source is unchanged since
     (comments aside)."""
-    path = os.path.join(ROOT, "profiles", "k_pass_verify_qwen3_0.6b_traffic.json")
+    path = os.path.join(ROOT, "profiles", "steps_verify_qwen3_0.6b_traffic.json")
     try:
         with open(path) as f:
             rec = json.load(f)
@@ -401,12 +401,12 @@ def main(args):
     floor_v = b_verify / (hbm * 1e9) * 1e6
     floor_d = b_draft / (hbm * 1e9) * 1e6
 
-    # ---- dominant kernel: the persistent pass kernel (all 28 layers of a verify pass), timed alone
+    # ---- dominant part: the kernel chain of a verify pass (all 28 layers), timed alone
     eng.pbd_prefill([prompt], max_new=G)
     ms_k, k_bytes = eng.pbd_time_pass(1, 16)
     ms_kd, kd_bytes = eng.pbd_time_pass(0, 16)
     achieved = k_bytes / (ms_k * 1e-3) / 1e9
-    traffic = traffic_for(os.path.join(ROOT, "paper_2607_12422_gb300", "csrc", "pass_kernel.cu"))
+    traffic = traffic_for(os.path.join(ROOT, "paper_2607_12422_gb300", "csrc", "steps.cu"))
 
     # ---- end to end through the public call with host buffers
     # (host prompt ids in, host token ids out; the binding copies the prompt to the device),
@@ -479,7 +479,7 @@ def main(args):
                    "break_even_accept": (draft_us + verify_us) / ar_us},
             "draft_variants": variants,
             "other_workloads": configs,
-            "roofline": {"bound": "hbm", "kernel": "k_pass (persistent; 28 layers of one verify pass, 17 rows)",
+            "roofline": {"bound": "hbm", "kernel": "k_step_* chain (28 layers of one verify pass, 17 rows)",
                          "achieved": achieved, "peak": hbm, "peak_kind": peak_kind + " hbm_gbs (burst)",
                          "unit": "GB/s", "frac": achieved / hbm, "traffic": traffic,
                          "algorithmic_bytes": k_bytes, "us_per_launch": ms_k * 1e3,

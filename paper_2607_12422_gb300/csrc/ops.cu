@@ -1,4 +1,4 @@
-// ops.cu -- small kernels around the persistent pass kernel:
+// ops.cu -- small kernels around the passes:
 //   k_build_ids       row token ids of a draft / verify / decode pass from the device state
 //   k_accept_commit   longest accepted prefix, emission, KV commit (Section 3, steps 4-5)
 //   k_prefill_finish  cached lengths and first tokens after prompts

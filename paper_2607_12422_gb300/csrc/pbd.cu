@@ -6,8 +6,10 @@
 // the persistent pass kernel, and the pass scratch (activations, split-K partial sums,
 // attention partials, completion counters, lm_head tile maxima).
 //
-// A pass is: zero the pass counters, build the rows' token ids, one persistent pass kernel
-// (all decoder layers), the lm_head over the read-out rows, the final argmax.  A speculative
+// A decoding pass is: build the rows' token ids, the decoder layers as a chain of small kernels (steps.cu; contexts
+// limited to fewer CTAs than SMs and shapes that do not fit it run the persistent kernel of
+// pass_kernel.cu instead, with the same results bit for bit), the lm_head over the read-out rows, the
+// final argmax.  Prompts of many rows go through rows.cu and gemm.cu.  A speculative
 // round (draft pass, verify pass, accept/commit) only reads and writes device memory, so it is
 // captured once as a CUDA graph and replayed; the host looks at the done flags every few rounds.
 #include <cuda.h>

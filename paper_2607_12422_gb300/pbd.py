@@ -438,7 +438,7 @@ class Engine:
         return int(status), int(code[0])
 
     def pbd_time_pass(self, kind: int, iters: int):
-        """(ms per launch, algorithmic bytes per launch) of the persistent pass kernel timed alone
+        """(ms per pass, algorithmic bytes per pass) of the decoder layers of one pass timed alone
         (kind 0 draft, 1 verify, 2 plain decoding)."""
         ms = np.zeros(1, np.float64)
         nb = np.zeros(1, np.float64)

@@ -1,10 +1,8 @@
-"""Small standalone driver of the persistent pass kernel, for profilers.
+"""Small standalone driver of a decoding pass's layers, for profilers.
 
 Builds a context for a workload (seeded weights), prefills its prompts, then launches
-`--iters` draft / verify / decode passes through pbd_time_pass (one warm-up launch first) and
-prints the mean device time per launch.  The prefill itself launches the pass kernel once per
-64-token chunk of each prompt, so a profiler that wants the first timed pass skips the printed
-prefill_launches + 1 launches.
+`--iters` draft / verify / decode passes through pbd_time_pass (one warm-up pass first) and
+prints the mean device time per pass.  A profiler picks the passes' kernels by name (k_step_*).
 
     python -m paper_2607_12422_gb300.profile_pass --kind verify --iters 3
 """
@@ -28,7 +26,7 @@ def main():
     kind = {"draft": 0, "verify": 1, "decode": 2}[a.kind]
     ms, nbytes = eng.pbd_time_pass(kind, a.iters)
     print(json.dumps({"workload": a.workload, "kind": a.kind, "batch": len(lens),
-                      "prefill_launches": sum(-(-P // 64) for P in lens), "ms_per_launch": ms,
+                      "ms_per_launch": ms,
                       "bytes_per_launch": nbytes}))
 
 
