@@ -149,3 +149,28 @@ def test_prefill_batch_and_passes_match_single_prompts(torch):
         k, v = eng.pbd_read_kv(S.n_layers - 1, 0, len(p))
         assert torch.equal(k, kv[b][0]) and torch.equal(v, kv[b][1]), b
     eng.close()
+
+
+@pytest.mark.parametrize("shape", ["tiny", "qwen2"])
+def test_prompt_over_pages_that_hold_nan(torch, shape):
+    """Pages keep what an earlier generation left there.  After a prompt whose every K and V is NaN (an
+    infinite embedding row), shorter prompts give the first token and K/V of a context without that past:
+    keys beyond the prompt's end take no part, whatever their page holds."""
+    import dataclasses
+    from paper_2607_12422_gb300 import pbd, synth
+    S = synth.TINY if shape == "tiny" else dataclasses.replace(synth.QWEN3_0_6B, n_layers=2, vocab=4096)
+    base, ad = synth.gen_base_weights(S), synth.gen_adapter(S)
+    base["embed"] = base["embed"].copy()
+    base["embed"][7] = 0x7F80
+    rng = np.random.default_rng(11)
+    used, fresh = (pbd.Engine(S, base, ad, block_D=4, max_batch=1, max_seq_len=300) for _ in range(2))
+    for P in (129, 143, 190):
+        used.pbd_prefill([np.full(250, 7, np.int32)], max_new=4)
+        assert torch.isnan(used.pbd_read_kv(1, 0, 250)[1].float()).all()
+        p = rng.integers(8, S.vocab, P).astype(np.int32)
+        assert int(used.pbd_prefill([p], max_new=4)[0]) == int(fresh.pbd_prefill([p], max_new=4)[0])
+        for l in range(S.n_layers):
+            for x, y in zip(used.pbd_read_kv(l, 0, P), fresh.pbd_read_kv(l, 0, P)):
+                assert torch.equal(x, y) and not torch.isnan(x.float()).any(), (P, l)
+    used.close()
+    fresh.close()
