@@ -153,9 +153,12 @@ __global__ void __launch_bounds__(RW_THREADS) k_rows_norm(const __grid_constant_
 
 // q|k|v of one row: per-head RMSNorm and RoPE of q and k; q to its buffer, k and v to the cache
 // pages.  A block per row, a warp per 128-feature tile (every eighth one): lane l holds features
-// 4l..4l+3, as in reduce_qkv (pass_kernel.cu).  Bound by L2: 8 bytes a feature, read and written.
+// 4l..4l+3, as in reduce_qkv (pass_kernel.cu).  Bound by issue slots (66% of them) and the loads' latency, not by
+// the 2 x 8 bytes a lane and tile: the row's loads go out before its position is looked up, and one lane
+// evaluates the root and divisions of each tile's 1/rms (4096 rows: 28 us without either, 24.5 with
+// both; 64 registers for four blocks an SM: at 74 registers 26.7, at 40 spills, 27).
 template <int DH>
-__global__ void __launch_bounds__(RW_THREADS) k_rows_rope(const __grid_constant__ RowsArgs a, int layer,
+__global__ void __launch_bounds__(RW_THREADS, 4) k_rows_rope(const __grid_constant__ RowsArgs a, int layer,
                                                           const bf16 *__restrict__ q_norm,
                                                           const bf16 *__restrict__ k_norm,
                                                           const float2 *__restrict__ rope_cs) {
@@ -177,6 +180,15 @@ __global__ void __launch_bounds__(RW_THREADS) k_rows_rope(const __grid_constant_
     gain4(k_norm, gk);
     pdl_begin();
     for (int m = blockIdx.x; m < a.M; m += gridDim.x) {
+        uint2 raw[U] = {};
+        auto load = [&](int t0) {
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int ft = (t0 + u * (RW_THREADS / 32)) * TILE_ROWS;
+                if (ft < qw + 2 * kvw) raw[u] = *reinterpret_cast<const uint2 *>(a.qkv + (size_t)m * (qw + 2 * kvw) + ft + 4 * lane);
+            }
+        };
+        load(warp);  // (on its way before the row's position is looked up)
         const RowSeg sg = a.segs[row_seg(a, m)];
         const int pos = sg.pos0 + m - sg.row0;
         const float4 *c4 = reinterpret_cast<const float4 *>(rope_cs + (size_t)pos * (DH / 2) + (e0 % (DH / 2)));
@@ -184,12 +196,22 @@ __global__ void __launch_bounds__(RW_THREADS) k_rows_rope(const __grid_constant_
         const float cs[4] = {ca.x, ca.z, cb.x, cb.z}, sn[4] = {ca.y, ca.w, cb.y, cb.w};
         const size_t slot = ((size_t)layer * a.kv.n_pages + a.kv.page_table[sg.seq * a.kv.pages_per_seq + pos / PAGE]) * dm.Hkv;
         for (int t0 = warp; t0 < nq; t0 += U * (RW_THREADS / 32)) {
-            uint2 raw[U];
+            if (t0 != warp) load(t0);
+            // the tiles' 1/rms: lane u of a head evaluates tile u's (the root and divisions are as long as the rest)
+            float mine = 0.f;
 #pragma unroll
             for (int u = 0; u < U; ++u) {
-                const int ft = (t0 + u * (RW_THREADS / 32)) * TILE_ROWS;
-                if (ft < qw + 2 * kvw) raw[u] = *reinterpret_cast<const uint2 *>(a.qkv + (size_t)m * (qw + 2 * kvw) + ft + 4 * lane);
+                const float2 ya = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&raw[u].x));
+                const float2 yb = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&raw[u].y));
+                const float y[4] = {ya.x, ya.y, yb.x, yb.y};
+                float ss = __fmul_rn(y[0], y[0]);
+#pragma unroll
+                for (int j = 1; j < 4; ++j) ss = __fadd_rn(ss, __fmul_rn(y[j], y[j]));
+#pragma unroll
+                for (int off = LPH / 2; off >= 1; off >>= 1) ss = __fadd_rn(ss, __shfl_xor_sync(0xffffffffu, ss, off));
+                if ((lane & (U - 1)) == u) mine = ss;
             }
+            const float rs_of = rms_scale(mine, DH, dm.eps);
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 const int ft = (t0 + u * (RW_THREADS / 32)) * TILE_ROWS;
@@ -201,12 +223,7 @@ __global__ void __launch_bounds__(RW_THREADS) k_rows_rope(const __grid_constant_
                     const float2 ya = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&raw[u].x));
                     const float2 yb = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&raw[u].y));
                     float y[4] = {ya.x, ya.y, yb.x, yb.y};
-                    float ss = __fmul_rn(y[0], y[0]);
-#pragma unroll
-                    for (int j = 1; j < 4; ++j) ss = __fadd_rn(ss, __fmul_rn(y[j], y[j]));
-#pragma unroll
-                    for (int off = LPH / 2; off >= 1; off >>= 1) ss = __fadd_rn(ss, __shfl_xor_sync(0xffffffffu, ss, off));
-                    const float rs = rms_scale(ss, DH, dm.eps);
+                    const float rs = __shfl_sync(0xffffffffu, rs_of, (lane & ~(LPH - 1)) | u);
                     float z[4];
 #pragma unroll
                     for (int j = 0; j < 4; ++j) y[j] = rbf(__fmul_rn(kind == 0 ? gq[j] : gk[j], rbf(__fmul_rn(y[j], rs))));
