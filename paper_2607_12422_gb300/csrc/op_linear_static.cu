@@ -19,8 +19,8 @@
 
 // Layout inside the array (offsets from the first 1024-byte boundary in it):
 //   [0, 256)     status word of the tensor-core kernels (cleared by every call)
-//   [1024, ...)  room for the weight and the adapter's rows as 16 KiB tiles, then for split-K partial sums;
-//                the second part holds the adapter's u rows (and padded B rows) of calls with many rows
+//   [1024, ...)  room for the weight and the adapter's rows as 16 KiB tiles, then for split-K partial sums: calls with
+//                many rows keep padded adapter B rows in the first and the adapter's u rows in the second
 static __device__ __align__(256) unsigned char g_linear_scratch[PBD_OP_LINEAR_STATIC_SCRATCH_BYTES];
 
 using namespace pbd;
@@ -107,8 +107,8 @@ extern "C" pbd_status pbd_op_linear_static(int32_t M, int32_t K, int32_t N, int3
     const pbd_status s = scratch_of_current_device(&ws);
     if (s != PBD_OK) return s;
 
-    // What must start at zero on every call, the status word and the tile counters, is cleared by
-    // it; every other byte this call reads is written by this call first.
+    // What must start at zero on every call, the status word, is cleared by it; every other byte this
+    // call reads is written by this call first.
     return run_linear_op(M, K, N, rr, scale, d_x, d_w, d_a, d_b, d_y, LinearScratch{ws, ws + p.tiles_off, ws + p.part_off},
                          static_cast<cudaStream_t>(d_stream), "pbd_op_linear_static");
 }

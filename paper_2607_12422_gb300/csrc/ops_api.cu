@@ -150,7 +150,9 @@ pbd_status run_linear_op(int M, int K, int N, int r, float scale, const void *d_
     a.status = status;
     if ((e = cudaMemsetAsync(status, 0, 256, st)) != cudaSuccess) return bad(PBD_ERR_CUDA, "memset", e);
     if (r > 0) {
-        uint8_t *u = ws.part, *bp = ws.part + ((size_t)M * 64 + 1023) / 1024 * 1024;  // [M][32], [N][32]
+        // u [M][32] and a padded B [N][32].  Each fits its area whatever the sizes: `part` holds at least 512 bytes a row,
+        // `tiles` 128 a column.  (Behind u, B would not: `part` is small for few rows.)
+        uint8_t *u = ws.part, *bp = ws.tiles;
         GemmArgs g = a;
         g.bn = 64;
         if (!encode_bf16_map(&g.xmap, d_x, M, K, g.bn)) return bad(PBD_ERR_INVALID_ARG, "x not TMA-mappable");

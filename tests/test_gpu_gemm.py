@@ -65,6 +65,29 @@ def test_linear_unaligned_adapter_and_output(torch, M):
     assert ((got.double() - ref).abs() <= tol).all() and float(y[0]) == 0.0
 
 
+@pytest.mark.parametrize("M,K,N,r", [(1, 4352, 128, 1), (1, 4352, 128, 7), (2, 4608, 128, 3), (64, 4352, 256, 5),
+                                     (65, 64, 128, 1), (70, 320, 128, 31), (17, 1024, 128, 3), (4096, 64, 128, 9)])
+def test_linear_stays_inside_its_workspace(torch, M, K, N, r):
+    """A workspace of exactly the reported size, bytes of a known value right behind it: they keep it.
+    Ranks whose B rows are padded to 32 columns, with few and with many slices of K."""
+    from paper_2607_12422_gb300 import pbd
+    lib = pbd.load()
+    g = torch.Generator(device="cuda").manual_seed(M + K + r)
+    x, W = _rand(torch, g, (M, K), 1.0), _rand(torch, g, (N, K), 0.02)
+    A, B = _rand(torch, g, (r, K), 0.02), _rand(torch, g, (N, r), 0.02)
+    need, guard = lib.pbd_op_linear_workspace_bytes(M, K, N, r), 1 << 16
+    buf = torch.full((need + guard + 1024,), 0xA5, dtype=torch.uint8, device="cuda")
+    off = -buf.data_ptr() % 1024
+    y = torch.empty(M, N, dtype=torch.bfloat16, device="cuda")
+    st = torch.cuda.current_stream().cuda_stream
+    args = [t.data_ptr() for t in (x, W, A, B, y)]
+    assert lib.pbd_op_linear(M, K, N, r, 2.0, *args, buf.data_ptr() + off, need, st) == 0
+    assert lib.pbd_op_status(buf.data_ptr() + off, st, None) == 0
+    assert (buf[off + need:] == 0xA5).all()
+    ref, tol = _linear_ref(x, W, A, B, 2.0)
+    assert ((y.double() - ref).abs() <= tol).all()
+
+
 def test_linear_rows_do_not_depend_on_the_row_count(torch):
     from paper_2607_12422_gb300 import pbd
     g = torch.Generator(device="cuda").manual_seed(9)
