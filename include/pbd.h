@@ -127,7 +127,9 @@ pbd_status pbd_destroy(pbd_ctx *ctx);
  * d_prompt_ids: the prompts' token ids packed back to back; h_prompt_lens[b] their lengths.
  * Runs the causal adapter-off prefill, sets each sequence's cached length L_b = P_b and its
  * pending token to the verifier's argmax after the prompt; that token is output token 0,
- * also written to d_first_token[b] when non-null.  Synchronous on return. */
+ * also written to d_first_token[b] when non-null.  Synchronous on return.  Refused arguments
+ * (PBD_ERR_INVALID_ARG, PBD_ERR_CAPACITY for a batch or length) leave the generation before as it was;
+ * any other error ends it, and the context takes no call but a prefill until one succeeds. */
 pbd_status pbd_prefill(pbd_ctx *ctx, int32_t batch, const int32_t *d_prompt_ids, const int32_t *h_prompt_lens,
                        int32_t max_new, int32_t *d_first_token);
 

@@ -856,6 +856,46 @@ pbd_status check_device(pbd_ctx *c) {
     return PBD_OK;
 }
 
+// Everything a prefill does once its arguments are checked.
+pbd_status start_generation(pbd_ctx *c, int batch, const int32_t *d_prompt_ids, const int32_t *h_prompt_lens, int max_new,
+                            int32_t *d_first_token) {
+    c->drop_bench_graphs(0);
+    c->drop_bench_graphs(1);
+    // pages of sequence b are interleaved across the batch: page (b, j) -> j * batch + b
+    std::vector<int> pt((size_t)c->cfg.max_batch * c->pages_per_seq, 0);
+    for (int b = 0; b < batch; ++b)
+        for (int j = 0; j < c->pages_per_seq; ++j) pt[(size_t)b * c->pages_per_seq + j] = j * batch + b;
+    CK(cudaMemcpyAsync(c->page_table, pt.data(), pt.size() * sizeof(int), cudaMemcpyHostToDevice, c->st));
+    CK(cudaMemsetAsync(c->s.L, 0, sizeof(int) * c->cfg.max_batch, c->st));
+    CK(cudaMemsetAsync(c->s.n_out, 0, sizeof(int) * c->cfg.max_batch, c->st));
+    CK(cudaMemsetAsync(c->s.done, 0, sizeof(int) * c->cfg.max_batch, c->st));
+    CK(cudaMemsetAsync(c->s.all_done, 0, 2 * sizeof(int), c->st));
+    CK(cudaMemsetAsync(c->s.stats, 0, 3 * sizeof(long long), c->st));
+    CK(cudaStreamSynchronize(c->st));
+    c->batch = batch;
+    c->max_new = max_new;
+    c->prompt_lens.assign(h_prompt_lens, h_prompt_lens + batch);
+    if (batch == 1 && short_prompt(c, h_prompt_lens[0]))
+        TRY(enqueue_short_prompt(c, h_prompt_lens[0], d_prompt_ids));
+    else
+        TRY(enqueue_prompts(c, d_prompt_ids));
+    if (d_first_token)
+        CK(cudaMemcpyAsync(d_first_token, c->s.pending, sizeof(int) * batch, cudaMemcpyDeviceToDevice, c->st));
+    TRY(check_device(c));
+    // the decode passes of this generation: kernel chains where they fit, else schedules of the persistent
+    // kernel (which max_ctas limits to fewer CTAs than SMs)
+    const std::vector<int> ns = decode_splits(c);
+    c->nsplit = ns;
+    const int longest = *std::max_element(ns.begin(), ns.end());
+    for (int kind = PK_DRAFT; kind <= PK_DECODE; ++kind) {
+        const PassDesc pd = block_pass(c, kind);
+        c->sched[kind].valid = false;
+        c->steps[kind] = c->cfg.max_ctas == 0 && step_pass_fits(c->dm, pd, att_subs_of(c), longest);
+        if (!c->steps[kind]) TRY(upload_schedule(c, kind, pd, ns));
+    }
+    return PBD_OK;
+}
+
 double pass_bytes(pbd_ctx *c, int kind, const std::vector<int> &Ls) {
     const pbd_config &k = c->cfg;
     double w = 0, lora = 0;
@@ -1016,39 +1056,13 @@ pbd_status pbd_prefill(pbd_ctx *c, int32_t batch, const int32_t *d_prompt_ids, c
         if (h_prompt_lens[b] < 1 || h_prompt_lens[b] + max_new > c->cfg.max_seq_len)
             return fail(c, PBD_ERR_CAPACITY, "sequence %d: prompt %d + max_new %d exceeds max_seq_len %d", b,
                         h_prompt_lens[b], max_new, c->cfg.max_seq_len);
-    c->drop_bench_graphs(0);
-    c->drop_bench_graphs(1);
-    // pages of sequence b are interleaved across the batch: page (b, j) -> j * batch + b
-    std::vector<int> pt((size_t)c->cfg.max_batch * c->pages_per_seq, 0);
-    for (int b = 0; b < batch; ++b)
-        for (int j = 0; j < c->pages_per_seq; ++j) pt[(size_t)b * c->pages_per_seq + j] = j * batch + b;
-    CK(cudaMemcpyAsync(c->page_table, pt.data(), pt.size() * sizeof(int), cudaMemcpyHostToDevice, c->st));
-    CK(cudaMemsetAsync(c->s.L, 0, sizeof(int) * c->cfg.max_batch, c->st));
-    CK(cudaMemsetAsync(c->s.n_out, 0, sizeof(int) * c->cfg.max_batch, c->st));
-    CK(cudaMemsetAsync(c->s.done, 0, sizeof(int) * c->cfg.max_batch, c->st));
-    CK(cudaMemsetAsync(c->s.all_done, 0, 2 * sizeof(int), c->st));
-    CK(cudaMemsetAsync(c->s.stats, 0, 3 * sizeof(long long), c->st));
-    CK(cudaStreamSynchronize(c->st));
-    c->batch = batch;
-    c->max_new = max_new;
-    c->prompt_lens.assign(h_prompt_lens, h_prompt_lens + batch);
-    if (batch == 1 && short_prompt(c, h_prompt_lens[0]))
-        TRY(enqueue_short_prompt(c, h_prompt_lens[0], d_prompt_ids));
-    else
-        TRY(enqueue_prompts(c, d_prompt_ids));
-    if (d_first_token)
-        CK(cudaMemcpyAsync(d_first_token, c->s.pending, sizeof(int) * batch, cudaMemcpyDeviceToDevice, c->st));
-    TRY(check_device(c));
-    // the decode passes of this generation: kernel chains where they fit, else schedules of the persistent
-    // kernel (which max_ctas limits to fewer CTAs than SMs)
-    const std::vector<int> ns = decode_splits(c);
-    c->nsplit = ns;
-    const int longest = *std::max_element(ns.begin(), ns.end());
-    for (int kind = PK_DRAFT; kind <= PK_DECODE; ++kind) {
-        const PassDesc pd = block_pass(c, kind);
-        c->sched[kind].valid = false;
-        c->steps[kind] = c->cfg.max_ctas == 0 && step_pass_fits(c->dm, pd, att_subs_of(c), longest);
-        if (!c->steps[kind]) TRY(upload_schedule(c, kind, pd, ns));
+    // Until the new generation stands there is none: an error on the way (a token id that the device refuses) leaves a
+    // context that only another prefill takes further, with no batch whose plan would be that of the old one.
+    c->phase = PH_NONE;
+    const pbd_status s = start_generation(c, batch, d_prompt_ids, h_prompt_lens, max_new, d_first_token);
+    if (s != PBD_OK) {
+        c->batch = 0;
+        return s;
     }
     c->phase = PH_READY;
     return PBD_OK;

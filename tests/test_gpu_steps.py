@@ -98,6 +98,42 @@ def test_graphs_follow_the_generation(torch):
     eng.close()
 
 
+def test_refused_prefill_leaves_no_generation(torch):
+    """A prefill that the device refuses (a token id beyond the vocabulary) after a good one of another batch
+    size: what needs a generation is refused until a prefill succeeds, which then gives what a new context
+    gives.  Arguments refused on the host leave the generation as it was."""
+    from paper_2607_12422_gb300 import pbd, synth
+    S = _shape("tiny")
+    base, ad = synth.gen_base_weights(S), synth.gen_adapter(S)
+    rng = np.random.default_rng(5)
+    one, three = ([rng.integers(0, S.vocab, n).astype(np.int32) for n in lens] for lens in ((40,), (200, 20, 64)))
+    bad = [p.copy() for p in three]
+    bad[1][7] = S.vocab
+    used, fresh = (pbd.Engine(S, base, ad, block_D=4, max_batch=3, max_seq_len=256) for _ in range(2))
+    used.pbd_prefill(one, max_new=16)
+    with pytest.raises(pbd.PbdError) as ei:
+        used.pbd_prefill(three + one, max_new=16)
+    assert ei.value.status == 3
+    for _ in range(3):
+        used.pbd_draft_block()
+        used.pbd_verify_block()
+        used.pbd_accept_commit()
+    with pytest.raises(pbd.PbdError) as ei:
+        used.pbd_prefill(bad, max_new=16)
+    assert ei.value.status == 6
+    drafts = np.zeros((1, 4), np.int32)
+    for call in (used.pbd_draft_block, lambda: used.pbd_verify_block(drafts=drafts), used.pbd_accept_commit,
+                 used.pbd_decode_step, used.pbd_get_tokens, lambda: used.pbd_time_pass(1, 1),
+                 lambda: used.pbd_bench_rounds(0, 0, 1), lambda: used.pbd_trace_pass(1)):
+        with pytest.raises(pbd.PbdError) as ei:
+            call()
+        assert ei.value.status == 4
+    got, want = used.pbd_generate(three, 16)[0], fresh.pbd_generate(three, 16)[0]
+    assert torch.equal(got, want)
+    used.close()
+    fresh.close()
+
+
 @pytest.mark.parametrize("shape,P", [("qwen2", 33), ("qwen2", 127), ("qwen2", 128), ("qwen2", 129), ("tiny", 100)])
 def test_prompt_of_few_tokens_equals_the_many_row_kernels(torch, shape, P):
     """A lone prompt up to the chain's limit is one decoding pass; in a batch it goes through the many-row
