@@ -17,8 +17,9 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t
                                   const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-// 2-D bf16 row-major [rows, cols] tensor map with box {64, box_rows}, 128-byte swizzle.
-bool encode_bf16_map(CUtensorMap *map, const void *base, int rows, int cols, int box_rows) {
+// 2-D bf16 row-major [rows, cols] tensor map with box {64, box_rows}, 128-byte swizzle; rows lie ld values apart
+// (0: cols).
+bool encode_bf16_map(CUtensorMap *map, const void *base, int rows, int cols, int box_rows, int ld) {
     static EncodeTiledFn enc = nullptr;
     if (!enc) {
         void *fn = nullptr;
@@ -29,9 +30,10 @@ bool encode_bf16_map(CUtensorMap *map, const void *base, int rows, int cols, int
             return false;
         enc = reinterpret_cast<EncodeTiledFn>(fn);
     }
-    if ((reinterpret_cast<uintptr_t>(base) & 15) || (cols * 2) % 16) return false;
+    if (ld == 0) ld = cols;
+    if ((reinterpret_cast<uintptr_t>(base) & 15) || (ld * 2) % 16) return false;
     cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-    cuuint64_t strides[1] = {(cuuint64_t)cols * 2};
+    cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
     cuuint32_t box[2] = {(cuuint32_t)KT, (cuuint32_t)box_rows};
     cuuint32_t es[2] = {1, 1};
     return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), dims, strides, box, es,
@@ -158,13 +160,14 @@ pbd_status run_linear_op(int M, int K, int N, int r, float scale, const void *d_
         if (!encode_bf16_map(&g.xmap, d_x, M, K, g.bn)) return bad(PBD_ERR_INVALID_ARG, "x not TMA-mappable");
         if (!encode_bf16_map(&g.wmap, d_a, r, K, TILE_ROWS)) return bad(PBD_ERR_INVALID_ARG, "A not TMA-mappable");
         g.f_tiles = 1;
-        g.rows = 32;  // (rows past r are zero)
+        g.rows = 32;
         g.y = reinterpret_cast<bf16 *>(u);
         g.ld = 32;
         g.vec_store = 1;
         if ((e = launch_gemm(GEMM_Y, g, 0, st)) != cudaSuccess) return bad(PBD_ERR_CUDA, "adapter rows", e);
         a.delta = 1;
-        bool ok = encode_bf16_map(&a.umap, u, M, 32, a.bn);
+        // (r columns: the rest arrive as zeros.  What the kernel computed there, 0 x, is NaN where x is infinite.)
+        bool ok = encode_bf16_map(&a.umap, u, M, r, a.bn, 32);
         if (r % 8 == 0 && (reinterpret_cast<uintptr_t>(d_b) & 15) == 0) {
             ok = ok && encode_bf16_map(&a.bmap, d_b, N, r, TILE_ROWS);
         } else {  // no TMA layout: rows padded to 32

@@ -324,8 +324,8 @@ cudaError_t launch_prefill_finish(const SeqState &s, const RowSeg *segs, const i
 // B [N, r] -> [N, 32], zero beyond r (standalone linear of many rows whose B has no TMA layout).
 cudaError_t launch_pack_b(const void *b, int N, int r, void *out, cudaStream_t st);
 
-// 2-D bf16 row-major [rows, cols] tensor map, box {64, box_rows}, 128-byte swizzle.
-bool encode_bf16_map(CUtensorMap *map, const void *base, int rows, int cols, int box_rows);
+// 2-D bf16 row-major [rows, cols] tensor map, rows ld values apart (0: cols), box {64, box_rows}, 128-byte swizzle.
+bool encode_bf16_map(CUtensorMap *map, const void *base, int rows, int cols, int box_rows, int ld = 0);
 
 // Per-instantiation kernel attributes (dynamic shared memory), set once before any capture.
 cudaError_t configure_linear_kernels();

@@ -88,6 +88,21 @@ def test_linear_stays_inside_its_workspace(torch, M, K, N, r):
     assert ((y.double() - ref).abs() <= tol).all()
 
 
+@pytest.mark.parametrize("M,K,r", [(17, 256, 1), (65, 256, 1), (70, 320, 3), (200, 256, 16), (65, 256, 32), (3, 4352, 5)])
+def test_linear_infinite_operand(torch, M, K, r):
+    """An infinite x among positive operands: its row is infinite, whatever the rank, and no other row is."""
+    from paper_2607_12422_gb300 import pbd
+    g = torch.Generator(device="cuda").manual_seed(M + r)
+    x, W = _rand(torch, g, (M, K), 1.0).abs(), _rand(torch, g, (256, K), 0.02).abs() + 0.01
+    A, B = _rand(torch, g, (r, K), 0.02).abs() + 0.01, _rand(torch, g, (256, r), 0.02).abs() + 0.01
+    ref, tol = _linear_ref(x, W, A, B, 2.0)
+    x[M // 2, 5] = float("inf")
+    y = pbd.pbd_op_linear(x, W, A, B, 2.0)
+    assert torch.isposinf(y[M // 2]).all()
+    rest = torch.arange(M, device="cuda") != M // 2
+    assert ((y.double() - ref).abs() <= tol)[rest].all()
+
+
 def test_linear_rows_do_not_depend_on_the_row_count(torch):
     from paper_2607_12422_gb300 import pbd
     g = torch.Generator(device="cuda").manual_seed(9)
