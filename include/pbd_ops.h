@@ -24,7 +24,8 @@ size_t pbd_op_linear_workspace_bytes(int32_t M, int32_t K, int32_t N, int32_t r)
  * d_x [M, K], d_w [N, K], d_a [r, K], d_b [N, r], d_y [M, N]: bf16, row-major, 16-byte aligned.
  * d_a == NULL or d_b == NULL (or r == 0) switches the delta off.  W and A are read in place; K is
  * summed in 256-wide slices in one fixed order, as in the decoder passes, so without the adapter a
- * row's result does not depend on M.  Requirements: N % 128 == 0, K % 64 == 0, 1 <= M <= 4096, r <= 32.
+ * row's result does not depend on M.  d_y may lie over an operand (one more copy of y).
+ * Requirements: N % 128 == 0, K % 64 == 0, 1 <= M <= 4096, r <= 32.
  * The workspace (d_ws, >= pbd_op_linear_workspace_bytes, 1024-byte aligned) is scratch; its first
  * word is the kernel's status word, cleared by each call and read by pbd_op_status.
  * The return value covers argument checks and launches only: a bounded device wait that ran out

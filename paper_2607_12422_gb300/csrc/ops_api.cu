@@ -98,12 +98,29 @@ pbd_status read_device_code(const int *d_status, cudaStream_t st, int *code, con
     return PBD_OK;
 }
 
+// whether [a, a + na) and [b, b + nb) share a byte
+static bool overlap(const void *a, size_t na, const void *b, size_t nb) {
+    const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+    return x < y + nb && y < x + na;
+}
+
 // Few rows (one operand tile of at most 64 tokens) and a K whose slices fit one cluster: linear_op.cu, one
 // launch that spreads the K slices over CTAs.  More rows: gemm.cu, whose CTAs keep whole tiles' sums in registers; the
 // adapter's u = bf16(x A^T) comes first, as one more such linear, and enters the tile as one more
 // MMA group.
 pbd_status run_linear_op(int M, int K, int N, int r, float scale, const void *d_x, const void *d_w, const void *d_a,
                          const void *d_b, void *d_y, const LinearScratch &ws, cudaStream_t st, const char *who) {
+    const size_t y_bytes = (size_t)M * N * 2;
+    if (overlap(d_y, y_bytes, d_x, (size_t)M * K * 2) || overlap(d_y, y_bytes, d_w, (size_t)N * K * 2) ||
+        (r > 0 && (overlap(d_y, y_bytes, d_a, (size_t)r * K * 2) || overlap(d_y, y_bytes, d_b, (size_t)N * r * 2)))) {
+        // The operands are read where they lie, by some CTAs after others have stored: y goes through the scratch.
+        // Of part's 4 M N bytes or more u takes the first 64 M (N is at least 128), y the second 2 M N.
+        uint8_t *y = ws.part + y_bytes;
+        const pbd_status s = run_linear_op(M, K, N, r, scale, d_x, d_w, d_a, d_b, y, ws, st, who);
+        if (s != PBD_OK) return s;
+        const cudaError_t e = cudaMemcpyAsync(d_y, y, y_bytes, cudaMemcpyDeviceToDevice, st);
+        return e == cudaSuccess ? PBD_OK : op_fail(PBD_ERR_CUDA, "copying an output that lies over an operand", e);
+    }
     auto bad = [&](pbd_status s, const char *what, cudaError_t e = cudaSuccess) {
         char b[160];
         snprintf(b, sizeof b, "%s: %s", who, what);

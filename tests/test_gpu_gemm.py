@@ -103,6 +103,34 @@ def test_linear_infinite_operand(torch, M, K, r):
     assert ((y.double() - ref).abs() <= tol)[rest].all()
 
 
+@pytest.mark.parametrize("M,K,N,r", [(17, 256, 256, 0), (64, 4096, 4096, 0), (64, 2048, 2048, 16), (4096, 2048, 2048, 0),
+                                     (300, 512, 512, 5), (1, 64, 128, 1), (65, 64, 128, 1)])
+@pytest.mark.parametrize("over", ["x", "W", "A", "B"])
+def test_linear_output_over_an_operand(torch, M, K, N, r, over):
+    """y may lie over an operand: the result is that of a y of its own, and nothing behind the workspace's or
+    y's end is written."""
+    from paper_2607_12422_gb300 import pbd
+    if over in "AB" and not r:
+        pytest.skip("no adapter")
+    lib = pbd.load()
+    g = torch.Generator(device="cuda").manual_seed(M + K + r)
+    ops = dict(x=_rand(torch, g, (M, K), 1.0), W=_rand(torch, g, (N, K), 0.02), A=_rand(torch, g, (max(r, 1), K), 0.02),
+               B=_rand(torch, g, (N, max(r, 1)), 0.02))
+    want = pbd.pbd_op_linear(ops["x"], ops["W"], *((ops["A"], ops["B"]) if r else ()), scale=2.0)
+    need, st = lib.pbd_op_linear_workspace_bytes(M, K, N, r), torch.cuda.current_stream().cuda_stream
+    ws = torch.full((need + 2048,), 0xA5, dtype=torch.uint8, device="cuda")
+    off = -ws.data_ptr() % 1024
+    size = max(M * N, ops[over].numel())
+    room = torch.full((size + 64,), 7.0, dtype=torch.bfloat16, device="cuda")  # the operand, and y over its start
+    room[:ops[over].numel()] = ops[over].flatten()
+    ptr = {k: (room if k == over else v).data_ptr() for k, v in ops.items()}
+    assert lib.pbd_op_linear(M, K, N, r, 2.0, ptr["x"], ptr["W"], ptr["A"] if r else None, ptr["B"] if r else None,
+                             room.data_ptr(), ws.data_ptr() + off, need, st) == 0
+    assert lib.pbd_op_status(ws.data_ptr() + off, st, None) == 0
+    assert torch.equal(room[:M * N].view(M, N), want)
+    assert (room[size:] == 7.0).all() and (ws[off + need:] == 0xA5).all()
+
+
 def test_linear_rows_do_not_depend_on_the_row_count(torch):
     from paper_2607_12422_gb300 import pbd
     g = torch.Generator(device="cuda").manual_seed(9)
