@@ -95,7 +95,8 @@ size_t pbd_op_lm_head_workspace_bytes(int32_t M, int32_t H, int32_t V);
  *     logits = x E^T (fp32, never rounded),  ids[m] = argmax_v logits[m, v], lowest v on ties.
  * d_x [M, H] and d_embed [V, H] bf16 row-major; d_ids [M] int32; d_logits_opt [M, V] fp32 or
  * NULL.  Requirements: V % 128 == 0, H % 64 == 0, 1 <= M <= 256.  The workspace's first word is
- * the kernel's status word: pbd_op_status(d_ws, ...) reports a device wait that ran out. */
+ * the kernel's status word: pbd_op_status(d_ws, ...) reports a device wait that ran out.  Its size
+ * counts a copy of d_embed, which is made only where d_logits_opt lies over d_embed. */
 pbd_status pbd_op_lm_head_argmax(int32_t M, int32_t H, int32_t V, const void *d_x, const void *d_embed,
                                  int32_t *d_ids, float *d_logits_opt, void *d_ws, size_t ws_bytes, void *d_stream);
 

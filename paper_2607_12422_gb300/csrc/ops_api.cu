@@ -259,8 +259,14 @@ pbd_status pbd_op_lm_head_argmax(int32_t M, int32_t H, int32_t V, const void *d_
     uint8_t *ws = static_cast<uint8_t *>(d_ws);
     int *status = reinterpret_cast<int *>(ws);
     const size_t tiles_bytes = (size_t)(V / TILE_ROWS) * (H / KT) * TILE_BYTES;
+    if (d_logits_opt && overlap(d_logits_opt, sizeof(float) * (size_t)M * V, d_embed, (size_t)V * H * 2)) {
+        // logits over the table that is read while they are stored: the table is read from a copy
+        const cudaError_t e = cudaMemcpyAsync(ws + 1024, d_embed, (size_t)V * H * 2, cudaMemcpyDeviceToDevice, st);
+        if (e != cudaSuccess) return op_fail(PBD_ERR_CUDA, "pbd_op_lm_head_argmax: copying the table", e);
+        d_embed = ws + 1024;
+    }
     TiledWeight w;
-    w.tiles = nullptr;  // read through w_map where the caller has it
+    w.tiles = nullptr;  // read through w_map
     w.n_main = V;
     w.lora_rows = 0;
     w.K = H;

@@ -160,6 +160,25 @@ def test_lm_head_edges(torch, M, H, V):
     assert none is None and torch.equal(plain, ids)
 
 
+@pytest.mark.parametrize("M,H,V", [(17, 256, 128 * 400), (136, 512, 128 * 320)])
+def test_lm_head_logits_over_the_table(torch, M, H, V):
+    from paper_2607_12422_gb300 import pbd
+    lib = pbd.load()
+    g = torch.Generator(device="cuda").manual_seed(M)
+    x, E = _rand(torch, g, (M, H), 1.0), _rand(torch, g, (V, H), 0.02)
+    ids, lg = pbd.pbd_op_lm_head_argmax(x, E, want_logits=True)
+    room = torch.empty(max(V * H, 2 * M * V), dtype=torch.bfloat16, device="cuda")
+    room[:V * H] = E.flatten()
+    need, st = lib.pbd_op_lm_head_workspace_bytes(M, H, V), torch.cuda.current_stream().cuda_stream
+    ws = torch.empty(need + 1024, dtype=torch.uint8, device="cuda")
+    off = -ws.data_ptr() % 1024
+    got = torch.empty(M, dtype=torch.int32, device="cuda")
+    assert lib.pbd_op_lm_head_argmax(M, H, V, x.data_ptr(), room.data_ptr(), got.data_ptr(), room.data_ptr(),
+                                     ws.data_ptr() + off, need, st) == 0
+    assert lib.pbd_op_status(ws.data_ptr() + off, st, None) == 0
+    assert torch.equal(room[:2 * M * V].view(torch.float32).view(M, V), lg) and torch.equal(got, ids)
+
+
 @pytest.mark.parametrize("shape,max_seq,start,rounds,ctas", [("tiny", 256, 1, 9, 0), ("qwen2", 420, 40, 21, 0),
                                                             ("qwen2", 4096, 301, 30, 0), ("grp4", 420, 17, 10, 0),
                                                             ("qwen2", 420, 130, 14, 20), ("tiny", 600, 130, 25, 4)])
