@@ -4,6 +4,7 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdio>
 #include <string>
 
@@ -104,10 +105,13 @@ static bool overlap(const void *a, size_t na, const void *b, size_t nb) {
     return x < y + nb && y < x + na;
 }
 
-// Few rows (one operand tile of at most 64 tokens) and a K whose slices fit one cluster: linear_op.cu, one
-// launch that spreads the K slices over CTAs.  More rows: gemm.cu, whose CTAs keep whole tiles' sums in registers; the
-// adapter's u = bf16(x A^T) comes first, as one more such linear, and enters the tile as one more
-// MMA group.
+// linear_op.cu, one launch that spreads the K slices over CTAs, or gemm.cu, whose CTAs keep whole tiles' sums in registers
+// and take all of K: up to 64 rows and 16 slices the first, beyond that the one with the shorter estimated
+// time.  Both ways, us per call with cold caches, rank 0 (and with re-tiling and split-K partial sums in
+// memory): M = 17, K = 16384, N = 128: 22 and 62 (28); M = 100, K = 4096, N = 128: 14 and 22 (26); M = 64,
+// K = 16384, N = 4096: 92 and 65 (127); M = 400, K = 3072, N = 1024: 31 and 19 (43).  With gemm.cu the adapter's
+// u = bf16(x A^T) comes first, one tile of features by either kernel (the whole of K in one CTA per 64 rows, or
+// spread: M = 100, K = 16384: 59 and 22 us), and enters the tile as one more MMA group.
 pbd_status run_linear_op(int M, int K, int N, int r, float scale, const void *d_x, const void *d_w, const void *d_a,
                          const void *d_b, void *d_y, const LinearScratch &ws, cudaStream_t st, const char *who) {
     const size_t y_bytes = (size_t)M * N * 2;
@@ -127,33 +131,39 @@ pbd_status run_linear_op(int M, int K, int N, int r, float scale, const void *d_
         return op_fail(s, b, e);
     };
     const int kt = K / KT, ks = kt % 4 == 0 ? kt / 4 : 1, f_tiles = N / TILE_ROWS;
-    const bool few = M <= LINEAR_OP_MAX_ROWS && ks <= LINEAR_OP_MAX_SLICES;
     int *status = reinterpret_cast<int *>(ws.status);
     cudaError_t e;
     if ((e = configure_linear_kernels()) != cudaSuccess) return bad(PBD_ERR_CUDA, "configure", e);
-    if (few) {
-        LinOpArgs a;
-        a.bn = M <= 32 ? 32 : 64;
-        if (!encode_bf16_map(&a.xmap, d_x, M, K, a.bn)) return bad(PBD_ERR_INVALID_ARG, "x not TMA-mappable");
-        if (!encode_bf16_map(&a.wmap, d_w, N, K, TILE_ROWS)) return bad(PBD_ERR_INVALID_ARG, "W not TMA-mappable");
+    // y[M][ld] = x w^T (+ the delta of rank ra) for the `rows` rows of w
+    auto op = [&](const void *w, int rows, int ld, int ra, void *y) {
+        LinOpArgs a{};
+        if (!encode_bf16_map(&a.xmap, d_x, M, K, linear_op_bn(M))) return bad(PBD_ERR_INVALID_ARG, "x not TMA-mappable");
+        if (!encode_bf16_map(&a.wmap, w, rows, K, TILE_ROWS))
+            return bad(PBD_ERR_INVALID_ARG, w == d_w ? "W not TMA-mappable" : "A not TMA-mappable");
         a.amap = a.wmap;
-        if (r > 0 && !encode_bf16_map(&a.amap, d_a, r, K, r)) return bad(PBD_ERR_INVALID_ARG, "A not TMA-mappable");
+        if (ra > 0 && !encode_bf16_map(&a.amap, d_a, ra, K, ra)) return bad(PBD_ERR_INVALID_ARG, "A not TMA-mappable");
         a.kt_per = kt / ks;
         a.ks = ks;
         a.M = M;
-        a.N = N;
-        a.r = r;
+        a.N = ld;
+        a.r = ra;
         a.scale = scale;
         a.b = static_cast<const bf16 *>(d_b);
-        a.y = static_cast<bf16 *>(d_y);
-        a.vec_store = (reinterpret_cast<uintptr_t>(d_y) & 7) == 0;
+        a.y = static_cast<bf16 *>(y);
+        a.vec_store = (reinterpret_cast<uintptr_t>(y) & 7) == 0;
         a.status = status;
+        const cudaError_t err = launch_linear_op(a, st);
+        return err == cudaSuccess ? PBD_OK : bad(PBD_ERR_CUDA, "linear", err);
+    };
+    const int bn = gemm_pick_bn(M, f_tiles, kt, 256, gemm_ctas());
+    const double u_gemm = gemm_us(M, 1, kt, 64), u_op = linear_op_us(M, 32, ks, kt / ks, 0) + 1.0;  // (+ a full launch)
+    if ((M <= LINEAR_OP_ROWS && ks <= LINEAR_OP_MAX_CLUSTER) ||
+        linear_op_us(M, N, ks, kt / ks, r) < gemm_us(M, f_tiles, kt, bn) + (r > 0 ? std::min(u_gemm, u_op) : 0.0)) {
         if ((e = cudaMemsetAsync(status, 0, 256, st)) != cudaSuccess) return bad(PBD_ERR_CUDA, "memset", e);
-        if ((e = launch_linear_op(a, st)) != cudaSuccess) return bad(PBD_ERR_CUDA, "linear", e);
-        return PBD_OK;
+        return op(d_w, N, N, r, d_y);
     }
     GemmArgs a{};
-    a.bn = gemm_pick_bn(M, f_tiles, kt, 256, gemm_ctas());
+    a.bn = bn;
     if (!encode_bf16_map(&a.xmap, d_x, M, K, a.bn)) return bad(PBD_ERR_INVALID_ARG, "x not TMA-mappable");
     if (!encode_bf16_map(&a.wmap, d_w, N, K, TILE_ROWS)) return bad(PBD_ERR_INVALID_ARG, "W not TMA-mappable");
     a.k_tiles = kt;
@@ -172,16 +182,21 @@ pbd_status run_linear_op(int M, int K, int N, int r, float scale, const void *d_
         // u [M][32] and a padded B [N][32].  Each fits its area whatever the sizes: `part` holds at least 512 bytes a row,
         // `tiles` 128 a column.  (Behind u, B would not: `part` is small for few rows.)
         uint8_t *u = ws.part, *bp = ws.tiles;
-        GemmArgs g = a;
-        g.bn = 64;
-        if (!encode_bf16_map(&g.xmap, d_x, M, K, g.bn)) return bad(PBD_ERR_INVALID_ARG, "x not TMA-mappable");
-        if (!encode_bf16_map(&g.wmap, d_a, r, K, TILE_ROWS)) return bad(PBD_ERR_INVALID_ARG, "A not TMA-mappable");
-        g.f_tiles = 1;
-        g.rows = 32;
-        g.y = reinterpret_cast<bf16 *>(u);
-        g.ld = 32;
-        g.vec_store = 1;
-        if ((e = launch_gemm(GEMM_Y, g, 0, st)) != cudaSuccess) return bad(PBD_ERR_CUDA, "adapter rows", e);
+        if (u_op < u_gemm) {
+            const pbd_status s = op(d_a, r, 32, 0, u);
+            if (s != PBD_OK) return s;
+        } else {
+            GemmArgs g = a;
+            g.bn = 64;
+            if (!encode_bf16_map(&g.xmap, d_x, M, K, g.bn)) return bad(PBD_ERR_INVALID_ARG, "x not TMA-mappable");
+            if (!encode_bf16_map(&g.wmap, d_a, r, K, TILE_ROWS)) return bad(PBD_ERR_INVALID_ARG, "A not TMA-mappable");
+            g.f_tiles = 1;
+            g.rows = 32;
+            g.y = reinterpret_cast<bf16 *>(u);
+            g.ld = 32;
+            g.vec_store = 1;
+            if ((e = launch_gemm(GEMM_Y, g, 0, st)) != cudaSuccess) return bad(PBD_ERR_CUDA, "adapter rows", e);
+        }
         a.delta = 1;
         // (r columns: the rest arrive as zeros.  What the kernel computed there, 0 x, is NaN where x is infinite.)
         bool ok = encode_bf16_map(&a.umap, u, M, r, a.bn, 32);

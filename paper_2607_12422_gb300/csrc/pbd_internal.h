@@ -230,19 +230,23 @@ __device__ __forceinline__ const bf16 *tiled_at(const bf16 *tiles, int K, int v,
 
 // ---- launchers (each returns cudaGetLastError()) ----
 
-// Standalone linear of few rows (linear_op.cu), one launch.
+// Standalone linear of few rows, or of few columns and a long K (linear_op.cu), one launch.  The caller fills
+// everything but the last line.
 struct LinOpArgs {
-    CUtensorMap xmap, wmap, amap;  // boxes {64, bn}, {64, 128}, {64, r}
-    int bn, kt_per, ks, M, N, r;   // kt_per: 64-wide K atoms per slice; ks <= LINEAR_OP_MAX_SLICES
+    CUtensorMap xmap, wmap, amap;  // boxes {64, linear_op_bn(M)}, {64, 128}, {64, r}
+    int kt_per, ks, M, N, r;       // kt_per: 64-wide K atoms per slice; N: columns of y (the weight's rows, or more)
     float scale;
     const bf16 *b;
     bf16 *y;
-    int vec_store;  // y is 8-byte aligned
+    int vec_store;  // y is 8-byte aligned and N a multiple of 4
     int *status;
+    int bn, cs, groups, stages;
 };
-constexpr int LINEAR_OP_MAX_ROWS = 64;
-constexpr int LINEAR_OP_MAX_SLICES = 16;  // one cluster
-cudaError_t launch_linear_op(const LinOpArgs &a, cudaStream_t st);
+constexpr int LINEAR_OP_ROWS = 64;         // token rows of a CTA
+constexpr int LINEAR_OP_MAX_CLUSTER = 16;
+int linear_op_bn(int M);
+double linear_op_us(int M, int N, int ks, int kt_per, int r);  // estimated time beyond an empty launch's
+cudaError_t launch_linear_op(LinOpArgs &a, cudaStream_t st);
 cudaError_t configure_linear_op();
 
 // Linears of many rows (gemm.cu).  The caller fills everything but the last line.
@@ -269,6 +273,7 @@ struct GemmArgs {
 // ctas: CTAs at most (0: one per SM)
 cudaError_t launch_gemm(GemmMode mode, GemmArgs &a, int ctas, cudaStream_t st);
 int gemm_pick_bn(int M, int f_tiles, int k_tiles, int max_bn, int ctas);
+double gemm_us(int M, int f_tiles, int k_tiles, int bn);  // estimated time of a GEMM_Y launch beyond an empty one's
 int gemm_ctas();  // CTAs of a launch with ctas = 0
 cudaError_t configure_gemm_kernels();
 
