@@ -428,4 +428,26 @@ cudaError_t launch_pdl(void (*kernel)(P...), int grid, int threads, size_t smem,
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
+// CTAs of the largest cluster (along y, up to `most`) that the current device can hold of `kernel`, whose attributes
+// are set.  Up to 8 always can; beyond that it takes a GPC with as many free SMs.
+inline int largest_cluster(const void *kernel, int threads, size_t smem, int most) {
+    for (int c = most; c > 8; --c) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(1, (unsigned)c);
+        cfg.blockDim = dim3((unsigned)threads);
+        cfg.dynamicSmemBytes = smem;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = 1;
+        attr[0].val.clusterDim.y = (unsigned)c;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n > 0) return c;
+        cudaGetLastError();  // (the answer is not an error of a later call)
+    }
+    return 8;
+}
+
 }  // namespace pbd

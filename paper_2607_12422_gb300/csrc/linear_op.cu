@@ -295,11 +295,12 @@ cudaError_t configure_linear_op() {
 
 int linear_op_bn(int M) { return M <= 32 ? 32 : 64; }
 
-// CTAs of a tile's cluster: groups of as equal a size as it gets (17 slices: two of 9 and 8), so that with several
-// groups a cluster has at least 9 CTAs and a row of 64 a warp of its own.
+// CTAs of a tile's cluster: groups of as equal a size as it gets (17 slices: two of 9 and 8), but with several groups
+// at least 8, so that each of 64 rows has a warp of its own.
 static int lo_cluster(int ks) {
-    const int groups = (ks + LINEAR_OP_MAX_CLUSTER - 1) / LINEAR_OP_MAX_CLUSTER;
-    return (ks + groups - 1) / groups;
+    static const int most = largest_cluster((const void *)k_linear_op<false>, LO_THREADS, LO_SMEM_MAX, LINEAR_OP_MAX_CLUSTER);
+    const int groups = (ks + most - 1) / most;
+    return groups == 1 ? ks : std::max(8, (ks + groups - 1) / groups);
 }
 
 // Per group: a chain of dependent steps, the slice's atoms, and the rows that a warp sums (and finishes) one after

@@ -931,6 +931,14 @@ static int attn_cluster(const Dims &dm, const PassDesc &pd, int subs, int nsplit
     return c >= nsplit && pd.nb * dm.Hkv * c <= gemm_ctas() && *smem <= (size_t)ST_SMEM ? c : 0;
 }
 
+// Slices of a linear at most: one cluster, and one that the device can place (0.6B shape but the hidden size, us a layer
+// of a verify pass, persistent kernel in brackets: 12 slices 57 (85), 13 64 (118), 14 72 (109), 15 93 (131), 16 76
+// (114); a draft 93 (102), 138 (138), 116 (130), 159 (157), 126 (137)).
+static int max_slices() {
+    static const int n = largest_cluster((const void *)k_step_linear<0, true, 128, 512>, 512, ST_SMEM, ST_MAX_CLUSTER);
+    return n;
+}
+
 bool step_pass_fits(const Dims &dm, const PassDesc &pd, int subs, int nsplit) {
     const int K[4] = {dm.H, dm.Hq * dm.d, dm.H, dm.I};
     const int bn = step_bn(pd.M);
@@ -940,7 +948,7 @@ bool step_pass_fits(const Dims &dm, const PassDesc &pd, int subs, int nsplit) {
         const int ks = K[lin] / (ka * KT), ru = pd.adapter ? (lin == 2 ? 2 : 1) * dm.r : 0;
         int push;
         size_t smem;
-        if (ks > ST_MAX_CLUSTER || lin_ring(bn, pd.M, ka, ks, pd.adapter, ru, &push, &smem) == 0) return false;
+        if (ks > max_slices() || lin_ring(bn, pd.M, ka, ks, pd.adapter, ru, &push, &smem) == 0) return false;
     }
     // (statistics a merging warp holds; a split's pages and the group's q rows)
     return nsplit * subs <= 32 * SA_STATS && attn_smem(dm, pd.R, 0, 0) <= ST_SMEM;

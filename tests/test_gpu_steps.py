@@ -26,6 +26,9 @@ def _shape(name):
         "qwen2": two,
         "grp4": dataclasses.replace(two, n_kv_heads=4, hidden=768, intermediate=1280),
         "grp1-d64": dataclasses.replace(synth.TINY, n_q_heads=8, n_kv_heads=8, hidden=512, intermediate=512, vocab=1024),
+        # 13 and 16 K slices: clusters beyond the portable size
+        "h3328": dataclasses.replace(two, n_layers=1, hidden=3328, vocab=512),
+        "h4096": dataclasses.replace(two, n_layers=1, hidden=4096, n_q_heads=32, n_kv_heads=16, intermediate=4096, vocab=512),
         "r8": dataclasses.replace(two, lora_rank=8, lora_alpha=16.0),
     }[name]
 
@@ -46,6 +49,8 @@ CASES = [
     ("grp4", 16, (333, 40), 500, {}),
     ("grp1-d64", 8, (150, 33), 300, {}),
     ("r8", 16, (140,), 300, {}),
+    ("h3328", 16, (140,), 300, {}),
+    ("h4096", 16, (40, 200), 300, {}),
 ]
 
 
