@@ -74,10 +74,12 @@ typedef struct {
                                  writes no K/V there); 0 = none.  Bits at or above n_layers must be
                                  clear, and the draft must keep at least one layer (together with
                                  draft_layers) */
-    int32_t max_ctas;         /* 0 = the whole GPU; otherwise at most max_ctas CTAs at a time (leaving SMs
-                                 to other work): decoding passes then run as the persistent pass kernel.  It must be at least the largest
-                                 number of K slices of one linear, whose reductions wait for one
-                                 another and so must sit on distinct CTAs: pbd_create fails with
+    int32_t max_ctas;         /* 0 = the whole GPU; otherwise each kernel of the decoder layers launches at
+                                 most max_ctas CTAs (leaving SMs to other work), and decoding passes run
+                                 as the persistent pass kernel.  The lm_head and the small kernels
+                                 around the layers use the whole GPU all the same.  It must be at least
+                                 the largest number of K slices of one linear, whose reductions wait for
+                                 one another and so must sit on distinct CTAs: pbd_create fails with
                                  PBD_ERR_INVALID_ARG below that */
 } pbd_config;
 
