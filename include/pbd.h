@@ -214,13 +214,17 @@ pbd_status pbd_time_pass(pbd_ctx *ctx, int32_t kind, int32_t iters, double *h_ms
 pbd_status pbd_trace_pass(pbd_ctx *ctx, int32_t kind, int32_t *h_items, uint64_t *h_trace, int32_t cap,
                           int32_t *h_n);
 
-/* Failure-detection check (no GPU fault is involved).  On a prefilled context, runs one verify
- * pass whose schedule lacks the first q|k|v item of layer 0: that item's partial sums never
- * arrive, so the waits polling for them run out after their bound (1 s), latch a device code
- * and end the pass.  Returns PBD_ERR_DEVICE with the latched code in *h_device_code (a
- * DEV_TIMEOUT_* value; 0 would mean the pass ended without noticing).  The cached tokens and
- * the decoding state are untouched (the pass writes scratch slots only) and the context stays
- * usable: the normal schedules are restored before returning.  Synchronous. */
+/* Failure-detection check (no GPU fault is involved).  On a prefilled context, makes bounded waits
+ * run out (after 1 s each) in the kernels that the context uses:
+ *   - a verify pass as it decodes them: the kernel chain, once with too few bytes of one linear's
+ *     activations and once of the attention's K pages; or, where the persistent kernel runs
+ *     (max_ctas, shapes that do not fit the chain), a schedule without the first q|k|v item of
+ *     layer 0, whose partial sums never arrive;
+ *   - the prompt kernels over the same rows, in the same two ways.
+ * Each wait that gives up latches a device code and ends its kernel.  Returns PBD_ERR_DEVICE with the
+ * first latched code in *h_device_code (a DEV_TIMEOUT_* value), or PBD_OK with 0 if one of the passes
+ * ended without noticing.  The cached tokens and the decoding state are untouched (the passes write
+ * scratch slots only) and the context stays usable.  Synchronous. */
 pbd_status pbd_check_stalled_pass(pbd_ctx *ctx, int32_t *h_device_code);
 
 /* The work schedule of one pass, computed on the host with no context and no GPU (for checks

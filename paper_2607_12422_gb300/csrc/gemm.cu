@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(GM_THREADS, 1) k_gemm(const __grid_constant__ 
             }
             if (*(volatile int *)&S.abort)  // error path: the copies in flight get a bounded chance to land
                 for (int h = issued > nst ? issued - nst : 0; h < issued; ++h)
-                    mbar_wait(&S.full[h % nst], (h / nst) & 1, nullptr, 0, nullptr);
+                    if (!mbar_wait(&S.full[h % nst], (h / nst) & 1, nullptr, 0, nullptr)) break;  // (all had this second)
         } else if (warp == 1 && elect_one()) {
             // ---- MMA issuer
             const uint32_t idesc = idesc_bf16_f32(128, a.bn);

@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(LO_THREADS, 2) k_linear_op(const __grid_consta
             }
             if (!dead && *(volatile int *)&s_abort) {  // error path: the copies in flight get a bounded chance to land
                 for (int h = sent > a.stages ? sent - a.stages : 0; h < sent; ++h)
-                    mbar_wait(&full[h % a.stages], (h / a.stages) & 1, nullptr, 0, nullptr);
+                    if (!mbar_wait(&full[h % a.stages], (h / a.stages) & 1, nullptr, 0, nullptr)) break;  // (all had this second)
                 dead = true;
             }
         } else if (warp == 1 && (ONE || (g < mine && !dead)) && elect_one()) {

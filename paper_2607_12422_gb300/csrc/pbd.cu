@@ -583,9 +583,21 @@ pbd_status ensure_schedule(pbd_ctx *c, int kind, const PassDesc &pd) {
     return c->sched[kind].valid ? PBD_OK : upload_schedule(c, kind, pd, decode_splits(c));
 }
 
+// What a pass is made to wait for in vain (pbd_check_stalled_pass): in its first layer, copies of one linear's
+// activations, or of the attention's K pages, that bring fewer bytes than the kernel counts on.
+enum Stall { STALL_NONE = 0, STALL_LINEAR, STALL_ATTN };
+
+// K map whose boxes hold half a page
+pbd_status short_kmap(pbd_ctx *c, CUtensorMap *m) {
+    const int kv_rows = c->cfg.n_layers * c->n_pages * c->cfg.n_kv_heads * PAGE;
+    return encode_bf16_map(m, c->kv.k, kv_rows, c->cfg.head_dim, PAGE / 2) ? PBD_OK : fail(c, PBD_ERR_CUDA, "tensor map encode failed");
+}
+
 // All decoder layers of a pass as a chain of kernels; nsplit: 128-key splits per sequence.
-pbd_status enqueue_steps(pbd_ctx *c, const PassDesc &pd, const std::vector<int> &nsplit) {
+pbd_status enqueue_steps(pbd_ctx *c, const PassDesc &pd, const std::vector<int> &nsplit, Stall stall = STALL_NONE) {
     const pbd_config &k = c->cfg;
+    CUtensorMap half = c->kmap;
+    if (stall == STALL_ATTN) TRY(short_kmap(c, &half));
     StepSplits sp{};
     for (int b = 0; b < pd.nb; ++b) sp.start[b + 1] = sp.start[b] + nsplit[b];
     StepArgs a{};
@@ -621,8 +633,9 @@ pbd_status enqueue_steps(pbd_ctx *c, const PassDesc &pd, const std::vector<int> 
             w.q_norm = static_cast<const bf16 *>(c->q_norm) + (size_t)l * k.head_dim;
             w.k_norm = static_cast<const bf16 *>(c->k_norm) + (size_t)l * k.head_dim;
             w.lora_b = static_cast<const bf16 *>(c->lb[lin]) + (size_t)l * w.n_main * k.lora_rank;
+            w.short_x = stall == STALL_LINEAR && l == 0 && lin == 1;
             CK(launch_step_linear(lin, a, w, c->st));
-            if (lin == 0) CK(launch_step_attn(a, c->kmap, c->vmap, l, sp, c->st));
+            if (lin == 0) CK(launch_step_attn(a, l == 0 ? half : c->kmap, c->vmap, l, sp, c->st));
         }
     }
     if (pd.ro_count > 0) CK(launch_step_final(a, c->final_norm, c->x_ro, c->st));
@@ -703,8 +716,9 @@ pbd_status enqueue_decode_commit(pbd_ctx *c) {
     return PBD_OK;
 }
 
-// One linear of a pass over prompt rows (adapter off): y[M][n] from the rows behind `maps`.
-pbd_status rows_linear(pbd_ctx *c, int lin, int layer, int M, const CUtensorMap *maps, void *y) {
+// One linear of a pass over prompt rows (adapter off): y[M][n] from the rows behind `maps`; stall: the rows of x in
+// boxes half as high as the smallest.
+pbd_status rows_linear(pbd_ctx *c, int lin, int layer, int M, const CUtensorMap *maps, void *y, bool stall = false) {
     const TiledWeight &w = c->w[lin][layer];
     const GemmMode mode = lin == 2 ? GEMM_GATE_UP : GEMM_Y;
     GemmArgs a{};
@@ -718,6 +732,8 @@ pbd_status rows_linear(pbd_ctx *c, int lin, int layer, int M, const CUtensorMap 
     a.bn = gemm_pick_bn(M, a.f_tiles, mode == GEMM_GATE_UP ? 2 * a.k_tiles : a.k_tiles, mode == GEMM_GATE_UP ? 128 : 256,
                         c->grid);
     a.xmap = maps[a.bn / 32 - 1];
+    if (stall && !encode_bf16_map(&a.xmap, c->rows.x, c->rows.cap, c->cfg.hidden, 16))
+        return fail(c, PBD_ERR_CUDA, "tensor map encode failed");
     a.y = static_cast<bf16 *>(y);
     a.vec_store = 1;
     a.status = c->status;
@@ -728,8 +744,11 @@ pbd_status rows_linear(pbd_ctx *c, int lin, int layer, int M, const CUtensorMap 
 // A causal adapter-off pass over prompt rows: `segs` (ascending rows) with their token ids behind
 // d_ids.  Segments listed in `ro` end their prompt: their first tokens are picked and the
 // sequences' state is set.
-pbd_status enqueue_rows_pass(pbd_ctx *c, const std::vector<RowSeg> &segs, const std::vector<int> &ro, const int32_t *d_ids) {
+pbd_status enqueue_rows_pass(pbd_ctx *c, const std::vector<RowSeg> &segs, const std::vector<int> &ro, const int32_t *d_ids,
+                             Stall stall = STALL_NONE) {
     const pbd_config &k = c->cfg;
+    CUtensorMap half = c->kmap;
+    if (stall == STALL_ATTN) TRY(short_kmap(c, &half));
     RowsBuf &rw = c->rows;
     const int grp = k.n_q_heads / k.n_kv_heads, tile = rows_attn_tile();
     RowsArgs a{};
@@ -765,9 +784,9 @@ pbd_status enqueue_rows_pass(pbd_ctx *c, const std::vector<RowSeg> &segs, const 
     auto gain = [&](void *g, int l) { return static_cast<const uint8_t *>(g) + H2 * l; };
     CK(launch_rows_embed(a, d_ids, c->w_lm.tiles, c->attn_norm, c->st));
     for (int l = 0; l < k.n_layers; ++l) {
-        TRY(rows_linear(c, 0, l, a.M, rw.xm, rw.qkv));
+        TRY(rows_linear(c, 0, l, a.M, rw.xm, rw.qkv, stall == STALL_LINEAR && l == 0));
         CK(launch_rows_rope(a, l, c->q_norm, c->k_norm, c->rope_cs, c->st));
-        CK(launch_rows_attn(a, c->kmap, c->vmap, l, rw.work, (int)work.size(), c->st));
+        CK(launch_rows_attn(a, l == 0 ? half : c->kmap, c->vmap, l, rw.work, (int)work.size(), c->st));
         TRY(rows_linear(c, 1, l, a.M, rw.attnm, rw.y));
         CK(launch_rows_norm(a, gain(c->mlp_norm, l), c->st));
         TRY(rows_linear(c, 2, l, a.M, rw.xm, rw.act));
@@ -844,16 +863,22 @@ pbd_status enqueue_short_prompt(pbd_ctx *c, int P, const int32_t *d_ids) {
     return PBD_OK;
 }
 
-pbd_status check_device(pbd_ctx *c) {
-    int code = 0;
-    CK(cudaMemcpyAsync(&code, c->status, sizeof(int), cudaMemcpyDeviceToHost, c->st));
+// Waits for the stream and takes the latched device code (0: none): it is reported once, and the context stays usable.
+pbd_status take_status(pbd_ctx *c, int *code) {
+    *code = 0;
+    CK(cudaMemcpyAsync(code, c->status, sizeof(int), cudaMemcpyDeviceToHost, c->st));
     CK(cudaStreamSynchronize(c->st));
-    if (code != 0) {
-        CK(cudaMemsetAsync(c->status, 0, sizeof(int), c->st));  // reported once; the context stays usable
+    if (*code != 0) {
+        CK(cudaMemsetAsync(c->status, 0, sizeof(int), c->st));
         CK(cudaStreamSynchronize(c->st));
-        return fail(c, PBD_ERR_DEVICE, "device status %d latched by a kernel", code);
     }
     return PBD_OK;
+}
+
+pbd_status check_device(pbd_ctx *c) {
+    int code;
+    TRY(take_status(c, &code));
+    return code == 0 ? PBD_OK : fail(c, PBD_ERR_DEVICE, "device status %d latched by a kernel", code);
 }
 
 // Everything a prefill does once its arguments are checked.
@@ -894,6 +919,38 @@ pbd_status start_generation(pbd_ctx *c, int batch, const int32_t *d_prompt_ids, 
         if (!c->steps[kind]) TRY(upload_schedule(c, kind, pd, ns));
     }
     return PBD_OK;
+}
+
+// The persistent kernel's verify pass without its first q|k|v item of layer 0; the normal schedule again afterwards.
+pbd_status stalled_pass_kernel(pbd_ctx *c, const PassDesc &pd, int *code) {
+    const std::vector<int> ns = decode_splits(c);
+    std::vector<MKItem> all, items;
+    std::vector<int> off;
+    mk_build_schedule(c->dm, pd, ns, 1, c->cl, &all, &off);  // one CTA: the items in order
+    bool dropped = false;
+    for (const MKItem &it : all) {
+        if (!dropped && it.op == MK_LINEAR && it.lin == 0 && it.layer == 0) {
+            dropped = true;
+            continue;
+        }
+        items.push_back(it);
+    }
+    // deal the remaining items round-robin, as mk_build_schedule does
+    std::vector<int> cta_off(c->grid + 1, 0);
+    for (size_t i = 0; i < items.size(); ++i) cta_off[i % c->grid + 1]++;
+    for (int k = 0; k < c->grid; ++k) cta_off[k + 1] += cta_off[k];
+    std::vector<MKItem> dealt(items.size());
+    std::vector<int> fill(cta_off.begin(), cta_off.end() - 1);
+    for (size_t i = 0; i < items.size(); ++i) dealt[fill[i % c->grid]++] = items[i];
+    Sched &sv = c->sched[PK_VERIFY];
+    TRY(ensure_schedule(c, PK_VERIFY, pd));  // (its split counts)
+    CK(cudaMemcpyAsync(sv.items, dealt.data(), dealt.size() * sizeof(MKItem), cudaMemcpyHostToDevice, c->st));
+    CK(cudaMemcpyAsync(sv.off, cta_off.data(), cta_off.size() * sizeof(int), cudaMemcpyHostToDevice, c->st));
+    CK(cudaStreamSynchronize(c->st));
+    TRY(enqueue_pass_kernel(c, pd, PK_VERIFY));
+    TRY(take_status(c, code));
+    sv.valid = false;
+    return c->steps[PK_VERIFY] ? PBD_OK : upload_schedule(c, PK_VERIFY, pd, ns);
 }
 
 double pass_bytes(pbd_ctx *c, int kind, const std::vector<int> &Ls) {
@@ -1360,41 +1417,26 @@ pbd_status pbd_check_stalled_pass(pbd_ctx *c, int32_t *h_device_code) {
     if (!c || !h_device_code) return fail(c, PBD_ERR_INVALID_ARG, "null argument");
     if (c->phase != PH_READY) return fail(c, PBD_ERR_STATE, "the check needs a prefilled or committed state");
     const PassDesc pd = block_pass(c, PK_VERIFY);
-    const std::vector<int> ns = decode_splits(c);
-    std::vector<MKItem> all, items;
-    std::vector<int> off;
-    mk_build_schedule(c->dm, pd, ns, 1, c->cl, &all, &off);  // one CTA: the items in order
-    bool dropped = false;
-    for (const MKItem &it : all) {
-        if (!dropped && it.op == MK_LINEAR && it.lin == 0 && it.layer == 0) {
-            dropped = true;
-            continue;
-        }
-        items.push_back(it);
-    }
-    // deal the remaining items round-robin, as mk_build_schedule does
-    std::vector<int> cta_off(c->grid + 1, 0);
-    for (size_t i = 0; i < items.size(); ++i) cta_off[i % c->grid + 1]++;
-    for (int k = 0; k < c->grid; ++k) cta_off[k + 1] += cta_off[k];
-    std::vector<MKItem> dealt(items.size());
-    std::vector<int> fill(cta_off.begin(), cta_off.end() - 1);
-    for (size_t i = 0; i < items.size(); ++i) dealt[fill[i % c->grid]++] = items[i];
-    Sched &sv = c->sched[PK_VERIFY];
-    TRY(ensure_schedule(c, PK_VERIFY, pd));  // (its split counts)
-    CK(cudaMemcpyAsync(sv.items, dealt.data(), dealt.size() * sizeof(MKItem), cudaMemcpyHostToDevice, c->st));
-    CK(cudaMemcpyAsync(sv.off, cta_off.data(), cta_off.size() * sizeof(int), cudaMemcpyHostToDevice, c->st));
-    CK(cudaStreamSynchronize(c->st));
     CK(launch_build_ids(pd, 1, c->s.pending, c->draft_ids, c->D, c->ids, c->st));
-    TRY(enqueue_pass_kernel(c, pd, PK_VERIFY));
+    // what the context decodes with, then the prompt kernels, over the verify pass's rows of sequence 0
+    int codes[4] = {0, 0, 0, 0}, n = 0, L0 = 0;
+    if (c->steps[PK_VERIFY]) {
+        for (Stall s : {STALL_LINEAR, STALL_ATTN}) {
+            TRY(enqueue_steps(c, pd, c->nsplit, s));
+            TRY(take_status(c, &codes[n++]));
+        }
+    } else {
+        TRY(stalled_pass_kernel(c, pd, &codes[n++]));
+    }
+    CK(cudaMemcpyAsync(&L0, c->s.L, sizeof(int), cudaMemcpyDeviceToHost, c->st));
     CK(cudaStreamSynchronize(c->st));
-    int code = 0;
-    CK(cudaMemcpy(&code, c->status, sizeof(int), cudaMemcpyDeviceToHost));
-    *h_device_code = code;
-    // the normal verify schedule again, where verify passes use it; the device code is reported (and cleared)
-    // below
-    c->sched[PK_VERIFY].valid = false;
-    if (!c->steps[PK_VERIFY]) TRY(upload_schedule(c, PK_VERIFY, pd, ns));
-    return check_device(c);
+    for (Stall s : {STALL_LINEAR, STALL_ATTN}) {
+        TRY(enqueue_rows_pass(c, {RowSeg{0, 0, L0, std::min(pd.R, c->rows.cap)}}, {}, c->ids, s));
+        TRY(take_status(c, &codes[n++]));
+    }
+    *h_device_code = *std::min_element(codes, codes + n) == 0 ? 0 : codes[0];
+    if (*h_device_code == 0) return PBD_OK;  // (one of them ended without noticing)
+    return fail(c, PBD_ERR_DEVICE, "device status %d latched by a kernel", codes[0]);
 }
 
 pbd_status pbd_trace_pass(pbd_ctx *c, int32_t kind, int32_t *h_items, uint64_t *h_trace, int32_t cap, int32_t *h_n) {

@@ -167,6 +167,7 @@ struct StepLin {
     const uint8_t *tiles;      // this layer's weight, pre-tiled, the adapter's rows in the last tile
     const bf16 *gain, *q_norm, *k_norm, *lora_b;  // this layer's
     int layer, K, n_main;
+    int short_x;               // (host, linears 1 and 3) the activations' copies bring fewer bytes than the kernel waits for
     // set by the launcher
     CUtensorMap xmap;
     int k_tiles, katoms, ks, ring_atoms, push;

@@ -379,7 +379,7 @@ __global__ void __launch_bounds__(RA_THREADS, 2)
             }
             if (*(volatile int *)&S.abort)  // error path: the copies in flight get a bounded chance to land
                 for (int h = issued > RA_RING ? issued - RA_RING : 0; h < issued; ++h)
-                    mbar_wait(&S.full[h % RA_RING], (h / RA_RING) & 1, nullptr, 0, nullptr);
+                    if (!mbar_wait(&S.full[h % RA_RING], (h / RA_RING) & 1, nullptr, 0, nullptr)) break;  // (all had this second)
         } else if (warp == 5 && elect_one()) {
             // ---- MMA warp
             const uint32_t ids = idesc_bf16_f32(128, RA_KEYS), ido = idesc_bf16_f32(128, DH) | IDESC_B_MN;

@@ -1005,7 +1005,8 @@ cudaError_t launch_step_linear(int lin, StepArgs &a, StepLin &w, cudaStream_t st
     w.tmem_cols = 32;
     while ((int)w.tmem_cols < (ad ? 2 : 1) * a.bn) w.tmem_cols <<= 1;
     if (lin == 1 || lin == 3)
-        if (!encode_bf16_map(&w.xmap, lin == 1 ? (const void *)a.attn : (const void *)a.act, a.rows_alloc, w.K, a.bn))
+        if (!encode_bf16_map(&w.xmap, lin == 1 ? (const void *)a.attn : (const void *)a.act, a.rows_alloc, w.K,
+                             w.short_x ? a.bn - 16 : a.bn))
             return cudaErrorInvalidValue;
     const dim3 grid(w.n_main / TILE_ROWS, w.ks);
     if (lin_threads(a.pd.M) == 256)

@@ -432,7 +432,7 @@ class Engine:
         return items[: 4 * k].reshape(k, 4), tr[: TRACE_STAMPS * k].reshape(k, TRACE_STAMPS)
 
     def pbd_check_stalled_pass(self):
-        """(status, device code) of a verify pass missing one item (see include/pbd.h)."""
+        """(status, device code) of passes made to wait in vain (see include/pbd.h)."""
         code = np.zeros(1, np.int32)
         status = self.lib.pbd_check_stalled_pass(self.ctx, code.ctypes.data)
         return int(status), int(code[0])

@@ -139,6 +139,30 @@ def test_refused_prefill_leaves_no_generation(torch):
     fresh.close()
 
 
+@pytest.mark.parametrize("P,max_seq,ctas", [(40, 256, 0), (1100, 1400, 0), (40, 256, 4)])
+def test_waits_that_run_out_are_reported(torch, P, max_seq, ctas):
+    """Every kind of pass that a context runs is made to wait in vain (kernel chain, with the attention merged in a
+    cluster or through memory; persistent kernel; prompt kernels): the codes are reported, the committed K/V and
+    the state are what they were, and the same context then decodes what a new one decodes."""
+    from paper_2607_12422_gb300 import pbd, synth
+    S = _shape("tiny")
+    base, ad = synth.gen_base_weights(S), synth.gen_adapter(S)
+    p = np.random.default_rng(P).integers(0, S.vocab, P).astype(np.int32)
+    eng = pbd.Engine(S, base, ad, block_D=16, max_batch=1, max_seq_len=max_seq, max_ctas=ctas)
+    want = eng.pbd_generate([p], 40)[0].clone()
+    eng.pbd_prefill([p], max_new=40)
+    kv, state = [eng.pbd_read_kv(l, 0, P) for l in range(S.n_layers)], eng.pbd_get_state()
+    status, code = eng.pbd_check_stalled_pass()
+    assert status == 6 and code in (1, 2, 3, 6)  # PBD_ERR_DEVICE, DEV_TIMEOUT_*
+    for l in range(S.n_layers):
+        assert all(torch.equal(x, y) for x, y in zip(kv[l], eng.pbd_read_kv(l, 0, P)))
+    assert all(np.array_equal(x, y) for x, y in zip(state, eng.pbd_get_state()))
+    got = [state[1][0]] + [int(eng.pbd_decode_step()[0][0]) for _ in range(39)]
+    assert got == [int(t) for t in want[0].cpu()]
+    assert torch.equal(eng.pbd_generate([p], 40)[0], want)
+    eng.close()
+
+
 @pytest.mark.parametrize("shape,P", [("qwen2", 33), ("qwen2", 127), ("qwen2", 128), ("qwen2", 129), ("tiny", 100)])
 def test_prompt_of_few_tokens_equals_the_many_row_kernels(torch, shape, P):
     """A lone prompt up to the chain's limit is one decoding pass; in a batch it goes through the many-row
