@@ -1085,6 +1085,8 @@ pbd_status pbd_create(const pbd_config *cfg, const pbd_base_weights *base, const
     if (e != cudaSuccess || (e = cudaMemsetAsync(c->cnt, 0, sizeof(int) * (size_t)(c->cl.total + 2), c->st)) != cudaSuccess ||
         (e = cudaMemsetAsync(c->kv.k, 0, kv_bytes, c->st)) != cudaSuccess ||
         (e = cudaMemsetAsync(c->kv.v, 0, kv_bytes, c->st)) != cudaSuccess ||
+        // (passes that are timed, traced or checked before the first draft verify these)
+        (e = cudaMemsetAsync(c->draft_ids, 0, sizeof(int) * cfg->max_batch * c->D, c->st)) != cudaSuccess ||
         (e = cudaMemsetAsync(c->status, 0, 64, c->st)) != cudaSuccess ||
         (e = cudaStreamSynchronize(c->st)) != cudaSuccess) {
         s = fail(c, PBD_ERR_CUDA, "workspace init: %s", cudaGetErrorString(e));

@@ -139,6 +139,20 @@ def test_refused_prefill_leaves_no_generation(torch):
     fresh.close()
 
 
+def test_pass_before_the_first_draft(torch):
+    """A verify pass that is timed before anything was drafted verifies zeros, not what the workspace held."""
+    import ctypes as C
+    from paper_2607_12422_gb300 import pbd, synth
+    S = _shape("tiny")
+    cfg = pbd.make_config(S, 16, 1, 256)
+    need = pbd.load().pbd_workspace_bytes(C.byref(cfg))
+    torch.full((need + 256,), 0x7F, dtype=torch.uint8, device="cuda")  # (the engine's workspace takes this place)
+    eng = pbd.Engine(S, synth.gen_base_weights(S), synth.gen_adapter(S), block_D=16, max_batch=1, max_seq_len=256)
+    eng.pbd_prefill([np.arange(50, dtype=np.int32)], max_new=8)
+    assert eng.pbd_time_pass(1, 2)[0] > 0
+    eng.close()
+
+
 @pytest.mark.parametrize("P,max_seq,ctas", [(40, 256, 0), (1100, 1400, 0), (40, 256, 4)])
 def test_waits_that_run_out_are_reported(torch, P, max_seq, ctas):
     """Every kind of pass that a context runs is made to wait in vain (kernel chain, with the attention merged in a
