@@ -183,7 +183,8 @@ bool valid_config(const pbd_config *cfg, std::string *why) {
     if (k.head_dim != 64 && k.head_dim != 128) return bad("head_dim must be 64 or 128");
     if (k.n_q_heads % k.n_kv_heads) return bad("n_q_heads must be a multiple of n_kv_heads");
     if (k.hidden % 256 || k.hidden > 4096) return bad("hidden must be a multiple of 256, at most 4096");
-    if ((k.n_q_heads * k.head_dim) % 256 || ((k.n_q_heads + 2 * k.n_kv_heads) * k.head_dim) % 128)
+    // (a 128-row tile of q|k|v is of one kind: the kernels normalise, rotate and store it as such)
+    if ((k.n_q_heads * k.head_dim) % 256 || (k.n_kv_heads * k.head_dim) % 128)
         return bad("q/k/v widths must tile by 128 and the attention width by 256");
     if (k.intermediate % 256 || k.intermediate > 16384)
         return bad("intermediate must be a multiple of 256, at most 16384");

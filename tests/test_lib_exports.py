@@ -55,6 +55,16 @@ def test_workspace_size_and_config_validation(lib):
         assert lib.pbd_workspace_bytes(C.byref(bad)) == 0, field
 
 
+def test_a_tile_that_is_half_k_and_half_v_is_refused(lib):
+    """k and v of an odd number of 64-wide heads share a 128-row tile, which the kernels take for k alone."""
+    for heads, ok in (((4, 1), False), ((12, 3), False), ((4, 2), True), ((12, 6), True), ((4, 4), True)):
+        cfg = pbd.make_config(synth.TINY, 16, 1, 256)
+        cfg.n_q_heads, cfg.n_kv_heads = heads
+        assert (lib.pbd_workspace_bytes(C.byref(cfg)) > 0) == ok, heads
+        cfg.head_dim = 128
+        assert lib.pbd_workspace_bytes(C.byref(cfg)) > 0, heads
+
+
 def test_create_rejects_bad_arguments_without_gpu(lib):
     cfg = pbd.make_config(synth.TINY, 16, 1, 128)
     bw, aw = pbd.pbd_base_weights(), pbd.pbd_adapter_weights()
