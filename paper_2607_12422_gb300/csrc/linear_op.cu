@@ -32,36 +32,6 @@ constexpr int LO_MAX_STAGES = 4;
 constexpr int LO_SMEM_HALF = 112 * 1024;  // dynamic shared memory with which two CTAs share an SM
 constexpr int LO_SMEM_MAX = 224 * 1024;
 
-__device__ __forceinline__ uint32_t map_cta(uint32_t addr, int rank) {
-    uint32_t a;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(addr), "r"(rank));
-    return a;
-}
-__device__ __forceinline__ float4 ld_cluster_v4(uint32_t a) {
-    float4 v;
-    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
-                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-                 : "r"(a)
-                 : "memory");
-    return v;
-}
-__device__ __forceinline__ float ld_cluster(uint32_t a) {
-    float v;
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
-    return v;
-}
-__device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
-// (by address: through a pointer into the dynamic array the compiler would use generic loads and stores)
-__device__ __forceinline__ float4 ld_shared_v4(uint32_t a) {
-    float4 v;
-    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a));
-    return v;
-}
-__device__ __forceinline__ void st_shared(uint32_t a, float v) { asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v)); }
-
 // Dynamic shared memory: `stages` of W tile, 16 KiB | x tile, bn x 128 bytes | adapter rows, whole KiB; then the
 // tile's B rows, transposed and widened, [r][128]; then, with several groups, the partial sums [rows][128]
 // and [rows][r] (one group: they take the ring's place).  The adapter's MMA reads 128 rows from its r rows on:

@@ -241,7 +241,7 @@ __device__ __forceinline__ float row_rms(const MKParams &P, int m) {
             a = __fadd_rn(a, v[u].y);
         }
     }
-    return __fdiv_rn(1.0f, __fsqrt_rn(__fadd_rn(__fdiv_rn(a, (float)P.dm.H), P.dm.eps)));
+    return rms_scale(a, P.dm.H, P.dm.eps);
 }
 
 // one B row (r bf16 values) of the adapter, for lora_dot_w
@@ -540,7 +540,7 @@ __device__ __noinline__ void reduce_qkv(const MKParams &P, int layer, int tile, 
             for (int j = 1; j < 4; ++j) ss = __fadd_rn(ss, __fmul_rn(y[j], y[j]));
 #pragma unroll
             for (int off = LPH / 2; off >= 1; off >>= 1) ss = __fadd_rn(ss, __shfl_xor_sync(0xffffffffu, ss, off));
-            const float rs = __fdiv_rn(1.0f, __fsqrt_rn(__fadd_rn(__fdiv_rn(ss, (float)DH), dm.eps)));
+            const float rs = rms_scale(ss, DH, dm.eps);
 #pragma unroll
             for (int j = 0; j < 4; ++j) y[j] = rbf(__fmul_rn(g[j], rbf(__fmul_rn(y[j], rs))));
             const float *cs = reinterpret_cast<const float *>(cs4);  // cos, sin of elements e0..e0+3

@@ -34,11 +34,6 @@ __device__ __forceinline__ int row_seg(const RowsArgs &a, int m) {
     return s;
 }
 
-// 1/sqrt(mean + eps) from a row's sum of squares, as row_rms in pass_kernel.cu
-__device__ __forceinline__ float rms_scale(float sum, int H, float eps) {
-    return __fdiv_rn(1.0f, __fsqrt_rn(__fadd_rn(__fdiv_rn(sum, (float)H), eps)));
-}
-
 __device__ __forceinline__ float warp_sum_butterfly(float s) {
 #pragma unroll
     for (int off = 16; off >= 1; off >>= 1) s = __fadd_rn(s, __shfl_xor_sync(0xffffffffu, s, off));

@@ -31,56 +31,6 @@ constexpr int ST_HALF = 4;         // 64-wide K atoms per half (256 of K)
 constexpr int ST_RANK = 16;        // adapter rank (8 or 16)
 constexpr int ST_A_BYTES = 2 * ST_RANK * 128;  // adapter rows of one K atom (gate and up: two ranks)
 
-__device__ __forceinline__ uint32_t map_cta(uint32_t addr, int rank) {
-    uint32_t a;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(addr), "r"(rank));
-    return a;
-}
-__device__ __forceinline__ float4 ld_cluster_v4(uint32_t a) {
-    float4 v;
-    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
-                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-                 : "r"(a)
-                 : "memory");
-    return v;
-}
-__device__ __forceinline__ float2 ld_cluster_v2(uint32_t a) {
-    float2 v;
-    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
-    return v;
-}
-__device__ __forceinline__ float ld_cluster(uint32_t a) {
-    float v;
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
-    return v;
-}
-__device__ __forceinline__ float4 ld_shared_v4(uint32_t a) {
-    float4 v;
-    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");
-    return v;
-}
-__device__ __forceinline__ float2 ld_shared_v2(uint32_t a) {
-    float2 v;
-    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
-    return v;
-}
-__device__ __forceinline__ float ld_shared(uint32_t a) {
-    float v;
-    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
-    return v;
-}
-__device__ __forceinline__ void st_cluster(uint32_t a, float v) {
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
-}
-__device__ __forceinline__ void st_cluster_v2(uint32_t a, float x, float y) {
-    asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(x), "f"(y) : "memory");
-}
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_sync() {
-    cluster_arrive();
-    cluster_wait();
-}
 template <int N>
 __device__ __forceinline__ void bar_stagers() {
     asm volatile("bar.sync 1, %0;" ::"n"(N) : "memory");
@@ -316,7 +266,7 @@ __global__ void __maxnreg__(NT == 256 ? 104 : 128)
                                 sum = __fadd_rn(sum, v[u].y);
                             }
                         }
-                        S.rs[m] = __fdiv_rn(1.0f, __fsqrt_rn(__fadd_rn(__fdiv_rn(sum, (float)dm.H), dm.eps)));
+                        S.rs[m] = rms_scale(sum, dm.H, dm.eps);
                     }
                 }
                 if (hf == 0 && both)
@@ -480,7 +430,7 @@ __global__ void __maxnreg__(NT == 256 ? 104 : 128)
                     for (int j = 1; j < 4; ++j) ssq = __fadd_rn(ssq, __fmul_rn(y[j], y[j]));
 #pragma unroll
                     for (int off = LPH / 2; off >= 1; off >>= 1) ssq = __fadd_rn(ssq, __shfl_xor_sync(0xffffffffu, ssq, off));
-                    const float rs = __fdiv_rn(1.0f, __fsqrt_rn(__fadd_rn(__fdiv_rn(ssq, (float)DH), dm.eps)));
+                    const float rs = rms_scale(ssq, DH, dm.eps);
                     float4 rope[2] = {rope1[0], rope1[1]};
                     if (m != m_first) row_rope(pos, rope);
                     const float4 ca = rope[0], cb = rope[1];
@@ -877,7 +827,7 @@ __global__ void __launch_bounds__(256) k_step_final(const __grid_constant__ Step
         const float v = __ldcg(a.ss + (size_t)m * nt + t);
         sum = t == 0 ? v : __fadd_rn(sum, v);
     }
-    const float rs = __fdiv_rn(1.0f, __fsqrt_rn(__fadd_rn(__fdiv_rn(sum, (float)H), a.dm.eps)));
+    const float rs = rms_scale(sum, H, a.dm.eps);
     for (int c = lane; c < H / 8; c += 32) {
         uint4 hv = __ldcg(reinterpret_cast<const uint4 *>(a.h + (size_t)m * H) + c);
         const uint4 gv = __ldg(reinterpret_cast<const uint4 *>(gain) + c);
