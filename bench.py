@@ -133,24 +133,26 @@ class ClockSampler:
                 "samples": len(sm)}
 
 
-def source_hash(path):
-    """Hash of a CUDA source with its comments and blank space removed: a comment edit leaves the
-    compiled kernel, and therefore its measured traffic, unchanged."""
+def source_hash(*paths):
+    """Hash of CUDA sources with their comments and blank space removed: a comment edit leaves the
+    compiled kernels, and therefore their measured traffic, unchanged."""
     import re
-    txt = open(path).read()
-    txt = re.sub(r"//[^\n]*", "", re.sub(r"/\*.*?\*/", "", txt, flags=re.S))
-    txt = re.sub(r"\s+", " ", txt).strip()
-    return hashlib.sha256(txt.encode()).hexdigest()[:16]
+    h = hashlib.sha256()
+    for path in paths:
+        txt = open(path).read()
+        txt = re.sub(r"//[^\n]*", "", re.sub(r"/\*.*?\*/", "", txt, flags=re.S))
+        h.update(re.sub(r"\s+", " ", txt).strip().encode())
+    return h.hexdigest()[:16]
 
 
-def traffic_for(kernel_src):
-    """DRAM bytes per pass from the committed ncu summary, if the kernel source is unchanged since
+def traffic_for(*kernel_srcs):
+    """DRAM bytes per pass from the committed ncu summary, if the kernels' sources are unchanged since
     (comments aside)."""
     path = os.path.join(ROOT, "profiles", "steps_verify_qwen3_0.6b_traffic.json")
     try:
         with open(path) as f:
             rec = json.load(f)
-        h = source_hash(kernel_src)
+        h = source_hash(*kernel_srcs)
         if rec.get("source_sha256_16") == h:
             return float(rec["dram_bytes_per_launch"])
     except Exception:
@@ -406,7 +408,9 @@ def main(args):
     ms_k, k_bytes = eng.pbd_time_pass(1, 16)
     ms_kd, kd_bytes = eng.pbd_time_pass(0, 16)
     achieved = k_bytes / (ms_k * 1e-3) / 1e9
-    traffic = traffic_for(os.path.join(ROOT, "paper_2607_12422_gb300", "csrc", "steps.cu"))
+    # (the chain's kernels, their attention steps and their copies)
+    traffic = traffic_for(*(os.path.join(ROOT, "paper_2607_12422_gb300", "csrc", f)
+                            for f in ("steps.cu", "attn.cuh", "common.cuh")))
 
     # ---- end to end through the public call with host buffers
     # (host prompt ids in, host token ids out; the binding copies the prompt to the device),

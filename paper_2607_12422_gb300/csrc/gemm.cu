@@ -248,9 +248,12 @@ __global__ void __launch_bounds__(GM_THREADS, 1) k_gemm(const __grid_constant__ 
                 __syncwarp();
                 if (lane == 0) mbarrier_arrive_one(&S.acc_empty[buf]);
             } else {
-                // The epilogue warps' issue slots are what this kernel runs out of first (with a few
-                // instructions more per element it took twice as long), so the sums use the packed
-                // fp32 add and each kind of slice has its own loop.
+                // No one thing bounds this kernel.  4096 x 1024 x 6144, us with the launch (8): 48.8; without the adds of
+                // slices 47.7, with half the bytes of token rows 46.7, with neither 45.0; finished tiles not
+                // rounded and stored 43.2.  Finishing a tile is the largest part: meanwhile the tensor core
+                // has the next tile's first two slices and no more.  With a few instructions more per
+                // element there it took twice as long, so the sums use the packed fp32 add and each kind of slice
+                // has its own loop.
                 uint32_t acc[NC][16];  // fp32 bits
                 for (int s = 0; s < parts; ++s, ++p) {
                     const int buf = p & 1;

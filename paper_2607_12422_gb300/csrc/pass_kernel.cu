@@ -1,7 +1,7 @@
 // pass_kernel.cu -- one persistent, cooperative kernel per decoder pass (draft, verify, plain
 // decoding, short prompt) of the PEFT-BD hot path.  It runs in contexts limited to fewer CTAs than SMs and
 // for shapes that steps.cu does not take; elsewhere that chain of cluster kernels is the faster one
-// (0.6B shape, verify pass at 512 tokens: 1136 us here, 757 there), with the same results bit for bit.
+// (0.6B shape, verify pass at 512 tokens: 1136 us here, 758 there), with the same results bit for bit.
 //
 // Why: at batch 1 and D = 16 a pass moves 1.2 GB of weights (~180 us at full HBM bandwidth)
 // through ~500 small dependent steps.  As separate kernel launches, launch gaps and latency

@@ -15,9 +15,9 @@
 // CTAs than SMs and for shapes whose slices or partial results do not fit a cluster; rows.cu computes the
 // same for prompts.
 //
-// 0.6B shape, all layers of one pass (the persistent kernel in brackets), us: verify 769 (1136), draft 963
-// (1287), one-row decoding 632 (945) at 512 tokens of context; 899 (1430), 1102 (1579), 750 (1196) at 4096;
-// 1619 (3637), 2059 (4080), 865 (1778) for eight sequences of 420 to 1757 tokens.
+// 0.6B shape, all layers of one pass (the persistent kernel in brackets), us: verify 758 (1136), draft 959
+// (1287), one-row decoding 619 (945) at 512 tokens of context; 880 (1430), 1090 (1579), 731 (1196) at 4096;
+// 1609 (3637), 2060 (4080), 846 (1778) for eight sequences of 420 to 1757 tokens.
 #include <algorithm>
 #include <cmath>
 
@@ -491,7 +491,10 @@ __global__ void __maxnreg__(NT == 256 ? 104 : 128)
 // loaded before its MMAs; with all of q's fragments in registers the compiler had too few left to batch
 // those loads (verify pass 779 us against 769; 4096 tokens 934 against 899).
 constexpr int SA_WARPS = 6;   // compute warps of a cluster's CTA: the units of 17 rows with two heads a group
-constexpr int SG_WARPS = 4;   // compute warps of a single split's CTA
+// compute warps of a single split's CTA, compiled for three CTAs an SM: one-row passes have three there, 17 rows two
+// (their q rows take shared memory), and the fewer registers suit both (17 rows at 4096 tokens, us a layer of a verify
+// pass: 33.1; compiled for two 34.4)
+constexpr int SG_WARPS = 4;
 constexpr int SA_STATS = 4;   // partial results per row at most: 32 x this
 
 // Merge of one row's nv partial results in key order, relative to the row's overall maximum (attn_combine in
@@ -848,7 +851,8 @@ constexpr int ST_SMEM = 216 * 1024;   // dynamic shared memory of one CTA at mos
 constexpr int ST_MAX_CLUSTER = 16;
 // Rows up to which partial sums are pushed: a pushed row costs a scalar remote store per thread (~40 ns), pulling
 // costs a remote round trip and a second cluster barrier (~0.8 us) once (17 rows: verify pass 896 us pulled, 799
-// pushed; 136 rows: 1823 pulled, 2032 pushed).
+// pushed; 136 rows: 1823 pulled, 2032 pushed).  Between them, us a layer, verify / draft: 33 rows 36.3 / 44.5
+// pulled, 35.1 / 44.2 pushed; 48 rows 40.2 / 47.9 and 39.0 / 48.7; 64 rows 46.7 / 55.4 and 45.4 / 56.7.
 constexpr int ST_PUSH_ROWS = 32;
 
 static int step_bn(int M) { return std::max(32, (M + 15) / 16 * 16); }
@@ -925,7 +929,9 @@ static cudaError_t launch_step(void (*kernel)(P...), dim3 grid, dim3 cluster, in
 }
 
 // More threads for more rows: staging and finishing rows are loops over them (136 rows, 0.6B
-// shape: verify pass 1763 us with 256 threads, 1619 with 512; at 17 rows the wider CTA starts later).
+// shape: verify pass 1763 us with 256 threads, 1619 with 512; at 17 rows the wider CTA starts later).  The line is
+// higher than it need be: us a layer, verify / draft, with 256 and with 512 threads: 33 rows 36.3 / 44.5 and
+// 34.4 / 42.2, 64 rows 46.7 / 55.4 and 42.6 / 52.3, 68 rows 41.2 / 53.9 and 38.8 / 50.2.
 static int lin_threads(int M) { return M <= 64 ? 256 : 512; }
 
 template <int DH, int NT>
