@@ -15,8 +15,8 @@
 // cluster barrier CTA c takes rows c, c + cs, ...: it reads the group's partials through distributed
 // shared memory and adds them in slice order, so a row's bits depend neither on M nor on timing.
 //
-// Bound: latency.  GPU time at M = 17, r = 16 (cold caches): 9.0 us for K = 1024, N = 6144 and 8.4 us for
-// K = 3072, N = 1024; 6.6 us at M = 1, K = 2048, N = 1024, r = 0.  With one CTA an SM, as before the adapter's place
+// Bound: latency.  GPU time at M = 17, r = 16 (cold caches): 8.8 us for K = 1024, N = 6144 and 8.5 us for
+// K = 3072, N = 1024; 6.7 us at M = 1, K = 2048, N = 1024, r = 0.  With one CTA an SM, as before the adapter's place
 // was cut to its rank, the first took 13.2.  With the partial sums in global memory and the last CTA of a tile
 // finishing it alone: 22.0, 17.4 and 8.2 us, of which 8 us that last step; as re-tiling, split-K and
 // reduction kernels: 21.4, 20.5 and 12.5 us and their gaps.
@@ -38,7 +38,7 @@ constexpr int LO_SMEM_MAX = 224 * 1024;
 // what follows them reaches only accumulator rows that nobody reads.
 struct LoSmem {
     int a_bytes, stage, b_off, part_off, total;
-    __host__ __device__ LoSmem(int bn, int r, int rows, int groups, int stages) {
+    LoSmem(int bn, int r, int rows, int groups, int stages) {
         a_bytes = (r * 128 + 1023) / 1024 * 1024;
         stage = TILE_BYTES + bn * 128 + a_bytes;
         const int ring = stages * stage, part = (rows * (TILE_ROWS + r) * 4 + 15) / 16 * 16;
@@ -60,12 +60,11 @@ __global__ void __launch_bounds__(LO_THREADS, 2) k_linear_op(const __grid_consta
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const int tile = blockIdx.x, rank = blockIdx.y, tok0 = blockIdx.z * LINEAR_OP_ROWS, rows = min(a.M - tok0, LINEAR_OP_ROWS);
     const int groups = ONE ? 1 : a.groups;
-    const LoSmem sm(a.bn, a.r, min(a.M, LINEAR_OP_ROWS), groups, a.stages);
-    const int stage = sm.stage, x_off = TILE_BYTES, a_off = TILE_BYTES + a.bn * 128;
-    const uint32_t s_b = smem_u32(base + sm.b_off);
+    const int stage = a.stage, x_off = TILE_BYTES, a_off = TILE_BYTES + a.bn * 128;
+    const uint32_t s_b = smem_u32(base + a.b_off);
     const uint32_t tmem_cols = (uint32_t)(a.r > 0 ? 2 * a.bn : a.bn);  // one or two accumulators of 32 or 64 columns
     if (threadIdx.x == 0) {
-        for (int s = 0; s < a.stages; ++s) {
+        for (int s = 0; s < LO_MAX_STAGES; ++s) {
             mbar_init(&full[s], 1);
             mbar_init(&empty[s], 1);
         }
@@ -84,7 +83,7 @@ __global__ void __launch_bounds__(LO_THREADS, 2) k_linear_op(const __grid_consta
     const int mine = ONE ? 1 : (a.ks - 1 - rank) / a.cs + 1;  // this CTA's slices
     const int atoms = mine * a.kt_per;
 
-    const uint32_t part = smem_u32(base + sm.part_off), part_u = part + (uint32_t)(rows * TILE_ROWS) * 4u;
+    const uint32_t part = smem_u32(base + a.part_off), part_u = part + (uint32_t)(rows * TILE_ROWS) * 4u;
     const uint32_t pa = part + 16u * lane, ua = part_u + 4u * (lane < a.r ? lane : 0);
 
     // partial sums of row m over the group's n slices, in slice order, onto (y, u)
@@ -296,7 +295,11 @@ cudaError_t launch_linear_op(LinOpArgs &a, cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((a.N + TILE_ROWS - 1) / TILE_ROWS, a.cs, (a.M + LINEAR_OP_ROWS - 1) / LINEAR_OP_ROWS);
     cfg.blockDim = dim3(LO_THREADS);
-    cfg.dynamicSmemBytes = smem(a.stages);
+    const LoSmem sm(a.bn, a.r, rows, a.groups, a.stages);
+    a.stage = sm.stage;
+    a.b_off = sm.b_off;
+    a.part_off = sm.part_off;
+    cfg.dynamicSmemBytes = sm.total + 1024;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;

@@ -241,7 +241,7 @@ struct LinOpArgs {
     bf16 *y;
     int vec_store;  // y is 8-byte aligned and N a multiple of 4
     int *status;
-    int bn, cs, groups, stages;
+    int bn, cs, groups, stages, stage, b_off, part_off;
 };
 constexpr int LINEAR_OP_ROWS = 64;         // token rows of a CTA
 constexpr int LINEAR_OP_MAX_CLUSTER = 16;
